@@ -13,7 +13,6 @@
 //                   the samples themselves for value-only tables.
 //   k_pack          re-encode a table into another dtype / layout.
 //   k_bounds        per-glyph bound of |interpolated r| for ray bracketing (§3.1).
-//   k_sh_eval       direct SH value, S^2 gradient and normal (ground truth, no table).
 //
 // SH convention: orthonormal real SH, index l*l + l + m, no Condon-Shortley phase,
 // Y_l0 = P~_l^0(z), Y_lm = sqrt2 P~_l^m(z) Re (x+iy)^m, Y_l-m = sqrt2 P~_l^m(z) Im (x+iy)^m, where
@@ -977,71 +976,6 @@ cudaError_t launch_bounds(const LutView& L, float* rmax, const Sizes& sz, cudaSt
             else k_bounds<SHM_BF16, SHM_LAYOUT_CELL, M><<<grid, 256, 0, s>>>(L, rmax, map);
         }
     });
-}
-
-// ------------------------------------------------------------------------------------------
-// Direct SH: r = sum_k c_k Y_k(w), Euclidean gradient of the polynomial projected onto the tangent
-// plane gives grad_{S^2} r, then the §3.4 normal.
-__global__ void __launch_bounds__(128) k_sh_eval(int L, int G, const float* __restrict__ coeffs, int64_t Q,
-                                                 const float* __restrict__ dirs, const int32_t* __restrict__ glyph,
-                                                 const int64_t* __restrict__ seg, float* R, float* grad,
-                                                 float* normal, int32_t* dev_status)
-{
-    const int K = (L + 1) * (L + 1);
-    uint32_t status = 0;
-    const float qnan = __int_as_float(0x7fc00000);
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < Q; q += (int64_t)gridDim.x * blockDim.x) {
-        int g = 0;
-        if (glyph) g = __ldg(glyph + q);
-        else if (seg) g = (q < __ldg(seg)) ? -1 : seg_find(seg, G, q);
-        const float d0 = __ldg(dirs + 3 * q), d1 = __ldg(dirs + 3 * q + 1), d2 = __ldg(dirs + 3 * q + 2);
-        const float n2 = d0 * d0 + d1 * d1 + d2 * d2;
-        bool ok = (g >= 0 && g < G);
-        if (!ok) status |= SHM_DEV_BOUNDS;
-        if (ok && !(n2 > 0.0f && n2 <= 3.0e38f)) { ok = false; status |= SHM_DEV_NONFINITE; }
-        float r = qnan;
-        Vec3 gs{qnan, qnan, qnan}, nn{qnan, qnan, qnan};
-        if (ok) {
-            const float il = rsqrtf(n2);
-            const Vec3 w{d0 * il, d1 * il, d2 * il};
-            float Tl[(SH_LMAX + 1) * (SH_LMAX + 2) / 2];
-            float C[SH_LMAX + 1], S[SH_LMAX + 1];
-            legendre_table(L, w.z, Tl);
-            cs_table(L, w.x, w.y, C, S);
-            const float* c = coeffs + (int64_t)g * K;
-            float rv = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-            for (int l = 0; l <= L; ++l)
-                for (int mm = -l; mm <= l; ++mm) {
-                    const int m = mm < 0 ? -mm : mm;
-                    const YDer y = ylm_derivs(Tl, l, m, mm < 0, C, S);
-                    const float ck = __ldg(c + l * l + l + mm);
-                    rv = fmaf(ck, y.v, rv);
-                    gx = fmaf(ck, y.gx, gx);
-                    gy = fmaf(ck, y.gy, gy);
-                    gz = fmaf(ck, y.gz, gz);
-                }
-            const float wg = w.x * gx + w.y * gy + w.z * gz;
-            r = rv;
-            gs = Vec3{gx - w.x * wg, gy - w.y * wg, gz - w.z * wg};
-            nn = surface_normal(d0, d1, d2, r, gs);
-        }
-        if (R) R[q] = r;
-        if (grad) { grad[3 * q] = gs.x; grad[3 * q + 1] = gs.y; grad[3 * q + 2] = gs.z; }
-        if (normal) { normal[3 * q] = nn.x; normal[3 * q + 1] = nn.y; normal[3 * q + 2] = nn.z; }
-    }
-    report_status(dev_status, status);
-}
-
-cudaError_t launch_sh_eval(int L, int G, const float* coeffs, int64_t Q, const float* dirs, const int32_t* glyph,
-                           const int64_t* seg, float* R, float* grad, float* normal, int32_t* dev_status,
-                           cudaStream_t s)
-{
-    if (Q == 0) return cudaSuccess;
-    int64_t blocks = (Q + 127) / 128;
-    const int64_t cap = (int64_t)sm_count() * 16;
-    if (blocks > cap) blocks = cap;
-    k_sh_eval<<<(unsigned)blocks, 128, 0, s>>>(L, G, coeffs, Q, dirs, glyph, seg, R, grad, normal, dev_status);
-    return cudaGetLastError();
 }
 
 }  // namespace shm
