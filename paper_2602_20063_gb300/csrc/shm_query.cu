@@ -33,11 +33,19 @@ cudaError_t launch_unstaged_shape(const QueryArgs& a, int shape, cudaStream_t s)
 
 }  // namespace
 
+// Staging reads every glyph's whole table, so it pays from about table bytes / 128 B queries per glyph
+// (a query gathers four 32-byte sectors by itself); below 256 per glyph the copy's latency dominates.
+// 3,000 glyphs, mean queries per glyph 256 / 512 / 1,024, staged against direct in us: N = 32 f32
+// 61.9 / 68.6 / 81.0 against 36.9 / 59.1 / 83.6; N = 32 f16 39.6 / 46.2 / 61.6 against 33.0 / 51.8 / 76.0;
+// N = 12 f32 30.4 / 37.4 / 53.2 against 29.4 / 47.1 / 71.8.  Both give the same bits.
 bool query_is_staged(const QueryArgs& a)
 {
     if (!a.seg || a.glyph || a.L.N_uniform <= 0 || a.L.layout != SHM_LAYOUT_TEXEL) return false;
     const int64_t P = (int64_t)a.L.N_uniform + 2;
-    return 6 * P * P * (a.L.dtype == SHM_F32 ? 16 : 8) <= STAGED_TABLE_MAX_BYTES;
+    const int64_t bytes = 6 * P * P * (a.L.dtype == SHM_F32 ? 16 : 8);
+    if (bytes > STAGED_TABLE_MAX_BYTES) return false;
+    const int64_t per = bytes / 128 > 256 ? bytes / 128 : 256;
+    return a.Q >= a.L.n_glyphs * per;
 }
 
 int query_shapes(const QueryArgs& a) { return query_is_staged(a) ? staged_shapes() : N_QSHAPES; }

@@ -1,18 +1,23 @@
 // Staged query (§3.2-§3.4) for per-glyph query segments on tables that fit in shared memory.
 //
-// With CSR segments every glyph's queries are contiguous, so a CTA can take a whole glyph: one
+// With CSR segments every glyph's queries are contiguous, so a CTA can take them together: one
 // bulk copy (cp.async.bulk, completion on an mbarrier) brings the glyph's padded table into shared
 // memory, then the CTA answers all of that glyph's queries from it.  The table is read from HBM
 // once, the 2x2 footprints become shared-memory reads, and HBM sees only the bulk copy and the
 // coalesced direction / output streams (for N = 32, f32: 111 KB + 4,096 x 40 B per glyph), instead
 // of texel reads that miss L1 about half of the time.  Two CTAs per SM overlap one CTA's copy with
-// the other's queries.
+// the other's queries, and where two tables fit a CTA's share (N <= 22 f32, N <= 32 16-bit) the next
+// glyph's copy runs under this glyph's queries.
+//
+// Each CTA takes one unit of equal cost of the path through glyphs and queries (shm_stage.cuh), so long
+// segments are shared and uneven ones balance: 37 glyphs, 2.2 M queries in uneven segments (f16, N = 32)
+// 348 -> 28.7 us, the glyph field (16,384 even segments) 1,229 -> 1,221 us with its bake.
 //
 // Results are bit-identical to k_query_fwd (same device functions on the same values).  Directions
 // and outputs are touched once, so they are loaded and stored with the streaming cache hint
 // (__ldcs / __stcs: evict first) and leave L2 to the tables.
 // The wait for the copy is bounded (1 s); on expiry the CTA raises SHM_DEV_TIMEOUT, waits up to
-// 100 ms more for its copy to land and returns without touching the outputs of that glyph.
+// 100 ms more for its copies to land and returns without touching the outputs of that glyph.
 #include "shm_stage.cuh"
 
 namespace shm {
@@ -28,12 +33,13 @@ constexpr int SSHAPES[N_SSHAPES] = {512, 1024, 256};
 // STD: the usual output set (R, gradient and normal; no chart derivatives, no cell indices), so the
 // per-query output checks drop out of the loop.
 template <int DT, int SBLOCK, bool STD>
-__global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArgs a, uint32_t table_bytes)
+__global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArgs a, uint32_t table_bytes, int nbuf)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_abort;
+    __shared__ stage::Pos s_unit[2];
     const uint32_t bar = (uint32_t)__cvta_generic_to_shared(smem);
-    const unsigned char* table = smem + stage::TABLE_OFFSET;
+    const unsigned char* tables = smem + stage::TABLE_OFFSET;
     const uint32_t table_s = bar + stage::TABLE_OFFSET;
     const int tid = threadIdx.x;
     const int G = a.L.n_glyphs, N = a.L.N_uniform, P = N + 2;
@@ -60,30 +66,43 @@ __global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArg
 
     if (tid == 0) {
         stage::init(bar);
+        stage::init(bar + 8);
         s_abort = 0;
     }
-    __syncthreads();
+    const int64_t w = table_bytes / stage::QUERY_BYTES;
+    stage::Pos start, end;
+    stage::unit_of(a.seg, G, a.Q, w, s_unit, start, end);  // its barrier also publishes the mbarriers
 
-    uint32_t phase = 0;
-    for (int g = blockIdx.x; g < G; g += gridDim.x) {
-        const int64_t s0 = min(max(__ldg(a.seg + g), (int64_t)0), a.Q);
-        const int64_t s1 = min(max(__ldg(a.seg + g + 1), s0), a.Q);
-        if (s1 <= s0) continue;  // block-uniform
-        if (tid == 0)
-            stage::issue(bar, table_s, reinterpret_cast<const unsigned char*>(a.L.data) + (size_t)g * table_bytes,
-                         table_bytes);
+    const auto copy = [&](int g, int buf) {
+        stage::issue(bar + 8 * buf, table_s + buf * table_bytes,
+                     reinterpret_cast<const unsigned char*>(a.L.data) + (size_t)g * table_bytes, table_bytes);
+    };
+    uint32_t phase = 0;  // bit buf: parity of the buffer's next completion
+    int buf = 0;
+    stage::Part part = stage::next_part(a.seg, G, a.Q, start.g, start, end);
+    if (tid == 0 && part.a < part.b) copy(part.g, 0);
+    while (part.a < part.b) {
+        const int g = part.g;
+        const int64_t s1 = part.b;
+        const stage::Part next = stage::next_part(a.seg, G, a.Q, g + 1, start, end);
+        const bool more = next.a < next.b;
+        if (tid == 0 && more && nbuf == 2) copy(next.g, buf ^ 1);
+        const unsigned char* table = tables + buf * table_bytes;
         // first direction of this thread while the copy runs
-        int64_t q = s0 + tid;
+        int64_t q = part.a + tid;
         float d0 = 0.f, d1 = 0.f, d2 = 0.f;
         if (q < s1) { d0 = __ldcs(a.dirs + 3 * q); d1 = __ldcs(a.dirs + 3 * q + 1); d2 = __ldcs(a.dirs + 3 * q + 2); }
-        if (!stage::bar_wait(bar, phase, stage::WAIT_NS)) s_abort = 1;
+        if (!stage::bar_wait(bar + 8 * buf, (phase >> buf) & 1, stage::WAIT_NS)) s_abort = 1;
         __syncthreads();
         if (s_abort) {
             status |= SHM_DEV_TIMEOUT;
-            if (tid == 0) stage::bar_wait(bar, phase, stage::DRAIN_NS);
+            if (tid == 0) {
+                stage::bar_wait(bar + 8 * buf, (phase >> buf) & 1, stage::DRAIN_NS);
+                if (more && nbuf == 2) stage::bar_wait(bar + 8 * (buf ^ 1), (phase >> (buf ^ 1)) & 1, stage::DRAIN_NS);
+            }
             break;
         }
-        phase ^= 1;
+        phase ^= 1u << buf;
         const float r0 = a.L.r0 ? __ldg(a.L.r0 + g) : 0.0f;
         for (; q < s1; q += SBLOCK) {
             const int64_t qn = q + SBLOCK;
@@ -116,6 +135,9 @@ __global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArg
             d0 = n0; d1 = n1; d2 = n2;
         }
         __syncthreads();  // every read of this table is done before the next copy lands
+        if (nbuf == 2) buf ^= 1;
+        else if (tid == 0 && more) copy(next.g, 0);
+        part = next;
     }
     report_status(a.dev_status, status);
 }
@@ -123,7 +145,10 @@ __global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArg
 template <int DT, int SBLOCK, bool STD>
 cudaError_t launch_staged_o(const QueryArgs& a, uint32_t table_bytes, cudaStream_t s)
 {
-    const int smem = stage::TABLE_OFFSET + (int)table_bytes;
+    // a second buffer takes the next glyph's table while this one is queried, where two CTAs per SM
+    // still fit
+    const int nbuf = 2 * (int64_t)table_bytes <= STAGED_TABLE_MAX_BYTES ? 2 : 1;
+    const int smem = stage::TABLE_OFFSET + nbuf * (int)table_bytes;
     cudaError_t e = ensure_dynamic_smem((const void*)k_query_staged<DT, SBLOCK, STD>, smem);
     if (e != cudaSuccess) return e;
     int resident = 0;
@@ -131,10 +156,9 @@ cudaError_t launch_staged_o(const QueryArgs& a, uint32_t table_bytes, cudaStream
             cudaSuccess ||
         resident < 1)
         resident = 1;
-    int64_t blocks = (int64_t)sm_count() * resident;
-    if (blocks > a.L.n_glyphs) blocks = a.L.n_glyphs;
-    if (blocks < 1) blocks = 1;
-    k_query_staged<DT, SBLOCK, STD><<<(unsigned)blocks, SBLOCK, smem, s>>>(a, table_bytes);
+    const int64_t blocks = stage::units_for(a.Q, a.L.n_glyphs, table_bytes / stage::QUERY_BYTES,
+                                            (int64_t)sm_count() * resident);
+    k_query_staged<DT, SBLOCK, STD><<<(unsigned)blocks, SBLOCK, smem, s>>>(a, table_bytes, nbuf);
     return cudaGetLastError();
 }
 

@@ -1,6 +1,12 @@
 // Shared-memory staging of one glyph's table for the per-glyph segment kernels (forward query,
 // reverse pass): one thread issues cp.async.bulk copies completing on an mbarrier, every thread
 // waits on it with a time limit.
+//
+// Work split: the segments are cut into `units` of equal cost along the path that runs through the
+// glyphs in order, paying `w` for every glyph (its table copy) and 1 for every query.  A unit is a CTA's
+// whole work: it starts and ends anywhere inside a glyph, so a few long segments spread over every SM
+// and uneven ones balance (one CTA per glyph left 37 glyphs of 60,000 queries on 37 of 304 CTAs).  w is
+// the copy's cost in queries at memory bandwidth, table bytes / 40 B of directions and outputs.
 #pragma once
 #include "shm_internal.h"
 
@@ -10,7 +16,9 @@ namespace stage {
 constexpr uint64_t WAIT_NS = 1000000000ull;   // 1 s
 constexpr uint64_t DRAIN_NS = 100000000ull;   // 100 ms
 constexpr uint32_t BULK_PIECE = 32768;        // bytes per cp.async.bulk
-constexpr int TABLE_OFFSET = 128;             // mbarrier first, table 128-byte aligned
+constexpr int TABLE_OFFSET = 128;             // mbarriers first, tables 128-byte aligned
+constexpr int QUERY_BYTES = 40;               // direction and outputs of one query
+constexpr int UNIT_MIN = 1024;                // queries a unit should have before another CTA pays for a copy
 
 __device__ __forceinline__ uint64_t gtimer()
 {
@@ -60,6 +68,74 @@ __device__ __forceinline__ void issue(uint32_t bar, uint32_t dst, const unsigned
                      ::"r"(dst + off), "l"(src + off), "r"(n), "r"(bar)
                      : "memory");
     }
+}
+
+// Position on the path: query q of glyph g (g = G: past the last one).
+struct Pos {
+    int g;
+    int64_t q;
+};
+
+// Part [a, b) of glyph g's queries; b <= a: no part left.
+struct Part {
+    int g;
+    int64_t a, b;
+};
+
+__device__ __forceinline__ int64_t seg_at(const int64_t* seg, int64_t Q, int g)
+{
+    return min(max(__ldg(seg + g), (int64_t)0), Q);
+}
+
+// The path position at cost D (a whole warp calls it; 32 probes per round).
+__device__ __forceinline__ Pos path_at(const int64_t* seg, int G, int64_t Q, int64_t w, int64_t D)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t lo = seg_at(seg, Q, 0);
+    int g = 0, n = G + 1;  // the largest g in [0, G] with cost(g) = seg[g] - seg[0] + w g <= D
+    while (n > 1) {
+        const int step = (n + 31) / 32, at = lane * step;
+        const unsigned m = __ballot_sync(0xffffffffu, at < n && seg_at(seg, Q, g + at) - lo + w * (g + at) <= D);
+        const int k = 31 - __clz((int)(m | 1u));
+        g += k * step;
+        n = min(step, n - k * step);
+    }
+    const int64_t s = seg_at(seg, Q, g);
+    return Pos{g, min(Q, s + max((int64_t)0, D - (s - lo + w * g) - w))};
+}
+
+// The first non-empty part of glyph g or a later one, up to the end position.
+__device__ __forceinline__ Part next_part(const int64_t* seg, int G, int64_t Q, int g, const Pos& start, const Pos& end)
+{
+    for (; g <= end.g && g < G; ++g) {
+        int64_t a = seg_at(seg, Q, g), b = max(seg_at(seg, Q, g + 1), a);
+        if (g == start.g) a = max(a, start.q);
+        if (g == end.g) b = min(b, end.q);
+        if (a < b) return Part{g, a, b};
+    }
+    return Part{G, 0, 0};
+}
+
+// This CTA's unit of the path: start and end positions through shared memory (every thread calls it).
+__device__ __forceinline__ void unit_of(const int64_t* seg, int G, int64_t Q, int64_t w, Pos* sh, Pos& start, Pos& end)
+{
+    const int warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        const int64_t total = seg_at(seg, Q, G) - seg_at(seg, Q, 0) + w * G;
+        const Pos p = path_at(seg, G, Q, w, total / gridDim.x * (blockIdx.x + warp) +
+                                                total % gridDim.x * (blockIdx.x + warp) / gridDim.x);
+        if ((threadIdx.x & 31) == 0) sh[warp] = p;
+    }
+    __syncthreads();
+    start = sh[0];
+    end = sh[1];
+}
+
+// Host: units for Q queries over G glyphs, at most `cap` (the CTAs that run at once).
+inline int64_t units_for(int64_t Q, int64_t G, int64_t w, int64_t cap)
+{
+    const int64_t n = (Q + w * G) / (UNIT_MIN + (w < UNIT_MIN ? w : UNIT_MIN)) + 1;
+    return n < cap ? n : cap;
 }
 
 template <int DT>
