@@ -190,13 +190,18 @@ __device__ __forceinline__ void report_status(int32_t* dev_status, uint32_t bits
     if (dev_status && any && (threadIdx.x & 31) == 0) atomicOr(dev_status, (int)any);
 }
 
-// Largest g in [0, G] with seg[g] <= q (q >= seg[0] assumed; g == G means q is past the end).
-__device__ __forceinline__ int seg_find(const int64_t* seg, int G, int64_t q)
+// Largest g in [0, G] with seg[g] <= q (q >= seg[0] assumed; g == G means q is past the end), searched by
+// a whole warp 32 ways at a time: three dependent loads for 16,384 glyphs instead of fourteen.
+__device__ __forceinline__ int seg_find_warp(const int64_t* seg, int G, int64_t q)
 {
-    int lo = 0, hi = G + 1;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(seg + mid) <= q) lo = mid; else hi = mid;
+    const int lane = threadIdx.x & 31;
+    int lo = 0, n = G + 1;
+    while (n > 1) {
+        const int step = (n + 31) / 32, at = lane * step;
+        const unsigned m = __ballot_sync(0xffffffffu, at < n && __ldg(seg + lo + at) <= q);
+        const int k = 31 - __clz((int)(m | 1u));
+        lo += k * step;
+        n = min(step, n - k * step);
     }
     return lo;
 }

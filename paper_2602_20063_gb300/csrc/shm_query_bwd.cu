@@ -88,9 +88,7 @@ __global__ void __launch_bounds__(BBLOCK, 4) k_query_bwd(BackwardArgs a)
     for (int64_t c0 = warp0 * chunk; c0 < a.Q; c0 += nwarps * chunk) {
         int g = 0;
         if (a.seg) {
-            int g0 = 0;
-            if (lane == 0) g0 = (c0 < __ldg(a.seg)) ? -1 : seg_find(a.seg, G, c0);
-            g = __shfl_sync(0xffffffffu, g0, 0);
+            g = (c0 < __ldg(a.seg)) ? -1 : seg_find_warp(a.seg, G, c0);
         }
 #pragma unroll 1
         for (int it = 0; it < BCHUNK; ++it) {

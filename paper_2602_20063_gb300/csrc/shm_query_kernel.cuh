@@ -15,18 +15,21 @@
 
 namespace shm {
 
-// Launch shapes (threads per CTA, rounds per CTA chunk): a CTA takes BLOCK * IT consecutive
-// queries.  Shape 0 is the default; shm_tune_query times the others on a caller's batch and
-// records the fastest per (path, dtype, layout) for later calls.
+// Launch shapes (threads per CTA, most rounds per CTA chunk): a CTA takes chunks of up to BLOCK * IT
+// consecutive queries.  Shape 0 is the default; shm_tune_query times the others on a caller's batch
+// and records the fastest per (path, dtype, layout) for later calls.
 struct QShape {
     int block, it;
 };
 constexpr int N_QSHAPES = 4;
 constexpr QShape QSHAPES[N_QSHAPES] = {{512, 8}, {256, 16}, {1024, 4}, {256, 8}};
 
-// Work is handed out per CTA in contiguous chunks (4,096 queries by default), so that for per-glyph query
-// segments a CTA serves whole glyphs and the glyph's table stays in that SM's L1 (two CTAs per SM
-// keep two tables of up to ~110 KB resident) instead of being pulled into several SMs.
+// Work is handed out per CTA in contiguous chunks (up to 4,096 queries by default), so that for
+// per-glyph query segments a CTA serves whole glyphs and the glyph's table stays in that SM's L1 (two
+// CTAs per SM keep two tables of up to ~110 KB resident) instead of being pulled into several SMs.
+// Without segments a chunk is one round of BLOCK queries: there is no glyph to keep, a small batch
+// spreads over every SM (65,536 queries: 128 CTAs instead of 16, kernel 18 -> 5 us) and a large one has
+// no last wave of eight rounds (4K planet view, f16 cells, 4.6 M queries: 71 -> 60 us).
 //
 // VEC (all of dirs / grad / normal 16-byte aligned): for a full warp round (32 queries) the 384 B
 // of directions are read with 24 128-bit loads and the 384 B of gradients and of normals are
@@ -40,133 +43,127 @@ struct QueryOccupancy {
     static constexpr int min_blocks = (RECON >= SHM_RECON_BICUBIC) ? 1 : (QBLOCK >= 1024 ? 1 : 1024 / QBLOCK);
 };
 
-template <int DT, int LAYOUT, bool VEC, int RECON, int QBLOCK = 512, int QIT = 8>
-__global__ void __launch_bounds__(QBLOCK, (QueryOccupancy<RECON, QBLOCK>::min_blocks)) k_query_fwd(QueryArgs a)
+template <int DT, int LAYOUT, bool VEC, int RECON, int QBLOCK = 512>
+__global__ void __launch_bounds__(QBLOCK, (QueryOccupancy<RECON, QBLOCK>::min_blocks)) k_query_fwd(QueryArgs a, int rounds)
 {
     __shared__ __align__(16) float sbuf[QBLOCK / 32][96];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* wb = sbuf[warp];
-    const int64_t CH = (int64_t)QBLOCK * QIT;
     const int G = a.L.n_glyphs;
     uint32_t status = 0;
     const float qnan = __int_as_float(0x7fc00000);
     const float4* dirs4 = reinterpret_cast<const float4*>(a.dirs);
 
-    for (int64_t c0 = (int64_t)blockIdx.x * CH; c0 < a.Q; c0 += (int64_t)gridDim.x * CH) {
-        // glyph of this lane's first query and the end of its segment (one search per warp and chunk)
-        int g = 0;
-        int64_t seg_end = INT64_MAX;
-        const int64_t qw0 = c0 + warp * 32;
-        if (a.seg) {
-            int g0 = 0;
-            long long e0 = 0;
-            if (lane == 0 && qw0 < a.Q) {
-                g0 = (qw0 < __ldg(a.seg)) ? -1 : seg_find(a.seg, G, qw0);
-                e0 = (g0 >= 0 && g0 < G) ? __ldg(a.seg + g0 + 1) : 0;
-            }
-            g = __shfl_sync(0xffffffffu, g0, 0);
-            seg_end = __shfl_sync(0xffffffffu, e0, 0);
+    // round i of the chunk at c0; the next round (of this chunk or of the CTA's next one) is known one
+    // round ahead, so its directions are always loaded under this round's table fetch
+    int64_t c0 = (int64_t)blockIdx.x * QBLOCK * rounds;
+    int64_t qw = c0 + warp * 32;
+    int i = 0;
+    // glyph of this lane's first query and the end of its segment (one search per warp and chunk)
+    int g = 0;
+    int64_t seg_end = INT64_MAX;
+    // direction of the first round: vector (full round) or scalar
+    float4 pv = make_float4(0.f, 0.f, 0.f, 0.f);
+    float n0 = 0.f, n1 = 0.f, n2 = 0.f;
+    const auto load_dirs = [&](int64_t qn) {
+        if (VEC && qn + 32 <= a.Q) {
+            if (lane < 24) pv = __ldg(dirs4 + (3 * qn) / 4 + lane);
+        } else if (qn + lane < a.Q) {
+            n0 = __ldcs(a.dirs + 3 * (qn + lane));
+            n1 = __ldcs(a.dirs + 3 * (qn + lane) + 1);
+            n2 = __ldcs(a.dirs + 3 * (qn + lane) + 2);
         }
-        // direction of the first round: vector (full round) or scalar
-        float4 pv = make_float4(0.f, 0.f, 0.f, 0.f);
-        float n0 = 0.f, n1 = 0.f, n2 = 0.f;
-        if (VEC && qw0 + 32 <= a.Q) {
-            if (lane < 24) pv = __ldg(dirs4 + (3 * qw0) / 4 + lane);
-        } else if (qw0 + lane < a.Q) {
-            const int64_t q = qw0 + lane;
-            n0 = __ldcs(a.dirs + 3 * q); n1 = __ldcs(a.dirs + 3 * q + 1); n2 = __ldcs(a.dirs + 3 * q + 2);
-        }
+    };
+    load_dirs(qw);
 #pragma unroll 1
-        for (int it = 0; it < QIT; ++it) {
-            const int64_t qw = qw0 + (int64_t)it * QBLOCK;
-            if (qw >= a.Q) break;
-            const bool full = VEC && (qw + 32 <= a.Q);
-            const int64_t q = qw + lane;
-            float d0, d1, d2;
-            if (full) {
-                // re-distribute the warp's 24 float4 of directions: lane L takes floats 3L..3L+2
-                if (lane < 24) reinterpret_cast<float4*>(wb)[lane] = pv;
+    while (qw < a.Q) {
+        if (a.seg && i == 0) {
+            g = (qw < __ldg(a.seg)) ? -1 : seg_find_warp(a.seg, G, qw);
+            seg_end = (g >= 0 && g < G) ? __ldg(a.seg + g + 1) : 0;
+        }
+        int64_t qn = qw + QBLOCK;
+        if (++i == rounds) {
+            i = 0;
+            c0 += (int64_t)gridDim.x * QBLOCK * rounds;
+            qn = c0 + warp * 32;
+        }
+        const bool full = VEC && (qw + 32 <= a.Q);
+        const int64_t q = qw + lane;
+        float d0, d1, d2;
+        if (full) {
+            // re-distribute the warp's 24 float4 of directions: lane L takes floats 3L..3L+2
+            if (lane < 24) reinterpret_cast<float4*>(wb)[lane] = pv;
+            __syncwarp();
+            d0 = wb[3 * lane]; d1 = wb[3 * lane + 1]; d2 = wb[3 * lane + 2];
+            __syncwarp();
+        } else {
+            if (q >= a.Q) break;
+            d0 = n0; d1 = n1; d2 = n2;
+        }
+        load_dirs(qn);
+        int gq = 0;
+        if (a.glyph) {
+            gq = __ldg(a.glyph + q);
+        } else if (a.seg) {
+            if (q >= seg_end || g < 0) {
+                if (g < 0 && q >= __ldg(a.seg)) g = 0;
+                while (g >= 0 && g < G && q >= __ldg(a.seg + g + 1)) ++g;
+                seg_end = (g >= 0 && g < G) ? __ldg(a.seg + g + 1) : INT64_MAX;
+            }
+            gq = g;
+        }
+        bool valid = true;
+        if (gq < 0 || gq >= G) { valid = false; status |= SHM_DEV_BOUNDS; }
+        QueryResult r;
+        Chart c;
+        if (valid) {
+            const GlyphRef Gr = glyph_ref(a.L, gq);
+            if constexpr (RECON < 0) valid = query_one<DT, LAYOUT>(a.L, Gr, d0, d1, d2, r, c);
+            else valid = recon_one<RECON, DT>(a.L, Gr, d0, d1, d2, r, c);
+            if (!valid) status |= SHM_DEV_NONFINITE;
+        }
+        if (!valid) {
+            r.R = r.Ru = r.Rv = qnan;
+            r.grad = Vec3{qnan, qnan, qnan};
+            r.f = r.i = r.j = -1;
+        }
+        const Vec3 n = (a.normal && valid) ? surface_normal(d0, d1, d2, r.R, r.grad) : Vec3{qnan, qnan, qnan};
+        if (a.R) __stcs(a.R + q, r.R);
+        if (full) {
+            if (a.grad) {
+                wb[3 * lane] = r.grad.x; wb[3 * lane + 1] = r.grad.y; wb[3 * lane + 2] = r.grad.z;
                 __syncwarp();
-                d0 = wb[3 * lane]; d1 = wb[3 * lane + 1]; d2 = wb[3 * lane + 2];
+                if (lane < 24) __stcs(reinterpret_cast<float4*>(a.grad) + (3 * qw) / 4 + lane, reinterpret_cast<const float4*>(wb)[lane]);
                 __syncwarp();
-            } else {
-                if (q >= a.Q) break;
-                d0 = n0; d1 = n1; d2 = n2;
             }
-            // prefetch the next round's directions: the latency overlaps the table fetch below
-            if (it + 1 < QIT) {
-                const int64_t qn = qw + QBLOCK;
-                if (VEC && qn + 32 <= a.Q) {
-                    if (lane < 24) pv = __ldg(dirs4 + (3 * qn) / 4 + lane);
-                } else if (qn + lane < a.Q) {
-                    n0 = __ldcs(a.dirs + 3 * (qn + lane));
-                    n1 = __ldcs(a.dirs + 3 * (qn + lane) + 1);
-                    n2 = __ldcs(a.dirs + 3 * (qn + lane) + 2);
-                }
+            if (a.normal) {
+                wb[3 * lane] = n.x; wb[3 * lane + 1] = n.y; wb[3 * lane + 2] = n.z;
+                __syncwarp();
+                if (lane < 24) __stcs(reinterpret_cast<float4*>(a.normal) + (3 * qw) / 4 + lane, reinterpret_cast<const float4*>(wb)[lane]);
+                __syncwarp();
             }
-            int gq = 0;
-            if (a.glyph) {
-                gq = __ldg(a.glyph + q);
-            } else if (a.seg) {
-                if (q >= seg_end || g < 0) {
-                    if (g < 0 && q >= __ldg(a.seg)) g = 0;
-                    while (g >= 0 && g < G && q >= __ldg(a.seg + g + 1)) ++g;
-                    seg_end = (g >= 0 && g < G) ? __ldg(a.seg + g + 1) : INT64_MAX;
-                }
-                gq = g;
+        } else {
+            if (a.grad) {
+                a.grad[3 * q] = r.grad.x;
+                a.grad[3 * q + 1] = r.grad.y;
+                a.grad[3 * q + 2] = r.grad.z;
             }
-            bool valid = true;
-            if (gq < 0 || gq >= G) { valid = false; status |= SHM_DEV_BOUNDS; }
-            QueryResult r;
-            Chart c;
-            if (valid) {
-                const GlyphRef Gr = glyph_ref(a.L, gq);
-                if constexpr (RECON < 0) valid = query_one<DT, LAYOUT>(a.L, Gr, d0, d1, d2, r, c);
-                else valid = recon_one<RECON, DT>(a.L, Gr, d0, d1, d2, r, c);
-                if (!valid) status |= SHM_DEV_NONFINITE;
-            }
-            if (!valid) {
-                r.R = r.Ru = r.Rv = qnan;
-                r.grad = Vec3{qnan, qnan, qnan};
-                r.f = r.i = r.j = -1;
-            }
-            const Vec3 n = (a.normal && valid) ? surface_normal(d0, d1, d2, r.R, r.grad) : Vec3{qnan, qnan, qnan};
-            if (a.R) __stcs(a.R + q, r.R);
-            if (full) {
-                if (a.grad) {
-                    wb[3 * lane] = r.grad.x; wb[3 * lane + 1] = r.grad.y; wb[3 * lane + 2] = r.grad.z;
-                    __syncwarp();
-                    if (lane < 24) __stcs(reinterpret_cast<float4*>(a.grad) + (3 * qw) / 4 + lane, reinterpret_cast<const float4*>(wb)[lane]);
-                    __syncwarp();
-                }
-                if (a.normal) {
-                    wb[3 * lane] = n.x; wb[3 * lane + 1] = n.y; wb[3 * lane + 2] = n.z;
-                    __syncwarp();
-                    if (lane < 24) __stcs(reinterpret_cast<float4*>(a.normal) + (3 * qw) / 4 + lane, reinterpret_cast<const float4*>(wb)[lane]);
-                    __syncwarp();
-                }
-            } else {
-                if (a.grad) {
-                    a.grad[3 * q] = r.grad.x;
-                    a.grad[3 * q + 1] = r.grad.y;
-                    a.grad[3 * q + 2] = r.grad.z;
-                }
-                if (a.normal) {
-                    a.normal[3 * q] = n.x;
-                    a.normal[3 * q + 1] = n.y;
-                    a.normal[3 * q + 2] = n.z;
-                }
-            }
-            if (a.chart) {
-                a.chart[2 * q] = r.Ru;
-                a.chart[2 * q + 1] = r.Rv;
-            }
-            if (a.fij) {
-                a.fij[3 * q] = r.f;
-                a.fij[3 * q + 1] = r.i;
-                a.fij[3 * q + 2] = r.j;
+            if (a.normal) {
+                a.normal[3 * q] = n.x;
+                a.normal[3 * q + 1] = n.y;
+                a.normal[3 * q + 2] = n.z;
             }
         }
+        if (a.chart) {
+            a.chart[2 * q] = r.Ru;
+            a.chart[2 * q + 1] = r.Rv;
+        }
+        if (a.fij) {
+            a.fij[3 * q] = r.f;
+            a.fij[3 * q + 1] = r.i;
+            a.fij[3 * q + 2] = r.j;
+        }
+        qw = qn;
     }
     report_status(a.dev_status, status);
 }
@@ -178,17 +175,19 @@ cudaError_t launch_fwd_v(const QueryArgs& a, cudaStream_t s)
     static int resident = 0;
     if (resident == 0) {
         int r = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK, QIT>, QBLOCK,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK>, QBLOCK,
                                                           0) != cudaSuccess ||
             r < 1)
             r = QueryOccupancy<RECON, QBLOCK>::min_blocks;
         resident = r;
     }
-    int64_t blocks = (a.Q + (int64_t)QBLOCK * QIT - 1) / ((int64_t)QBLOCK * QIT);
     const int64_t cap = (int64_t)sm_count() * resident;
+    const int64_t total = (a.Q + QBLOCK - 1) / QBLOCK;
+    int64_t rounds = a.seg ? (total + cap - 1) / cap : 1;
+    if (rounds > QIT) rounds = QIT;
+    int64_t blocks = (total + rounds - 1) / rounds;
     if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK, QIT><<<(unsigned)blocks, QBLOCK, 0, s>>>(a);
+    k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK><<<(unsigned)blocks, QBLOCK, 0, s>>>(a, (int)rounds);
     return cudaGetLastError();
 }
 

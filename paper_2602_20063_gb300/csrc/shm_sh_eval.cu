@@ -193,21 +193,6 @@ __device__ __forceinline__ void ev_slab(const EvArgs& a, const float4* co, const
     }
 }
 
-// Largest g in [0, G] with seg[g] <= q (q >= seg[0]), searched by the whole warp 32 ways at a time.
-__device__ __forceinline__ int seg_find_warp(const int64_t* seg, int G, int64_t q, int lane)
-{
-    int lo = 0, n = G + 1;
-    while (n > 1) {
-        const int step = (n + 31) / 32;
-        const int at = lane * step;
-        const unsigned m = __ballot_sync(0xffffffffu, at < n && __ldg(seg + lo + at) <= q);
-        const int k = 31 - __clz((int)(m | 1u));
-        lo += k * step;
-        n = min(step, n - k * step);
-    }
-    return lo;
-}
-
 // Warp w of W takes queries [Q w / W, Q (w + 1) / W) and walks the glyphs they belong to.
 __global__ void __launch_bounds__(EV_BLOCK, EV_RES) k_sh_eval_seg(EvArgs a, const __grid_constant__ EvTable T)
 {
@@ -224,7 +209,7 @@ __global__ void __launch_bounds__(EV_BLOCK, EV_RES) k_sh_eval_seg(EvArgs a, cons
     const int64_t qe = min(a.Q, q + per);
     uint32_t status = 0;
     int g = 0;
-    if (a.seg && q < qe) g = (q < __ldg(a.seg)) ? -1 : seg_find_warp(a.seg, a.G, q, lane);
+    if (a.seg && q < qe) g = (q < __ldg(a.seg)) ? -1 : seg_find_warp(a.seg, a.G, q);
     while (q < qe) {
         int64_t e = qe;  // end of glyph g's queries within the warp's range
         if (a.seg) {
