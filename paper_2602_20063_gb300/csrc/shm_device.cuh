@@ -384,8 +384,8 @@ __device__ __forceinline__ void bspline3(float s, float w[4])
     w[3] = s3 * (1.0f / 6.0f);
 }
 
-template <int DT>
-__device__ __forceinline__ float tensor16(const ValueFace<DT>& V, int i, int j, const float wu[4], const float wv[4])
+template <class VF>
+__device__ __forceinline__ float tensor16(const VF& V, int i, int j, const float wu[4], const float wv[4])
 {
     float acc = 0.0f;
 #pragma unroll
@@ -398,8 +398,8 @@ __device__ __forceinline__ float tensor16(const ValueFace<DT>& V, int i, int j, 
     return acc;
 }
 
-template <int DT>
-__device__ __forceinline__ float bilinear_at(const ValueFace<DT>& V, int i, int j, float s, float t)
+template <class VF>
+__device__ __forceinline__ float bilinear_at(const VF& V, int i, int j, float s, float t)
 {
     const float a = V(i, j), b = V(i + 1, j), c = V(i, j + 1), d = V(i + 1, j + 1);
     const float lo = fmaf(s, b - a, a), hi = fmaf(s, d - c, c);
@@ -408,8 +408,8 @@ __device__ __forceinline__ float bilinear_at(const ValueFace<DT>& V, int i, int 
 
 // Cubic B-spline value at cell (k, l) shifted by (di, dj) texels, the cell clamped to [0, N]
 // and the local coordinate carried along.
-template <int DT>
-__device__ __forceinline__ float bspline_at(const ValueFace<DT>& V, int N, int i, int j, float s, float t)
+template <class VF>
+__device__ __forceinline__ float bspline_at(const VF& V, int N, int i, int j, float s, float t)
 {
     const int ic = min(max(i, 0), N), jc = min(max(j, 0), N);
     float wu[4], wv[4];
@@ -418,18 +418,57 @@ __device__ __forceinline__ float bspline_at(const ValueFace<DT>& V, int N, int i
     return tensor16(V, ic, jc, wu, wv);
 }
 
-template <int METHOD, int DT>
-__device__ __forceinline__ bool recon_one(const LutView& L, const GlyphRef& G, float d0, float d1, float d2,
-                                          QueryResult& out, Chart& c)
+// B-spline value at a cell and at its four shifted neighbours (v[0]; i + 1, i - 1, j + 1, j - 1 in
+// v[1..4]) where no shifted cell is clamped: all five share the weights, and the five 16-tap
+// footprints share 32 taps and their row sums (the operations and their order are tensor16's).
+template <class VF>
+__device__ __forceinline__ void bspline_cross(const VF& V, int i, int j, float s, float t, float v[5])
+{
+    float wu[4], wv[4];
+    bspline3(s, wu);
+    bspline3(t, wv);
+    float row[6];  // rows j-2 .. j+3 at cell i
+#pragma unroll
+    for (int b = 0; b < 5; ++b) v[b] = 0.0f;
+#pragma unroll
+    for (int b = 0; b < 6; ++b) {
+        const bool mid = b >= 1 && b <= 4;
+        float x[6];  // taps i-2 .. i+3
+#pragma unroll
+        for (int a = 0; a < 6; ++a) x[a] = (mid || (a >= 1 && a <= 4)) ? V(i - 2 + a, j - 2 + b) : 0.0f;
+        row[b] = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) row[b] = fmaf(wu[a], x[a + 1], row[b]);
+        if (mid) {
+            float up = 0.0f, dn = 0.0f;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                up = fmaf(wu[a], x[a + 2], up);
+                dn = fmaf(wu[a], x[a], dn);
+            }
+            v[0] = fmaf(wv[b - 1], row[b], v[0]);
+            v[1] = fmaf(wv[b - 1], up, v[1]);
+            v[2] = fmaf(wv[b - 1], dn, v[2]);
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        v[3] = fmaf(wv[b], row[b + 2], v[3]);
+        v[4] = fmaf(wv[b], row[b], v[4]);
+    }
+}
+
+// One baseline query; face(f) gives the value face (a functor of texel indices).
+template <int METHOD, class Face>
+__device__ __forceinline__ bool recon_eval(const Face& face, int N, float r0, float d0, float d1, float d2,
+                                           QueryResult& out, Chart& c)
 {
     if (!chart_of(d0, d1, d2, c)) return false;
-    const int N = G.N;
     int i, j;
     float s, t;
     cell_of(pick3(c.k1, d0, d1, d2), c.m, c.im, N, i, s);
     cell_of(pick3(c.k2, d0, d1, d2), c.m, c.im, N, j, t);
-    const int S = N + 4;
-    const ValueFace<DT> V{L.data, G.base + (int64_t)c.f * S * S, S};
+    const auto V = face(c.f);
     const float hN = 0.5f * (float)N;
     float r, Ru = 0.0f, Rv = 0.0f;
     if (METHOD == SHM_RECON_NEAREST) {
@@ -444,29 +483,32 @@ __device__ __forceinline__ bool recon_one(const LutView& L, const GlyphRef& G, f
         float wu[4], dwu[4], wv[4], dwv[4];
         catmull_rom(s, wu, dwu);
         catmull_rom(t, wv, dwv);
-        float acc = 0.0f, au = 0.0f, av = 0.0f;
+        // (row, s-derivative row) and (value, s-derivative) as pairs
+        float2 acc = bc(0.0f);
+        float av = 0.0f;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            float row = 0.0f, drow = 0.0f;
+            float2 row = bc(0.0f);
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const float v = V(i - 1 + a, j - 1 + b);
-                row = fmaf(wu[a], v, row);
-                drow = fmaf(dwu[a], v, drow);
-            }
-            acc = fmaf(wv[b], row, acc);
-            au = fmaf(wv[b], drow, au);
-            av = fmaf(dwv[b], row, av);
+            for (int a = 0; a < 4; ++a) row = pfma(make_float2(wu[a], dwu[a]), bc(V(i - 1 + a, j - 1 + b)), row);
+            acc = pfma(bc(wv[b]), row, acc);
+            av = fmaf(dwv[b], row.x, av);
         }
-        r = acc;
-        Ru = (float)N * au;
+        r = acc.x;
+        Ru = (float)N * acc.y;
         Rv = (float)N * av;
+    } else if (i >= 1 && i < N && j >= 1 && j < N) {
+        float v[5];
+        bspline_cross(V, i, j, s, t, v);
+        r = v[0];
+        Ru = (v[1] - v[2]) * hN;
+        Rv = (v[3] - v[4]) * hN;
     } else {
         r = bspline_at(V, N, i, j, s, t);
         Ru = (bspline_at(V, N, i + 1, j, s, t) - bspline_at(V, N, i - 1, j, s, t)) * hN;
         Rv = (bspline_at(V, N, i, j + 1, s, t) - bspline_at(V, N, i, j - 1, s, t)) * hN;
     }
-    out.R = G.r0 + r;
+    out.R = r0 + r;
     out.Ru = Ru;
     out.Rv = Rv;
     out.grad = s2_gradient(c, Ru, Rv);
@@ -474,6 +516,15 @@ __device__ __forceinline__ bool recon_one(const LutView& L, const GlyphRef& G, f
     out.i = i;
     out.j = j;
     return true;
+}
+
+template <int METHOD, int DT>
+__device__ __forceinline__ bool recon_one(const LutView& L, const GlyphRef& G, float d0, float d1, float d2,
+                                          QueryResult& out, Chart& c)
+{
+    const int S = G.N + 4;
+    const auto face = [&](int f) { return ValueFace<DT>{L.data, G.base + (int64_t)f * S * S, S}; };
+    return recon_eval<METHOD>(face, G.N, G.r0, d0, d1, d2, out, c);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -50,3 +50,28 @@ def test_split_equals_per_query(S, N, dtype, lens):
         for k in want:
             assert torch.equal(got[k].view(torch.int32), ref[k].view(torch.int32)), (k, want)
         assert st[0].item() == st[1].item() != 0
+
+
+@pytest.mark.parametrize("method", [0, 1, 2, 3])
+@pytest.mark.parametrize("N,dtype", [(1, 0), (2, 1), (9, 0), (9, 1), (32, 0), (33, 2), (44, 0), (45, 1), (64, 0)])
+def test_split_value_tables_equal_per_query(S, method, N, dtype):
+    """Value-only baselines: tables that are no multiple of 16 bytes (odd N), one and two per CTA, and
+    (N = 64 f32, 111 KB) near the largest that is staged; the last glyph ends at the pool's end."""
+    n = np.asarray([1300 + 211 * (g % 9) for g in range(23)] + [0, 120000])
+    G, lead, tail = len(n), 33, 40
+    seg = np.concatenate([[0], np.cumsum(n)]).astype(np.int64) + lead
+    Q = int(seg[-1]) + tail
+    ids = np.full(Q, -1, dtype=np.int32)
+    ids[lead:Q - tail] = np.repeat(np.arange(G), n)
+    lut = S.alloc_lut(G, N, dtype, S.SHM_LAYOUT_VALUE, r0=np.linspace(-0.2, 0.3, G).astype(np.float32))
+    g = torch.Generator(device="cuda").manual_seed(N)
+    lut.data.copy_(1.0 + 0.1 * torch.randn(lut.data.shape, generator=g, device="cuda"))
+    d = torch.from_numpy(I.directions(Q, 60 + N)).cuda()
+    d[lead + 1] = 0.0
+    want = ("R", "grad", "normal", "chart", "fij")
+    st = torch.zeros(2, dtype=torch.int32, device="cuda")
+    ref = S.query_recon(lut, method, d, glyph=torch.from_numpy(ids).cuda(), want=want, dev_status=st[:1])
+    got = S.query_recon(lut, method, d, seg=torch.from_numpy(seg).cuda(), want=want, dev_status=st[1:])
+    for k in want:
+        assert torch.equal(got[k].view(torch.int32), ref[k].view(torch.int32)), k
+    assert st[0].item() == st[1].item() != 0
