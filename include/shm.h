@@ -298,6 +298,14 @@ shm_status shm_query_backward(const shm_lut* lut, int64_t Q, const float* dirs,
                               const float* ggrad, const float* gnormal, const shm_lut* dlut,
                               float* ddirs, uint32_t flags, int32_t* dev_status, shm_stream stream);
 
+/* shm_query_backward with dlut written (=) instead of accumulated into: every record of every glyph
+ * is set, to zero where no query contributes, and dlut needs no clearing before the call.  Uniform
+ * resolution (dlut->N_uniform > 0, else SHM_ERR_UNSUPPORTED); everything else as shm_query_backward. */
+shm_status shm_query_backward_set(const shm_lut* lut, int64_t Q, const float* dirs,
+                                  const int32_t* glyph, const int64_t* seg, const float* gR,
+                                  const float* ggrad, const float* gnormal, const shm_lut* dlut,
+                                  float* ddirs, uint32_t flags, int32_t* dev_status, shm_stream stream);
+
 /* Reverse mode of the SH bake (Algorithm 1 is linear in the coefficients): dcoeffs[g][k] (=) sum
  * over texels and channels of dlut[g] * basis_k.  dlut: float32 texel layout, uniform N, 16-byte
  * aligned; basis from shm_sh_basis(N, L).

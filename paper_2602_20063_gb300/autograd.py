@@ -35,11 +35,13 @@ class _Query(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gR, gG, gN):
         table, dirs = ctx.saved_tensors
-        dl = B.like_lut(ctx.lut, zero=True)
+        # a uniform pool's gradient is written by the reverse pass; only uneven pools are cleared first
+        uniform = ctx.lut.N_uniform > 0
+        dl = B.like_lut(ctx.lut, zero=not uniform)
         want_dirs = ctx.needs_input_grad[1]
         c = lambda t: None if t is None else t.contiguous()
         dd = B.query_backward(ctx.lut, dirs.contiguous(), dl, gR=c(gR), ggrad=c(gG), gnormal=c(gN), glyph=ctx.glyph,
-                              seg=ctx.seg, want_ddirs=want_dirs, deterministic=ctx.deterministic)
+                              seg=ctx.seg, want_ddirs=want_dirs, deterministic=ctx.deterministic, overwrite=uniform)
         return (dl.data if ctx.needs_input_grad[0] else None), dd, None, None, None, None
 
 

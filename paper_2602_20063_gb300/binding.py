@@ -84,6 +84,7 @@ _SIGS = {
     "shm_lut_bounds": (C.c_int, [_VP, _VP, _VP]),
     "shm_build_mip": (C.c_int, [_VP, _VP, _VP, _VP]),
     "shm_query_backward": (C.c_int, [_VP, _I64, _VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP, C.c_uint32, _VP, _VP]),
+    "shm_query_backward_set": (C.c_int, [_VP, _I64, _VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP, C.c_uint32, _VP, _VP]),
     "shm_build_lut_backward": (C.c_int, [_VP, _I32, _VP, _VP, C.c_uint32, _VP]),
     "shm_fit_backward": (C.c_int, [_VP, _I64, _VP, _VP, _VP, _VP, _VP, C.c_float, C.c_float, _VP, _VP, _VP, _VP]),
     "shm_adam_step": (C.c_int, [_VP, _VP, _VP, _VP, _I64, C.c_float, C.c_float, C.c_float, C.c_float, _I32, _I32, _VP]),
@@ -456,18 +457,19 @@ def mip_chain(fine: Lut, levels: int, dtype: int = None, layout: int = None, str
 
 # ------------------------------------------------------------------------------------------- adjoint
 def query_backward(lut: Lut, dirs: torch.Tensor, dlut: Lut, gR=None, ggrad=None, gnormal=None, glyph=None, seg=None,
-                   want_ddirs=True, dev_status=None, stream=None, deterministic=False):
+                   want_ddirs=True, dev_status=None, stream=None, deterministic=False, overwrite=False):
     """shm_query_backward: accumulates into dlut (float32 texel layout); returns ddirs or None.
-    deterministic=True (SHM_BWD_DETERMINISTIC, segments only): dlut bit-identical run to run."""
+    deterministic=True (SHM_BWD_DETERMINISTIC, segments only): dlut bit-identical run to run.
+    overwrite=True (shm_query_backward_set, uniform resolution): dlut is written, whatever it held."""
     _need(dirs, torch.float32, name="dirs")
     Q = dirs.shape[0]
     for t, nm in ((gR, "gR"), (ggrad, "ggrad"), (gnormal, "gnormal")):
         _need(t, torch.float32, name=nm)
     ddirs = _io_empty((Q, 3), torch.float32, dirs) if want_ddirs else None
-    st = lib().shm_query_backward(C.byref(lut.c()), Q, _io_ptr(dirs), _io_ptr(glyph), _io_ptr(seg), _io_ptr(gR),
-                                  _io_ptr(ggrad), _io_ptr(gnormal), C.byref(dlut.c()), _io_ptr(ddirs),
-                                  C.c_uint32(SHM_BWD_DETERMINISTIC if deterministic else 0), _io_ptr(dev_status),
-                                  _stream(stream))
+    fn = lib().shm_query_backward_set if overwrite else lib().shm_query_backward
+    st = fn(C.byref(lut.c()), Q, _io_ptr(dirs), _io_ptr(glyph), _io_ptr(seg), _io_ptr(gR), _io_ptr(ggrad),
+            _io_ptr(gnormal), C.byref(dlut.c()), _io_ptr(ddirs),
+            C.c_uint32(SHM_BWD_DETERMINISTIC if deterministic else 0), _io_ptr(dev_status), _stream(stream))
     _check(st, "shm_query_backward")
     return ddirs
 

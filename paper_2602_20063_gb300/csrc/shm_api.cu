@@ -468,10 +468,10 @@ shm_status shm_build_mip(const shm_lut* fine, const shm_lut* coarse, int32_t* de
     return map_cuda(launch_mip(view(fine), view(coarse), coarse->data, dev_status, z, s));
 }
 
-shm_status shm_query_backward(const shm_lut* lut, int64_t Q, const float* dirs, const int32_t* glyph,
-                              const int64_t* seg, const float* gR, const float* ggrad, const float* gnormal,
-                              const shm_lut* dlut, float* ddirs, uint32_t flags, int32_t* dev_status,
-                              shm_stream stream)
+static shm_status query_backward(const shm_lut* lut, int64_t Q, const float* dirs, const int32_t* glyph,
+                                 const int64_t* seg, const float* gR, const float* ggrad, const float* gnormal,
+                                 const shm_lut* dlut, float* ddirs, uint32_t flags, int32_t* dev_status,
+                                 shm_stream stream, bool set)
 {
     shm_status st = check_lut(lut);
     if (st != SHM_OK) return st;
@@ -483,6 +483,7 @@ shm_status shm_query_backward(const shm_lut* lut, int64_t Q, const float* dirs, 
     if (Q < 0 || (Q > 0 && !dirs)) return SHM_ERR_INVALID_ARG;
     const bool det = (flags & SHM_BWD_DETERMINISTIC) != 0;
     if (det && (glyph || !seg)) return SHM_ERR_UNSUPPORTED;
+    if (set && dlut->N_uniform <= 0) return SHM_ERR_UNSUPPORTED;
     if ((st = same_resolutions(lut, dlut, (cudaStream_t)stream)) != SHM_OK) return st;
     BackwardArgs a;
     a.L = view(lut);
@@ -498,11 +499,28 @@ shm_status shm_query_backward(const shm_lut* lut, int64_t Q, const float* dirs, 
     a.ddirs = ddirs;
     a.dev_status = dev_status;
     a.fit = 0;
+    a.set = set ? 1 : 0;
     a.R_target = a.n_target = nullptr;
     a.w_value = a.w_normal = 0.0f;
     a.loss = nullptr;
     if ((st = resolve_io(a)) != SHM_OK) return st;
     return map_cuda(det ? launch_query_bwd_det(a, (cudaStream_t)stream) : launch_query_bwd(a, (cudaStream_t)stream));
+}
+
+shm_status shm_query_backward(const shm_lut* lut, int64_t Q, const float* dirs, const int32_t* glyph,
+                              const int64_t* seg, const float* gR, const float* ggrad, const float* gnormal,
+                              const shm_lut* dlut, float* ddirs, uint32_t flags, int32_t* dev_status,
+                              shm_stream stream)
+{
+    return query_backward(lut, Q, dirs, glyph, seg, gR, ggrad, gnormal, dlut, ddirs, flags, dev_status, stream, false);
+}
+
+shm_status shm_query_backward_set(const shm_lut* lut, int64_t Q, const float* dirs, const int32_t* glyph,
+                                  const int64_t* seg, const float* gR, const float* ggrad, const float* gnormal,
+                                  const shm_lut* dlut, float* ddirs, uint32_t flags, int32_t* dev_status,
+                                  shm_stream stream)
+{
+    return query_backward(lut, Q, dirs, glyph, seg, gR, ggrad, gnormal, dlut, ddirs, flags, dev_status, stream, true);
 }
 
 shm_status shm_fit_backward(const shm_lut* lut, int64_t Q, const float* dirs, const int32_t* glyph,
@@ -529,6 +547,7 @@ shm_status shm_fit_backward(const shm_lut* lut, int64_t Q, const float* dirs, co
     a.ddirs = nullptr;
     a.dev_status = dev_status;
     a.fit = 1;
+    a.set = 0;
     a.R_target = R_target;
     a.n_target = n_target;
     a.w_value = w_value;

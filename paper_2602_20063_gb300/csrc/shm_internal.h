@@ -118,6 +118,7 @@ struct BackwardArgs {
     int32_t* dev_status;
     // fused fit loss (fit != 0): upstream gradients from L = sum_q w_v (R - R_t)^2 + w_n |n - n_t|^2
     int fit;
+    int set;  // != 0: dL/dtable is written, not accumulated into (uniform resolution)
     const float* R_target;
     const float* n_target;
     float w_value, w_normal;

@@ -134,20 +134,51 @@ __global__ void __launch_bounds__(BBLOCK, 4) k_query_bwd(BackwardArgs a)
     report_status(a.dev_status, status);
 }
 
-// Per-glyph segments on tables that fit in shared memory: one CTA per glyph stages the table (as
-// the forward does) and answers the footprint reads from it; the gradient atomics of a glyph then
-// all come from one SM within a short window, so its dL/dtable slab stays in L2 while it is hit.
+// Per-glyph segments on tables that fit in shared memory: a CTA takes one unit of the path through
+// glyphs and queries (shm_stage.cuh), stages each glyph's table (as the forward does) and answers the
+// footprint reads from it; the gradient atomics of a glyph then come from one SM, or the few that share
+// it, within a short window, so its dL/dtable slab stays in L2 while it is hit.
+//
+// SET: the gradient table is written instead of accumulated into.  A glyph that lies wholly inside a unit
+// has its slab zeroed by that CTA while its table copy is in flight, so the zeros and the sums meet in L2
+// and DRAM sees one write of the slab instead of a fill, a read and a write; the glyphs that a unit
+// boundary cuts are zeroed first by k_zero_cut.
 constexpr int SBB = 512;
+constexpr int BWD_PATH_BYTES = 64;  // table bytes per unit of path cost: the copy and the slab's traffic in queries
 
-template <int DT, bool FIT>
-__global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uint32_t table_bytes)
+__device__ __forceinline__ void zero_slab(float4* slab, int records, int tid, int threads)
+{
+    for (int r = tid; r < records; r += threads) slab[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// Block b zeroes the slab of the glyph that the boundary between units b and b + 1 cuts, unless an
+// earlier boundary cuts it too.
+__global__ void __launch_bounds__(1024) k_zero_cut(const int64_t* seg, int G, int64_t Q, int64_t w, int64_t units,
+                                                   float4* dlut, int records)
+{
+    __shared__ int s_g;
+    if (threadIdx.x < 32) {
+        const int64_t D = stage::unit_cost(seg, G, Q, w, blockIdx.x + 1, units), before = stage::unit_cost(seg, G, Q, w, blockIdx.x, units);
+        const int g = stage::path_at(seg, G, Q, w, D).g;
+        const bool cut = g < G && stage::cost_of(seg, Q, w, g) < D && stage::cost_of(seg, Q, w, g) >= before;
+        if (threadIdx.x == 0) s_g = cut ? g : -1;
+    }
+    __syncthreads();
+    if (s_g >= 0) zero_slab(dlut + (int64_t)s_g * records, records, threadIdx.x, 1024);
+}
+
+template <int DT, bool FIT, bool SET>
+__global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uint32_t table_bytes, int nbuf)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_abort;
+    __shared__ stage::Pos s_unit[2];
     const uint32_t bar = (uint32_t)__cvta_generic_to_shared(smem);
-    const unsigned char* table = smem + stage::TABLE_OFFSET;
+    const unsigned char* tables = smem + stage::TABLE_OFFSET;
+    const uint32_t table_s = bar + stage::TABLE_OFFSET;
     const int tid = threadIdx.x;
     const int G = a.L.n_glyphs, N = a.L.N_uniform, P = N + 2;
+    const int records = 6 * P * P;
     uint32_t status = 0;
     float loss_acc = 0.0f;
     const float qnan = __int_as_float(0x7fc00000);
@@ -165,30 +196,57 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
     }
     if (tid == 0) {
         stage::init(bar);
+        stage::init(bar + 8);
         s_abort = 0;
     }
-    __syncthreads();
-    auto fetch = [table, P](int f, int i, int j) { return stage::corners<DT>(table, P, f, i, j); };
-    uint32_t phase = 0;
-    for (int g = blockIdx.x; g < G; g += gridDim.x) {
-        const int64_t s0 = min(max(__ldg(a.seg + g), (int64_t)0), a.Q);
-        const int64_t s1 = min(max(__ldg(a.seg + g + 1), s0), a.Q);
-        if (s1 <= s0) continue;  // block-uniform
-        if (tid == 0)
-            stage::issue(bar, bar + stage::TABLE_OFFSET,
-                         reinterpret_cast<const unsigned char*>(a.L.data) + (size_t)g * table_bytes, table_bytes);
-        if (!stage::bar_wait(bar, phase, stage::WAIT_NS)) s_abort = 1;
+    const int64_t w = table_bytes / BWD_PATH_BYTES;
+    stage::Pos start, end;
+    stage::unit_of(a.seg, G, a.Q, w, s_unit, start, end);  // its barrier also publishes the mbarriers
+
+    // SET: glyphs z .. are still to be zeroed (those wholly inside this unit, through glyph `last`)
+    int z = start.g;
+    int64_t D0 = 0, D1 = 0;
+    if (SET) {
+        D0 = stage::unit_cost(a.seg, G, a.Q, w, blockIdx.x, gridDim.x);
+        D1 = stage::unit_cost(a.seg, G, a.Q, w, blockIdx.x + 1, gridDim.x);
+    }
+    const auto zero_through = [&](int last) {
+        for (; z <= last && z < G; ++z)
+            if (stage::cost_of(a.seg, a.Q, w, z) >= D0 && stage::cost_of(a.seg, a.Q, w, z + 1) <= D1)
+                zero_slab(reinterpret_cast<float4*>(a.dlut) + (int64_t)z * records, records, tid, SBB);
+    };
+    const auto copy = [&](int g, int buf) {
+        stage::issue(bar + 8 * buf, table_s + buf * table_bytes,
+                     reinterpret_cast<const unsigned char*>(a.L.data) + (size_t)g * table_bytes, table_bytes);
+    };
+    uint32_t phase = 0;  // bit buf: parity of the buffer's next completion
+    int buf = 0;
+    stage::Part part = stage::next_part(a.seg, G, a.Q, start.g, start, end);
+    if (tid == 0 && part.a < part.b) copy(part.g, 0);
+    while (part.a < part.b) {
+        const int g = part.g;
+        const int64_t s1 = part.b;
+        const stage::Part next = stage::next_part(a.seg, G, a.Q, g + 1, start, end);
+        const bool more = next.a < next.b;
+        if (tid == 0 && more && nbuf == 2) copy(next.g, buf ^ 1);
+        if (SET) zero_through(g);
+        if (!stage::bar_wait(bar + 8 * buf, (phase >> buf) & 1, stage::WAIT_NS)) s_abort = 1;
         __syncthreads();
         if (s_abort) {
             status |= SHM_DEV_TIMEOUT;
-            if (tid == 0) stage::bar_wait(bar, phase, stage::DRAIN_NS);
+            if (tid == 0) {
+                stage::bar_wait(bar + 8 * buf, (phase >> buf) & 1, stage::DRAIN_NS);
+                if (more && nbuf == 2) stage::bar_wait(bar + 8 * (buf ^ 1), (phase >> (buf ^ 1)) & 1, stage::DRAIN_NS);
+            }
             break;
         }
-        phase ^= 1;
+        phase ^= 1u << buf;
+        const unsigned char* table = tables + buf * table_bytes;
+        auto fetch = [table, P](int f, int i, int j) { return stage::corners<DT>(table, P, f, i, j); };
         const GlyphRef Gr = glyph_ref(a.L, g);
         const int64_t dbase = glyph_ref(a.D, g).base;
         // warp-uniform trip count: the paired reductions need every lane of the warp
-        for (int64_t qw = s0 + (tid & ~31); qw < s1; qw += SBB) {
+        for (int64_t qw = part.a + (tid & ~31); qw < s1; qw += SBB) {
             const int64_t q = qw + (tid & 31);
             CaptureEmit sink;
             sink.base = dbase;
@@ -211,7 +269,11 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
             paired_reds(reinterpret_cast<float4*>(a.dlut), sink, tid & 31);
         }
         __syncthreads();  // every read of this table is done before the next copy lands
+        if (nbuf == 2) buf ^= 1;
+        else if (tid == 0 && more) copy(next.g, 0);
+        part = next;
     }
+    if (SET) zero_through(end.g);
     if (FIT) {
         for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
         if ((tid & 31) == 0 && a.loss) atomicAdd(a.loss, loss_acc);
@@ -219,22 +281,30 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
     report_status(a.dev_status, status);
 }
 
-template <int DT, bool FIT>
+template <int DT, bool FIT, bool SET>
 static cudaError_t launch_bwd_staged_ft(const BackwardArgs& a, uint32_t table_bytes, cudaStream_t s)
 {
-    const int smem = stage::TABLE_OFFSET + (int)table_bytes;
-    cudaError_t e = ensure_dynamic_smem((const void*)k_query_bwd_staged<DT, FIT>, smem);
+    const int nbuf = 2 * (int64_t)table_bytes <= STAGED_TABLE_MAX_BYTES ? 2 : 1;
+    const int smem = stage::TABLE_OFFSET + nbuf * (int)table_bytes;
+    cudaError_t e = ensure_dynamic_smem((const void*)k_query_bwd_staged<DT, FIT, SET>, smem);
     if (e != cudaSuccess) return e;
-    int64_t blocks = (int64_t)sm_count() * 2;
-    if (blocks > a.L.n_glyphs) blocks = a.L.n_glyphs;
-    k_query_bwd_staged<DT, FIT><<<(unsigned)blocks, SBB, smem, s>>>(a, table_bytes);
+    const int64_t w = table_bytes / BWD_PATH_BYTES;
+    const int64_t blocks = stage::units_for(a.Q, a.L.n_glyphs, w, (int64_t)sm_count() * 2);
+    if (SET && blocks > 1) {
+        const int P = a.L.N_uniform + 2;
+        k_zero_cut<<<(unsigned)(blocks - 1), 1024, 0, s>>>(a.seg, a.L.n_glyphs, a.Q, w, blocks,
+                                                           reinterpret_cast<float4*>(a.dlut), 6 * P * P);
+    }
+    k_query_bwd_staged<DT, FIT, SET><<<(unsigned)blocks, SBB, smem, s>>>(a, table_bytes, nbuf);
     return cudaGetLastError();
 }
 
 template <int DT>
 static cudaError_t launch_bwd_staged(const BackwardArgs& a, uint32_t table_bytes, cudaStream_t s)
 {
-    return a.fit ? launch_bwd_staged_ft<DT, true>(a, table_bytes, s) : launch_bwd_staged_ft<DT, false>(a, table_bytes, s);
+    if (a.fit) return launch_bwd_staged_ft<DT, true, false>(a, table_bytes, s);
+    return a.set ? launch_bwd_staged_ft<DT, false, true>(a, table_bytes, s)
+                 : launch_bwd_staged_ft<DT, false, false>(a, table_bytes, s);
 }
 
 template <int DT, int LAYOUT>
@@ -252,17 +322,24 @@ static cudaError_t launch_bwd_t(const BackwardArgs& a, cudaStream_t s)
 
 cudaError_t launch_query_bwd(const BackwardArgs& a, cudaStream_t s)
 {
-    if (a.Q == 0) return cudaSuccess;
+    if (a.Q == 0 && !a.set) return cudaSuccess;
     const int dt = a.L.dtype, ly = a.L.layout;
     // per-glyph segments on small uniform tables: stage each glyph's table in shared memory
-    if (a.seg && !a.glyph && a.L.N_uniform > 0 && a.D.N_uniform == a.L.N_uniform && ly == SHM_LAYOUT_TEXEL) {
+    if (a.Q > 0 && a.seg && !a.glyph && a.L.N_uniform > 0 && a.D.N_uniform == a.L.N_uniform && ly == SHM_LAYOUT_TEXEL) {
         const int64_t P = (int64_t)a.L.N_uniform + 2;
         const int64_t bytes = 6 * P * P * (dt == SHM_F32 ? 16 : 8);
-        if (bytes <= STAGED_TABLE_MAX_BYTES) {
+        const int64_t per = bytes / 128 > 256 ? bytes / 128 : 256;  // as query_is_staged
+        if (bytes <= STAGED_TABLE_MAX_BYTES && a.Q >= a.L.n_glyphs * per) {
             if (dt == SHM_F32) return launch_bwd_staged<SHM_F32>(a, (uint32_t)bytes, s);
             if (dt == SHM_F16) return launch_bwd_staged<SHM_F16>(a, (uint32_t)bytes, s);
             return launch_bwd_staged<SHM_BF16>(a, (uint32_t)bytes, s);
         }
+    }
+    if (a.set) {
+        const int64_t P = (int64_t)a.D.N_uniform + 2;
+        const cudaError_t e = cudaMemsetAsync(a.dlut, 0, (size_t)(6 * P * P * 16) * a.D.n_glyphs, s);
+        if (e != cudaSuccess) return e;
+        if (a.Q == 0) return cudaSuccess;
     }
     if (ly == SHM_LAYOUT_TEXEL) {
         if (dt == SHM_F32) return launch_bwd_t<SHM_F32, SHM_LAYOUT_TEXEL>(a, s);

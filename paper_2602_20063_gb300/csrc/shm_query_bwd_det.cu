@@ -209,6 +209,11 @@ cudaError_t launch_det_t(const BackwardArgs& a, cudaStream_t s)
 
 cudaError_t launch_query_bwd_det(const BackwardArgs& a, cudaStream_t s)
 {
+    if (a.set) {
+        const int64_t P = (int64_t)a.D.N_uniform + 2;
+        const cudaError_t e = cudaMemsetAsync(a.dlut, 0, (size_t)(6 * P * P * 16) * a.D.n_glyphs, s);
+        if (e != cudaSuccess) return e;
+    }
     if (a.Q == 0) return cudaSuccess;
     const int dt = a.L.dtype;
     if (a.L.layout == SHM_LAYOUT_TEXEL) {

@@ -116,14 +116,24 @@ __device__ __forceinline__ Part next_part(const int64_t* seg, int G, int64_t Q, 
     return Part{G, 0, 0};
 }
 
+// Cost of the path up to glyph g, and up to the start of unit u of `units`.
+__device__ __forceinline__ int64_t cost_of(const int64_t* seg, int64_t Q, int64_t w, int g)
+{
+    return seg_at(seg, Q, g) - seg_at(seg, Q, 0) + w * g;
+}
+
+__device__ __forceinline__ int64_t unit_cost(const int64_t* seg, int G, int64_t Q, int64_t w, int64_t u, int64_t units)
+{
+    const int64_t total = cost_of(seg, Q, w, G);
+    return total / units * u + total % units * u / units;
+}
+
 // This CTA's unit of the path: start and end positions through shared memory (every thread calls it).
 __device__ __forceinline__ void unit_of(const int64_t* seg, int G, int64_t Q, int64_t w, Pos* sh, Pos& start, Pos& end)
 {
     const int warp = threadIdx.x >> 5;
     if (warp < 2) {
-        const int64_t total = seg_at(seg, Q, G) - seg_at(seg, Q, 0) + w * G;
-        const Pos p = path_at(seg, G, Q, w, total / gridDim.x * (blockIdx.x + warp) +
-                                                total % gridDim.x * (blockIdx.x + warp) / gridDim.x);
+        const Pos p = path_at(seg, G, Q, w, unit_cost(seg, G, Q, w, blockIdx.x + warp, gridDim.x));
         if ((threadIdx.x & 31) == 0) sh[warp] = p;
     }
     __syncthreads();

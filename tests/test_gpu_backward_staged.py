@@ -205,3 +205,33 @@ def test_paired_reductions_across_glyphs_of_different_n(S):
     _check_dlut(dl.data.view(-1, 4).double().cpu().numpy(), dref)
     ddn = dd.double().cpu().numpy()
     assert np.isnan(ddn[~ok]).all() and np.isfinite(ddn[ok]).all()
+
+
+@pytest.mark.parametrize("dtype,N", [(0, 9), (0, 23), (1, 32)])
+@pytest.mark.parametrize("mode", ["few", "many", "sparse", "ids", "none", "det"])
+def test_written_gradient_equals_accumulated(S, mode, dtype, N):
+    """shm_query_backward_set over a gradient table full of NaN equals the accumulating pass over zeros:
+    glyphs cut by work units and whole ones, empty glyphs, batches too sparse to stage, ids, no query."""
+    counts = {"few": [0, 90000, 0, 3, 40000, 0], "many": [(g * 97) % 2600 * (g % 7 != 0) for g in range(900)],
+              "sparse": [g % 40 for g in range(300)], "ids": [4000, 0, 700], "none": [0, 0, 0],
+              "det": [700, 0, 5000, 1]}[mode]
+    seg, glyph, Q = _segments(counts, 0 if mode == "none" else 21, 0 if mode == "none" else 40)
+    G = len(counts)
+    g = torch.Generator(device="cuda").manual_seed(N)
+    lut = S.alloc_lut(G, N, dtype)
+    lut.data.copy_(1.0 + 0.1 * torch.randn(lut.data.shape, generator=g, device="cuda"))
+    d = _t(I.directions(Q, 8)) if Q else torch.empty((0, 3), device="cuda")
+    up = [torch.randn(s, generator=g, device="cuda") for s in ((Q,), (Q, 3), (Q, 3))]
+    sel = {"glyph": _t(glyph)} if mode == "ids" else {"seg": _t(seg)}
+    ref, got = S.like_lut(lut, dtype=0, zero=True), S.like_lut(lut, dtype=0)
+    got.data.fill_(float("nan"))
+    kw = dict(gR=up[0], ggrad=up[1], gnormal=up[2], deterministic=mode == "det", **sel)
+    a = S.query_backward(lut, d, ref, **kw)
+    b = S.query_backward(lut, d, got, overwrite=True, **kw)
+    assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+    r, x = ref.data.view(-1, 4).double(), got.data.view(-1, 4).double()
+    assert torch.isfinite(x).all()
+    # the same sums in another order: a few float32 roundings of the largest entry
+    assert ((x - r).abs().amax(0) <= 2e-6 * r.abs().amax(0)).all()
+    if mode == "det":
+        assert torch.equal(ref.data, got.data)
