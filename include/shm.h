@@ -256,6 +256,13 @@ int64_t shm_build_workspace_bytes(const shm_lut* lut, const shm_source* src);
 shm_status shm_build_lut(const shm_lut* lut, const shm_source* src, void* ws, size_t ws_bytes,
                          shm_stream stream);
 
+/* shm_build_lut with the tensor-core engine (SH source, float32 texel table, ws as there), which also
+ * writes the same records to `copy` (device, 16-byte aligned, not overlapping the table) from the same
+ * pass: a snapshot that a later bake into `lut` leaves alone, without reading the table back.  Other
+ * sources, dtypes and layouts, and ws == NULL: SHM_ERR_UNSUPPORTED. */
+shm_status shm_build_lut_twice(const shm_lut* lut, const shm_source* src, float* copy, void* ws,
+                               size_t ws_bytes, shm_stream stream);
+
 /* Re-encodes table `src` into `dst` (same glyphs and resolutions; any dtype/layout pair).
  * 16-bit stores round to nearest even.  dst channel 0 = src r0 + src channel 0 - dst r0. */
 shm_status shm_pack_lut(const shm_lut* src, const shm_lut* dst, shm_stream stream);

@@ -50,20 +50,37 @@ def query_fn(table: torch.Tensor, dirs: torch.Tensor, lut: B.Lut, seg=None, glyp
     return _Query.apply(table, dirs, lut, seg, glyph, deterministic)
 
 
+def _dense_texels(t: torch.Tensor, lut: B.Lut) -> bool:
+    """Whether `t` holds exactly the records of `lut`'s float32 texel layout, where the kernels may read or
+    write them in place of a copy."""
+    return (lut.dtype == B.SHM_F32 and lut.layout == B.SHM_LAYOUT_TEXEL and lut.N_uniform > 0
+            and t.dtype == torch.float32 and t.is_contiguous() and t.device == lut.data.device
+            and t.numel() == lut.n_glyphs * B.records_per_glyph_host(lut.N_uniform, lut.layout) * 4
+            and t.data_ptr() % 16 == 0)
+
+
 class _ShBake(torch.autograd.Function):
     @staticmethod
     def forward(ctx, coeffs, basis, lut, L, ws, deterministic):
-        B.build_lut(lut, B.Source(kind=B.SHM_SRC_SH, L=L, coeffs=coeffs.contiguous(), basis=basis), ws=ws)
+        src = B.Source(kind=B.SHM_SRC_SH, L=L, coeffs=coeffs.contiguous(), basis=basis)
+        if ws is not None and _dense_texels(lut.data, lut):
+            table = B.build_lut_twice(lut, src, ws)
+        else:
+            B.build_lut(lut, src, ws=ws)
+            table = lut.data.clone()
         ctx.lut, ctx.L = lut, L
         ctx.deterministic = bool(deterministic) or torch.are_deterministic_algorithms_enabled()
         ctx.save_for_backward(basis)
-        return lut.data.clone()
+        return table
 
     @staticmethod
     def backward(ctx, gtable):
         (basis,) = ctx.saved_tensors
-        D = B.like_lut(ctx.lut, r0=None)
-        D.data.copy_(gtable)
+        D = B.Lut(data=gtable, n_glyphs=ctx.lut.n_glyphs, N_uniform=ctx.lut.N_uniform)
+        if not _dense_texels(gtable, ctx.lut):
+            # strided, broadcast or unaligned upstream gradients: a dense copy first
+            D = B.like_lut(ctx.lut, r0=None)
+            D.data.copy_(gtable)
         return B.build_lut_backward(D, ctx.L, basis, deterministic=ctx.deterministic), None, None, None, None, None
 
 

@@ -79,6 +79,7 @@ _SIGS = {
     "shm_sh_basis_bytes": (C.c_int64, [_I32, _I32]),
     "shm_sh_basis": (C.c_int, [_I32, _I32, _VP, _VP]),
     "shm_build_lut": (C.c_int, [_VP, _VP, _VP, _SZ, _VP]),
+    "shm_build_lut_twice": (C.c_int, [_VP, _VP, _VP, _VP, _SZ, _VP]),
     "shm_build_workspace_bytes": (C.c_int64, [_VP, _VP]),
     "shm_pack_lut": (C.c_int, [_VP, _VP, _VP]),
     "shm_lut_bounds": (C.c_int, [_VP, _VP, _VP]),
@@ -407,6 +408,15 @@ def build_lut(lut: Lut, src: Source, ws: torch.Tensor = None, stream=None):
     engine; ws=None runs the float32 CUDA-core engine."""
     wp, wn = (None, 0) if ws is None else (_ptr(ws), ws.numel() * ws.element_size())
     _check(lib().shm_build_lut(C.byref(lut.c()), C.byref(src.c()), wp, wn, _stream(stream)), "shm_build_lut")
+
+
+def build_lut_twice(lut: Lut, src: Source, ws: torch.Tensor, stream=None) -> torch.Tensor:
+    """shm_build_lut_twice: bakes an SH source into a float32 texel `lut` and returns a second tensor with
+    the same records, written by the same pass."""
+    copy = torch.empty_like(lut.data)
+    _check(lib().shm_build_lut_twice(C.byref(lut.c()), C.byref(src.c()), _ptr(copy), _ptr(ws),
+                                     ws.numel() * ws.element_size(), _stream(stream)), "shm_build_lut_twice")
+    return copy
 
 
 def build_workspace(lut: Lut, src: Source) -> torch.Tensor:

@@ -379,7 +379,8 @@ int64_t shm_build_workspace_bytes(const shm_lut* lut, const shm_source* src)
     return sh_build_workspace_bytes(lut->n_glyphs, src->L);
 }
 
-shm_status shm_build_lut(const shm_lut* lut, const shm_source* src, void* ws, size_t ws_bytes, shm_stream stream)
+static shm_status build_lut(const shm_lut* lut, const shm_source* src, void* ws, size_t ws_bytes, shm_stream stream,
+                            float* copy)
 {
     shm_status st = check_lut(lut);
     if (st != SHM_OK) return st;
@@ -397,7 +398,7 @@ shm_status shm_build_lut(const shm_lut* lut, const shm_source* src, void* ws, si
         if (ws) {
             if ((int64_t)ws_bytes < sh_build_workspace_bytes(lut->n_glyphs, src->L) || ((uintptr_t)ws & 15u))
                 return SHM_ERR_WORKSPACE;
-            return map_cuda(launch_sh_build_tc(v, lut->data, src->L, src->coeffs, src->basis, ws, s, src->dev_status));
+            return map_cuda(launch_sh_build_tc(v, lut->data, src->L, src->coeffs, src->basis, ws, s, src->dev_status, copy));
         }
         return map_cuda(launch_sh_build(v, lut->data, src->L, src->coeffs, src->basis, s));
     case SHM_SRC_SAMPLES:
@@ -416,6 +417,21 @@ shm_status shm_build_lut(const shm_lut* lut, const shm_source* src, void* ws, si
     default:
         return SHM_ERR_INVALID_ARG;
     }
+}
+
+shm_status shm_build_lut(const shm_lut* lut, const shm_source* src, void* ws, size_t ws_bytes, shm_stream stream)
+{
+    return build_lut(lut, src, ws, ws_bytes, stream, nullptr);
+}
+
+shm_status shm_build_lut_twice(const shm_lut* lut, const shm_source* src, float* copy, void* ws, size_t ws_bytes,
+                               shm_stream stream)
+{
+    const shm_status st = check_lut(lut);
+    if (st != SHM_OK) return st;
+    if (!src || !copy || ((uintptr_t)copy & 15u) != 0) return SHM_ERR_INVALID_ARG;
+    if (src->kind != SHM_SRC_SH || lut->dtype != SHM_F32 || lut->layout != SHM_LAYOUT_TEXEL || !ws) return SHM_ERR_UNSUPPORTED;
+    return build_lut(lut, src, ws, ws_bytes, stream, copy);
 }
 
 shm_status shm_pack_lut(const shm_lut* src, const shm_lut* dst, shm_stream stream)

@@ -56,6 +56,7 @@ struct Args {
     LutView view;         // output table (any dtype / layout) for the generic epilogue
     void* data;
     int direct;           // 1: f32 texel layout, uniform N, write out[g*M + c]
+    int twice;            // direct: the same boxes also go to a second table
     int32_t* dev_status;
 };
 
@@ -91,7 +92,7 @@ __device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uin
 __global__ void __launch_bounds__(256, 1)
     k_sh_gemm_tc(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
                  const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl,
-                 const __grid_constant__ CUtensorMap mOut, Args a)
+                 const __grid_constant__ CUtensorMap mOut, const __grid_constant__ CUtensorMap mOut2, Args a)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -240,6 +241,7 @@ __global__ void __launch_bounds__(256, 1)
                     epi_bar();
                     if (issuer) {
                         tma_store_2d(&mOut, smem_u32(buf), mt * TM, g0);  // clipped at M columns, G rows
+                        if (a.twice) tma_store_2d(&mOut2, smem_u32(buf), mt * TM, g0);
                         bulk_commit();
                     }
                     ++box;
@@ -291,32 +293,15 @@ __global__ void k_split_rows(const float* __restrict__ in, int rows, int K, int6
 
 static bool make_map(CUtensorMap* m, const float* base, int rows, int Kp, int box_rows)
 {
-    EncodeFn enc = encode_fn();
-    if (!enc) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)Kp, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)Kp * 4};
-    const cuuint32_t box[2] = {(cuuint32_t)KC, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_map_2d(m, base, Kp, rows, KC, box_rows, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 
 // Output table as a 2-D tensor [G rows][M columns] f32 (row pitch M * 4 B, a multiple of 16 since
 // M = 4 * 6 (N+2)^2), stored in boxes of [OG glyphs][TM columns] without swizzle.
 static bool make_out_map(CUtensorMap* m, float* base, int G, int M)
 {
-    EncodeFn enc = encode_fn();
-    if (!enc || ((uintptr_t)base & 15u) != 0) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)M, (cuuint64_t)G};
-    const cuuint64_t strides[1] = {(cuuint64_t)M * 4};
-    const cuuint32_t box[2] = {(cuuint32_t)TM, (cuuint32_t)OG};
-    const cuuint32_t estr[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_map_2d(m, base, M, G, TM, OG, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE);
 }
-
 
 }  // namespace tc
 
@@ -338,7 +323,7 @@ cudaError_t launch_basis_split(int N, int L, float* basis, cudaStream_t s)
 }
 
 cudaError_t launch_sh_build_tc(const LutView& out, void* data, int L, const float* coeffs, const float* basis,
-                               void* ws, cudaStream_t s, int32_t* dev_status)
+                               void* ws, cudaStream_t s, int32_t* dev_status, float* copy)
 {
     const int N = out.N_uniform, G = out.n_glyphs;
     const int K = (L + 1) * (L + 1), Kp = sh_kpad(L), M = 4 * 6 * (N + 2) * (N + 2);
@@ -351,7 +336,7 @@ cudaError_t launch_sh_build_tc(const LutView& out, void* data, int L, const floa
     if (e != cudaSuccess) return e;
     const float* bhi = basis + (int64_t)K * M;
     const float* blo = bhi + (int64_t)M * Kp;
-    CUtensorMap mAh, mAl, mBh, mBl, mOut;
+    CUtensorMap mAh, mAl, mBh, mBl, mOut, mOut2;
     if (!tc::make_map(&mAh, bhi, M, Kp, tc::TM) || !tc::make_map(&mAl, blo, M, Kp, tc::TM) ||
         !tc::make_map(&mBh, chi, G, Kp, tc::TN) || !tc::make_map(&mBl, clo, G, Kp, tc::TN))
         return cudaErrorInvalidValue;
@@ -361,6 +346,8 @@ cudaError_t launch_sh_build_tc(const LutView& out, void* data, int L, const floa
     } else {
         mOut = mAh;  // unused by the generic epilogue
     }
+    mOut2 = mOut;
+    if (copy && (!direct || !tc::make_out_map(&mOut2, copy, G, M))) return cudaErrorInvalidValue;
     tc::Args a;
     a.M = M;
     a.G = G;
@@ -370,13 +357,14 @@ cudaError_t launch_sh_build_tc(const LutView& out, void* data, int L, const floa
     a.data = data;
     a.out = reinterpret_cast<float*>(data);
     a.direct = direct ? 1 : 0;
+    a.twice = copy ? 1 : 0;
     a.dev_status = dev_status;
     e = ensure_dynamic_smem((const void*)tc::k_sh_gemm_tc, (int)tc::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     const int tiles = ((M + tc::TM - 1) / tc::TM) * ((G + tc::TN - 1) / tc::TN);
     int grid = sm_count();
     if (grid > tiles) grid = tiles;
-    tc::k_sh_gemm_tc<<<grid, 256, tc::SMEM_BYTES, s>>>(mAh, mAl, mBh, mBl, mOut, a);
+    tc::k_sh_gemm_tc<<<grid, 256, tc::SMEM_BYTES, s>>>(mAh, mAl, mBh, mBl, mOut, mOut2, a);
     return cudaGetLastError();
 }
 

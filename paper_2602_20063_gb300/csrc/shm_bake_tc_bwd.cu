@@ -346,15 +346,8 @@ __global__ void k_split_basis_t(const float* __restrict__ full, int K, int Kp, i
 static bool make_map_c(CUtensorMap* m, const float* base, int rows, int M4, int box_rows, int box_c = KC,
                        bool swizzle = true)
 {
-    EncodeFn enc = encode_fn();
-    if (!enc || ((uintptr_t)base & 15u) != 0) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)M4, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)M4 * 4};
-    const cuuint32_t box[2] = {(cuuint32_t)box_c, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_map_2d(m, base, M4, rows, box_c, box_rows, swizzle ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 
 // Plan of the tensor-core adjoint for (G, K, Kp, M4) on `sms` SMs; false when it does not apply

@@ -109,7 +109,9 @@ struct GlobalUp {
 // ggrad, gnormal; zero where absent), so that their latency overlaps it.
 struct PreUp {
     float r, g0, g1, g2, n0, n1, n2;
-    __device__ __forceinline__ PreUp(const BackwardArgs& a, int64_t q)
+    PreUp() = default;
+    __device__ __forceinline__ PreUp(const BackwardArgs& a, int64_t q) { load(a, q); }
+    __device__ __forceinline__ void load(const BackwardArgs& a, int64_t q)
     {
         r = a.gR ? __ldcs(a.gR + q) : 0.0f;
         g0 = g1 = g2 = n0 = n1 = n2 = 0.0f;
@@ -127,7 +129,9 @@ struct PreUp {
 // latency overlaps it.
 struct PreFit {
     float rt, t0, t1, t2;
-    __device__ __forceinline__ PreFit(const BackwardArgs& a, int64_t q)
+    PreFit() = default;
+    __device__ __forceinline__ PreFit(const BackwardArgs& a, int64_t q) { load(a, q); }
+    __device__ __forceinline__ void load(const BackwardArgs& a, int64_t q)
     {
         rt = __ldcs(a.R_target + q);
         t0 = __ldcs(a.n_target + 3 * q);

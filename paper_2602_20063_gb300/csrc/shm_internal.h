@@ -159,7 +159,7 @@ cudaError_t launch_adam(float* param, float* grad, float* m, float* v, int64_t n
 cudaError_t launch_sh_basis(int N, int L, float* basis, cudaStream_t s);
 cudaError_t launch_basis_split(int N, int L, float* basis, cudaStream_t s);
 cudaError_t launch_sh_build_tc(const LutView& out, void* data, int L, const float* coeffs, const float* basis,
-                               void* ws, cudaStream_t s, int32_t* dev_status);
+                               void* ws, cudaStream_t s, int32_t* dev_status, float* copy);
 int sh_kpad(int L);
 int64_t sh_build_workspace_bytes(int G, int L);
 cudaError_t launch_sh_build(const LutView& out, void* data, int L, const float* coeffs, const float* basis,

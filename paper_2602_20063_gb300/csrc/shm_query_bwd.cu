@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
     const int tid = threadIdx.x;
     const int G = a.L.n_glyphs, N = a.L.N_uniform, P = N + 2;
     const int records = 6 * P * P;
+    using Up = std::conditional_t<FIT, PreFit, PreUp>;
     uint32_t status = 0;
     float loss_acc = 0.0f;
     const float qnan = __int_as_float(0x7fc00000);
@@ -229,6 +230,16 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
         const stage::Part next = stage::next_part(a.seg, G, a.Q, g + 1, start, end);
         const bool more = next.a < next.b;
         if (tid == 0 && more && nbuf == 2) copy(next.g, buf ^ 1);
+        // this thread's first inputs load while the table copy runs, each later round's under the
+        // reductions of the round before
+        float d0 = 0.f, d1 = 0.f, d2 = 0.f;
+        Up up;
+        const auto load = [&](int64_t q) {
+            if (q >= s1) return;
+            d0 = __ldcs(a.dirs + 3 * q); d1 = __ldcs(a.dirs + 3 * q + 1); d2 = __ldcs(a.dirs + 3 * q + 2);
+            up.load(a, q);
+        };
+        load(part.a + tid);
         if (SET) zero_through(g);
         if (!stage::bar_wait(bar + 8 * buf, (phase >> buf) & 1, stage::WAIT_NS)) s_abort = 1;
         __syncthreads();
@@ -253,19 +264,12 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
             sink.P = P;
             if (q < s1) {
                 float3 dd = make_float3(qnan, qnan, qnan);
-                const float d0 = __ldcs(a.dirs + 3 * q), d1 = __ldcs(a.dirs + 3 * q + 1), d2 = __ldcs(a.dirs + 3 * q + 2);
                 Chart c;
-                if constexpr (FIT) {
-                    const PreFit up(a, q);
-                    if (chart_of(d0, d1, d2, c)) bwd_query<FIT>(a, up, Gr, c, d0, d1, d2, fetch, sink, dd, loss_acc);
-                    else status |= SHM_DEV_NONFINITE;
-                } else {
-                    const PreUp up(a, q);  // issued before the chart, used after the forward recompute
-                    if (chart_of(d0, d1, d2, c)) bwd_query<FIT>(a, up, Gr, c, d0, d1, d2, fetch, sink, dd, loss_acc);
-                    else status |= SHM_DEV_NONFINITE;
-                }
+                if (chart_of(d0, d1, d2, c)) bwd_query<FIT>(a, up, Gr, c, d0, d1, d2, fetch, sink, dd, loss_acc);
+                else status |= SHM_DEV_NONFINITE;
                 if (a.ddirs) { __stcs(a.ddirs + 3 * q, dd.x); __stcs(a.ddirs + 3 * q + 1, dd.y); __stcs(a.ddirs + 3 * q + 2, dd.z); }
             }
+            load(q + SBB);
             paired_reds(reinterpret_cast<float4*>(a.dlut), sink, tid & 31);
         }
         __syncthreads();  // every read of this table is done before the next copy lands

@@ -146,6 +146,27 @@ inline EncodeFn encode_fn()
     return fn;
 }
 
+// 2-D float32 tensor map.  The driver call needs a context current on the calling thread, which a thread
+// that has made no runtime call of its own yet (an autograd worker, say) does not have: it is bound by
+// cudaSetDevice, which is legal during capture, and the call repeated.
+inline bool encode_map_2d(CUtensorMap* m, const float* base, uint64_t cols, uint64_t rows, uint32_t box_cols,
+                          uint32_t box_rows, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion promotion)
+{
+    EncodeFn enc = encode_fn();
+    if (!enc || ((uintptr_t)base & 15u) != 0) return false;
+    const cuuint64_t dims[2] = {cols, rows};
+    const cuuint64_t strides[1] = {cols * 4};
+    const cuuint32_t box[2] = {box_cols, box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        if (enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, promotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
+            return true;
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) break;
+    }
+    return false;
+}
 
 }  // namespace tc
 }  // namespace shm

@@ -166,3 +166,31 @@ def test_build_backward_glyph_group_sizing(S, per_sm):
     for r in sorted({0, R - 1, R, 2 * R - 1, G // 2, G - R, G - 1} & set(range(G))):
         oref = O.bake_sh_vjp(N, L, dl[r].double().cpu().numpy().reshape(6, N + 2, N + 2, 4))
         assert np.abs(dcn[r] - oref).max() <= 2e-5 * np.abs(oref).max(), r
+
+
+@pytest.mark.parametrize("G,N", [(1, 10), (300, 9), (257, 17)])
+def test_bake_snapshot_and_gradient_in_place(G, N):
+    """sh_bake_fn's table is a snapshot (a later bake into the lut leaves it alone) with the lut's records,
+    and its backward gives the same coefficients' gradient for a dense upstream gradient (used in place),
+    a strided one, an offset (unaligned) one and a broadcast one."""
+    import torch
+    S = shm()
+    L = 4
+    c = [torch.from_numpy(I.sh_coeffs(G, L, 3 + k).astype(np.float32)).cuda().requires_grad_(True) for k in range(2)]
+    lut = S.alloc_lut(G, N, r0=np.full(G, 0.25, np.float32))
+    src = S.Source(kind=S.SHM_SRC_SH, L=L, coeffs=c[0], basis=S.sh_basis(N, L))
+    ws = S.build_workspace(lut, src)
+    t0 = S.sh_bake_fn(c[0], src.basis, lut, L, ws=ws)
+    kept = t0.detach().clone()
+    assert torch.equal(kept, lut.data)
+    S.sh_bake_fn(c[1], src.basis, lut, L, ws=ws)
+    assert torch.equal(t0.detach(), kept) and not torch.equal(lut.data, kept)
+    g = torch.randn(t0.shape, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    n = g.numel()
+    dense = torch.autograd.grad(t0, c[0], g, retain_graph=True)[0]
+    strided = torch.empty(2 * n, device="cuda")[::2].copy_(g)
+    offset = torch.empty(n + 1, device="cuda")[1:].copy_(g)
+    for other in (strided, offset):
+        assert torch.equal(dense, torch.autograd.grad(t0, c[0], other, retain_graph=True)[0])
+    ones = torch.autograd.grad(t0.sum(), c[0], retain_graph=True)[0]
+    assert torch.equal(ones, torch.autograd.grad(t0, c[0], torch.ones_like(g))[0])
