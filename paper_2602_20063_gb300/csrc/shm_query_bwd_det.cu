@@ -27,6 +27,7 @@ namespace {
 constexpr int DBLOCK = 256;
 constexpr int DBITS = 8;   // log2(DBLOCK): query slot in the low bits of the sort key
 constexpr int DMINB = 4;   // CTAs per SM
+constexpr int DOUTSIDE = 608;  // CTAs that mark the queries outside every segment
 // Shared memory: two key buffers [DBLOCK] of KT, then the payload [5][DBLOCK] f32.
 template <class KT>
 constexpr uint32_t det_smem() { return 2 * DBLOCK * sizeof(KT) + 5 * DBLOCK * 4; }
@@ -99,11 +100,12 @@ __global__ void __launch_bounds__(DBLOCK, DMINB) k_query_bwd_det(BackwardArgs a)
     uint32_t status = 0;
     float loss_unused = 0.0f;
     const float qnan = __int_as_float(0x7fc00000);
-    {
+    const int outside = min((int)gridDim.x, DOUTSIDE);
+    if ((int)blockIdx.x < outside) {
         // queries outside every segment: NaN d/ddirs and SHM_DEV_BOUNDS
         const int64_t lo = min(max(__ldg(a.seg), (int64_t)0), a.Q);
         const int64_t hi = min(max(__ldg(a.seg + G), lo), a.Q);
-        const int64_t stride = (int64_t)gridDim.x * DBLOCK;
+        const int64_t stride = (int64_t)outside * DBLOCK;
         for (int part = 0; part < 2; ++part) {
             const int64_t b = part ? hi : 0, e = part ? a.Q : lo;
             for (int64_t q = b + (int64_t)blockIdx.x * DBLOCK + tid; q < e; q += stride) {
@@ -112,10 +114,10 @@ __global__ void __launch_bounds__(DBLOCK, DMINB) k_query_bwd_det(BackwardArgs a)
             }
         }
     }
-    for (int g = blockIdx.x; g < G; g += gridDim.x) {
+    {
+        const int g = blockIdx.x;
         const int64_t s0 = min(max(__ldg(a.seg + g), (int64_t)0), a.Q);
         const int64_t s1 = min(max(__ldg(a.seg + g + 1), s0), a.Q);
-        if (s1 <= s0) continue;  // block-uniform
         const GlyphRef Gr = glyph_ref(a.L, g);
         const int P = Gr.N + 2;
         float4* dbase = reinterpret_cast<float4*>(a.dlut) + glyph_ref(a.D, g).base;
@@ -190,10 +192,10 @@ cudaError_t launch_det_k(const BackwardArgs& a, cudaStream_t s)
     const int smem = (int)det_smem<KT>();
     cudaError_t e = ensure_dynamic_smem((const void*)k_query_bwd_det<DT, LAYOUT, KT>, smem);
     if (e != cudaSuccess) return e;
-    int64_t blocks = (int64_t)sm_count() * DMINB;
-    if (blocks > a.L.n_glyphs) blocks = a.L.n_glyphs;
-    if (blocks < 1) blocks = 1;
-    k_query_bwd_det<DT, LAYOUT, KT><<<(unsigned)blocks, DBLOCK, smem, s>>>(a);
+    // one CTA per glyph, scheduled as slots free up: with uneven segments a fixed share of the glyphs per
+    // resident CTA left most of them waiting for the longest share (4,096 glyphs, 6.1 M queries in random
+    // cuts: 533 -> 404 us; even segments 350 -> 325 us)
+    k_query_bwd_det<DT, LAYOUT, KT><<<(unsigned)a.L.n_glyphs, DBLOCK, smem, s>>>(a);
     return cudaGetLastError();
 }
 
