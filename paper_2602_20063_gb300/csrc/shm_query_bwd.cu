@@ -70,17 +70,37 @@ __device__ __forceinline__ void paired_reds(float4* dl, const CaptureEmit& e, in
     }
 }
 
-constexpr int BCHUNK = 4;
-constexpr int BBLOCK = 256;
+// Sum of a CTA's per-thread losses, added once: with an addition per warp (9,728 on the fit workload) the
+// rounding of the growing float32 sum alone reached 1e-6 of it and varied from run to run; with one per
+// CTA (152) it stays near 2e-7.
+__device__ __forceinline__ void add_loss(float* loss, float v)
+{
+    __shared__ float s_loss[32];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) s_loss[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        v = threadIdx.x < blockDim.x / 32 ? s_loss[threadIdx.x] : 0.0f;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (threadIdx.x == 0) atomicAdd(loss, v);
+    }
+}
+
+// CTA of the per-query pass, and the most consecutive rounds of 32 queries per warp.  Its warps' queries lie
+// side by side (4,096 of them), so a glyph's records are reused in L1, while all CTAs together still work
+// on few glyphs, whose tables and gradients (836 KB each at N = 64) must stay in L2: fit workload 502 ->
+// 470 us; CTAs of 256 threads 488; a contiguous range of glyphs per CTA 770 to 1,800 (L2 thrashes).
+constexpr int BBLOCK = 1024;
+constexpr int BROUNDS = 4;
 
 template <int DT, int LAYOUT, bool FIT>
-__global__ void __launch_bounds__(BBLOCK, 4) k_query_bwd(BackwardArgs a)
+__global__ void __launch_bounds__(BBLOCK, 1) k_query_bwd(BackwardArgs a, int rounds)
 {
     float loss_acc = 0.0f;
     const int lane = threadIdx.x & 31;
+    const int64_t chunk = 32 * rounds;
     const int64_t warp0 = ((int64_t)blockIdx.x * BBLOCK + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * BBLOCK) >> 5;
-    const int64_t chunk = 32 * BCHUNK;
     const int G = a.L.n_glyphs;
     uint32_t status = 0;
     const float qnan = __int_as_float(0x7fc00000);
@@ -91,7 +111,7 @@ __global__ void __launch_bounds__(BBLOCK, 4) k_query_bwd(BackwardArgs a)
             g = (c0 < __ldg(a.seg)) ? -1 : seg_find_warp(a.seg, G, c0);
         }
 #pragma unroll 1
-        for (int it = 0; it < BCHUNK; ++it) {
+        for (int it = 0; it < rounds; ++it) {
             const int64_t q = c0 + it * 32 + lane;
             if (c0 + it * 32 >= a.Q) break;  // warp-uniform: the paired reductions need every lane
             CaptureEmit sink;
@@ -127,10 +147,7 @@ __global__ void __launch_bounds__(BBLOCK, 4) k_query_bwd(BackwardArgs a)
             paired_reds(reinterpret_cast<float4*>(a.dlut), sink, lane);
         }
     }
-    if (FIT) {
-        for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
-        if ((threadIdx.x & 31) == 0 && a.loss) atomicAdd(a.loss, loss_acc);
-    }
+    if (FIT && a.loss) add_loss(a.loss, loss_acc);
     report_status(a.dev_status, status);
 }
 
@@ -278,10 +295,7 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
         part = next;
     }
     if (SET) zero_through(end.g);
-    if (FIT) {
-        for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
-        if ((tid & 31) == 0 && a.loss) atomicAdd(a.loss, loss_acc);
-    }
+    if (FIT && a.loss) add_loss(a.loss, loss_acc);
     report_status(a.dev_status, status);
 }
 
@@ -314,13 +328,13 @@ static cudaError_t launch_bwd_staged(const BackwardArgs& a, uint32_t table_bytes
 template <int DT, int LAYOUT>
 static cudaError_t launch_bwd_t(const BackwardArgs& a, cudaStream_t s)
 {
-    const int64_t chunks = (a.Q + 32 * BCHUNK - 1) / (32 * BCHUNK);
-    int64_t blocks = (chunks + (BBLOCK / 32) - 1) / (BBLOCK / 32);
-    const int64_t cap = (int64_t)sm_count() * 8;
+    const int64_t cap = sm_count();
+    int64_t rounds = (a.Q + cap * BBLOCK - 1) / (cap * BBLOCK);  // small batches: every SM first
+    if (rounds > BROUNDS) rounds = BROUNDS;
+    int64_t blocks = (a.Q + BBLOCK * rounds - 1) / (BBLOCK * rounds);
     if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    if (a.fit) k_query_bwd<DT, LAYOUT, true><<<(unsigned)blocks, BBLOCK, 0, s>>>(a);
-    else k_query_bwd<DT, LAYOUT, false><<<(unsigned)blocks, BBLOCK, 0, s>>>(a);
+    if (a.fit) k_query_bwd<DT, LAYOUT, true><<<(unsigned)blocks, BBLOCK, 0, s>>>(a, (int)rounds);
+    else k_query_bwd<DT, LAYOUT, false><<<(unsigned)blocks, BBLOCK, 0, s>>>(a, (int)rounds);
     return cudaGetLastError();
 }
 
