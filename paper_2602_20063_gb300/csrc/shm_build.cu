@@ -381,70 +381,45 @@ __device__ float fbm(const Vec3& w, const shm_source& src)
     return src.amplitude * sum;
 }
 
-// value_noise with the lattice values read from a table of the box [x0, x0+nx) x [y0, ...) x
-// [z0, ...) (same corners and interpolation, so the same result).
-__device__ __forceinline__ float value_noise_box(float px, float py, float pz, const float* T, int x0, int y0, int z0,
-                                                 int nx, int ny, int nz)
-{
-    const float fx = floorf(px), fy = floorf(py), fz = floorf(pz);
-    const float wx = quintic(px - fx), wy = quintic(py - fy), wz = quintic(pz - fz);
-    // the corner stays inside the box (the callers' box is padded; the clamps only guard it)
-    const int nxy = nx * ny;
-    const int bx = min(max((int)fx - x0, 0), nx - 2), by = min(max((int)fy - y0, 0), ny - 2);
-    const int bz = min(max((int)fz - z0, 0), nz - 2);
-    const float* b = T + bz * nxy + by * nx + bx;
-    float c[2][2];
-    for (int dz = 0; dz < 2; ++dz)
-        for (int dy = 0; dy < 2; ++dy) {
-            const float* r = b + dz * nxy + dy * nx;
-            const float v0 = r[0], v1 = r[1];
-            c[dz][dy] = v0 + wx * (v1 - v0);
-        }
-    const float e0 = c[0][0] + wy * (c[0][1] - c[0][0]);
-    const float e1 = c[1][0] + wy * (c[1][1] - c[1][0]);
-    return e0 + wz * (e1 - e0);
-}
-
-// value_noise_box at two points at once (.x and .y): the same operations lane by lane (so the same
-// values), the fade and the trilinear interpolation on float2 pairs, the box corners per lane.
 __device__ __forceinline__ float2 quintic2(float2 t)
 {
     return pmul(pmul(pmul(t, t), t), pfma(t, pfma(t, bc(6.0f), bc(-15.0f)), bc(10.0f)));
 }
 
-__device__ __forceinline__ float2 value_noise_box2(float2 px, float2 py, float2 pz, const float* T, int x0, int y0,
-                                                   int z0, int nx, int ny, int nz)
+// value_noise at two points at once (.x and .y): w times the octave's frequency, with the lattice from a
+// table in shared memory: entry = (value, difference to the next value along x), at index
+// ix + nx iy + nxy iz + c (modulo 2^32) for lattice coordinates given as the bits of (floor + FLOOR_MAGIC).
+// w f + 1.5 2^23 rounded down is floor(w f) + 1.5 2^23 exactly for |w f| < 2^22, its low bits are the
+// integer, and neither it nor the fraction w f - floor(w f) rounds the product first; no conversion
+// instruction (16 lanes per clock) is used.  The x interpolation is scalar: an entry's two halves belong to
+// one lane, and pairing them across lanes would cost more moves than it saves.
+constexpr float FLOOR_MAGIC = 12582912.0f;
+constexpr uint32_t FLOOR_MAGIC_BITS = 0x4B400000u;
+
+__device__ __forceinline__ float2 value_noise_lattice2(float2 x, float2 y, float2 z, float freq, const float2* T, uint32_t c,
+                                                       uint32_t nx, uint32_t nxy)
 {
-    const float2 fx = make_float2(floorf(px.x), floorf(px.y)), fy = make_float2(floorf(py.x), floorf(py.y));
-    const float2 fz = make_float2(floorf(pz.x), floorf(pz.y));
-    const float2 wx = quintic2(psub(px, fx)), wy = quintic2(psub(py, fy)), wz = quintic2(psub(pz, fz));
-    const int nxy = nx * ny;
-    const float* b[2];
-#pragma unroll
-    for (int l = 0; l < 2; ++l) {
-        const int bx = min(max((int)(l ? fx.y : fx.x) - x0, 0), nx - 2);
-        const int by = min(max((int)(l ? fy.y : fy.x) - y0, 0), ny - 2);
-        const int bz = min(max((int)(l ? fz.y : fz.x) - z0, 0), nz - 2);
-        b[l] = T + bz * nxy + by * nx + bx;
-    }
-    float2 c[2][2];
-#pragma unroll
-    for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy) {
-            const int o = dz * nxy + dy * nx;
-            const float2 v0 = make_float2(b[0][o], b[1][o]), v1 = make_float2(b[0][o + 1], b[1][o + 1]);
-            c[dz][dy] = pfma(wx, psub(v1, v0), v0);
-        }
-    const float2 e0 = pfma(wy, psub(c[0][1], c[0][0]), c[0][0]);
-    const float2 e1 = pfma(wy, psub(c[1][1], c[1][0]), c[1][0]);
+    const float2 mx = __ffma2_rd(x, bc(freq), bc(FLOOR_MAGIC)), my = __ffma2_rd(y, bc(freq), bc(FLOOR_MAGIC)),
+                 mz = __ffma2_rd(z, bc(freq), bc(FLOOR_MAGIC));
+    const auto fade = [&](float2 v, float2 m) { return quintic2(pfma(v, bc(freq), psub(bc(FLOOR_MAGIC), m))); };
+    const float2 wx = fade(x, mx), wy = fade(y, my), wz = fade(z, mz);
+    const float2* ta = T + (__float_as_uint(mx.x) + nx * __float_as_uint(my.x) + nxy * __float_as_uint(mz.x) + c);
+    const float2* tb = T + (__float_as_uint(mx.y) + nx * __float_as_uint(my.y) + nxy * __float_as_uint(mz.y) + c);
+    const auto row = [&](uint32_t o) {
+        const float2 a = ta[o], b = tb[o];
+        return make_float2(fmaf(wx.x, a.y, a.x), fmaf(wx.y, b.y, b.x));
+    };
+    const float2 c00 = row(0), c01 = row(nx), c10 = row(nxy), c11 = row(nxy + nx);
+    const float2 e0 = pfma(wy, psub(c01, c00), c00), e1 = pfma(wy, psub(c11, c10), c10);
     return pfma(wz, psub(e1, e0), e0);
 }
 
 // ------------------------------------------------------------------------------------------
 // Sampled sources: value tables (k_value_build) and finite-difference records (k_fd_face).
 constexpr int FS = 18, MAX_BUMPS_SMEM = 128;
-constexpr int FBM_CACHE = 4096;  // lattice values of the octaves' boxes per CTA (16 KB)
+constexpr int FBM_T = 48;        // region edge of the fBm bake: 64 / 48 / 32 texels measured 470 / 474 / 590 us at
+                                 // N = 2048, 160 / 154 / 186 at N = 1024 (larger regions miss the cache there)
+constexpr int FBM_CACHE = 5376;  // lattice entries of the octaves' boxes per CTA (42 KB, four CTAs per SM)
 constexpr int FBM_MAX_OCT = 16;  // octaves whose boxes may be cached
 
 // Gaussian bumps of one glyph, staged in shared memory: centre and amplitude as one float4 (a
@@ -578,9 +553,25 @@ constexpr int REGION_T = 64;      // region edge for larger tables: 66^2 floats 
 constexpr int FACE_SPLIT_T = 66;  // uneven pools: N <= 64 faces stay whole, N = 128 faces split 2 x 2
 constexpr int FACE_SPLIT_SMEM = 45 * 1024;
 
-// FBM: the fBm source (its lattice cache is only allocated in that instantiation); otherwise stored
-// samples or Gaussian bumps.
-template <bool FBM, class Map>
+// Records of the region's ti x tj texels from its samples Sf [tj+2][ti+2], by central differences.
+__device__ __forceinline__ void fd_records(const LutView& out, void* data, const GlyphRef& Gr, int f, int i0, int j0, int ti,
+                                           int tj, const float* Sf, float base)
+{
+    const int Si = ti + 2;
+    const uint32_t inv = 0xffffffffu / (uint32_t)ti + 1u;  // e / ti = umulhi(e, inv): e ti < 2^32 (ti = 1: 0)
+    for (int e = threadIdx.x; e < ti * tj; e += 256) {
+        const int lj = ti == 1 ? e : (int)__umulhi(e, inv), li = e - lj * ti;
+        const float* c = Sf + (lj + 1) * Si + (li + 1);  // texel (i0+li, j0+lj) is local sample (li+1, lj+1)
+        float4 v;
+        v.x = c[0] + base;
+        v.y = 0.5f * (c[1] - c[-1]);
+        v.z = 0.5f * (c[Si] - c[-Si]);
+        v.w = 0.25f * ((c[Si + 1] - c[-Si + 1]) - (c[Si - 1] - c[-Si - 1]));
+        store_texel(data, out.dtype, out.layout, Gr, f, j0 + lj, i0 + li, v);
+    }
+}
+
+template <class Map>
 __global__ void __launch_bounds__(256) k_fd_face(LutView out, void* data, shm_source src, int T,
                                                  const __grid_constant__ Map map)
 {
@@ -608,129 +599,7 @@ __global__ void __launch_bounds__(256) k_fd_face(LutView out, void* data, shm_so
     };
     const int S = N + 4;
     float base = 0.0f;
-    if constexpr (FBM) {
-        // fBm over the region with the lattice values in shared memory: the corners an octave of
-        // frequency f needs lie in the box [floor(f wmin), floor(f wmax) + 1] per axis (floor(f w)
-        // is monotone in w), padded by one lattice step on each side; the boxes of all octaves that
-        // fit are hashed once, the others are hashed per sample.  Chart coordinates X, Y of the
-        // region's columns and rows are divided once.
-        __shared__ float cache[FBM_CACHE];
-        __shared__ float s_w[8][6];
-        __shared__ float s_xy[2 * (REGION_T + 2)];
-        __shared__ int s_box[FBM_MAX_OCT][8];  // x0, y0, z0, nx, ny, nz, cache offset, boxed
-        const bool xy_tab = (Si <= REGION_T + 2 && Sj <= REGION_T + 2);  // block-uniform
-        if (xy_tab) {
-            for (int e = tid; e < Si + Sj; e += 256) {
-                const int g2 = (e < Si) ? 2 * (i0 + e) : 2 * (j0 + e - Si);
-                s_xy[e] = (float)(g2 - 3 - N) / (float)N;
-            }
-            __syncthreads();
-        }
-        auto wdir = [&](int li, int lj) {
-            if (!xy_tab) return dir(i0 + li, j0 + lj);
-            const float X = s_xy[li], Y = s_xy[Si + lj];
-            const float ir = rsqrtf(1.0f + X * X + Y * Y);
-            return Vec3{(a.x + X * bb.x + Y * cc.x) * ir, (a.y + X * bb.y + Y * cc.y) * ir,
-                        (a.z + X * bb.z + Y * cc.z) * ir};
-        };
-        float lo[3] = {3.0f, 3.0f, 3.0f}, hi[3] = {-3.0f, -3.0f, -3.0f};
-        for (int e = tid; e < Si * Sj; e += 256) {
-            const Vec3 w = wdir(e % Si, e / Si);
-            lo[0] = fminf(lo[0], w.x); lo[1] = fminf(lo[1], w.y); lo[2] = fminf(lo[2], w.z);
-            hi[0] = fmaxf(hi[0], w.x); hi[1] = fmaxf(hi[1], w.y); hi[2] = fmaxf(hi[2], w.z);
-        }
-        for (int o = 16; o > 0; o >>= 1)
-            for (int a3 = 0; a3 < 3; ++a3) {
-                lo[a3] = fminf(lo[a3], __shfl_xor_sync(0xffffffffu, lo[a3], o));
-                hi[a3] = fmaxf(hi[a3], __shfl_xor_sync(0xffffffffu, hi[a3], o));
-            }
-        if ((tid & 31) == 0)
-            for (int a3 = 0; a3 < 3; ++a3) { s_w[tid >> 5][a3] = lo[a3]; s_w[tid >> 5][3 + a3] = hi[a3]; }
-        __syncthreads();
-        const int octaves = min(src.octaves, FBM_MAX_OCT);
-        if (tid == 0) {
-            for (int a3 = 0; a3 < 3; ++a3) {
-                lo[a3] = s_w[0][a3];
-                hi[a3] = s_w[0][3 + a3];
-                for (int wp = 1; wp < 8; ++wp) { lo[a3] = fminf(lo[a3], s_w[wp][a3]); hi[a3] = fmaxf(hi[a3], s_w[wp][3 + a3]); }
-            }
-            float freq = src.base_freq;
-            int used = 0;
-            for (int o = 0; o < octaves; ++o) {
-                int* bx = s_box[o];
-                bx[0] = (int)floorf(lo[0] * freq) - 1;
-                bx[1] = (int)floorf(lo[1] * freq) - 1;
-                bx[2] = (int)floorf(lo[2] * freq) - 1;
-                bx[3] = (int)floorf(hi[0] * freq) - bx[0] + 3;
-                bx[4] = (int)floorf(hi[1] * freq) - bx[1] + 3;
-                bx[5] = (int)floorf(hi[2] * freq) - bx[2] + 3;
-                const int64_t n = (int64_t)bx[3] * bx[4] * bx[5];
-                bx[6] = used;
-                bx[7] = (used + n <= FBM_CACHE) ? 1 : 0;
-                if (bx[7]) used += (int)n;
-                freq *= src.lacunarity;
-            }
-        }
-        __syncthreads();
-        for (int o = 0; o < octaves; ++o) {
-            const int* bx = s_box[o];
-            if (!bx[7]) continue;  // block-uniform
-            const int nx = bx[3], ny = bx[4], n = nx * ny * bx[5];
-            const uint32_t k0 = __ldg(src.keys + 3 * o), k1 = __ldg(src.keys + 3 * o + 1), k2 = __ldg(src.keys + 3 * o + 2);
-            for (int idx = tid; idx < n; idx += 256) {
-                const int ix = idx % nx, iy = (idx / nx) % ny, iz = idx / (nx * ny);
-                cache[bx[6] + idx] = lattice_value(bx[0] + ix, bx[1] + iy, bx[2] + iz, k0, k1, k2);
-            }
-        }
-        __syncthreads();
-        // two samples per thread at a time (e and e + 256), the last odd one alone: per octave the
-        // box parameters are read once for both and the cached lattice is interpolated on pairs
-        for (int e = tid; e < Si * Sj; e += 512) {
-            const int e2 = e + 256;
-            if (e2 < Si * Sj) {
-                const Vec3 wa = wdir(e % Si, e / Si), wb = wdir(e2 % Si, e2 / Si);
-                float2 sum = make_float2(0.0f, 0.0f);
-                float freq = src.base_freq, amp = 1.0f;
-                for (int o = 0; o < src.octaves; ++o) {
-                    const float2 px = pmul(make_float2(wa.x, wb.x), bc(freq));
-                    const float2 py = pmul(make_float2(wa.y, wb.y), bc(freq));
-                    const float2 pz = pmul(make_float2(wa.z, wb.z), bc(freq));
-                    float2 v;
-                    if (o < FBM_MAX_OCT && s_box[o][7]) {
-                        const int* bx = s_box[o];
-                        v = value_noise_box2(px, py, pz, cache + bx[6], bx[0], bx[1], bx[2], bx[3], bx[4], bx[5]);
-                    } else {
-                        const uint32_t* key = src.keys + 3 * o;
-                        const uint32_t k0 = __ldg(key), k1 = __ldg(key + 1), k2 = __ldg(key + 2);
-                        v = make_float2(value_noise(px.x, py.x, pz.x, k0, k1, k2), value_noise(px.y, py.y, pz.y, k0, k1, k2));
-                    }
-                    sum = pfma(bc(amp), v, sum);
-                    freq *= src.lacunarity;
-                    amp *= src.gain;
-                }
-                Sf[e] = src.amplitude * sum.x;
-                Sf[e2] = src.amplitude * sum.y;
-            } else {
-                const Vec3 w = wdir(e % Si, e / Si);
-                float sum = 0.0f, freq = src.base_freq, amp = 1.0f;
-                for (int o = 0; o < src.octaves; ++o) {
-                    const float px = w.x * freq, py = w.y * freq, pz = w.z * freq;
-                    float v;
-                    if (o < FBM_MAX_OCT && s_box[o][7]) {
-                        const int* bx = s_box[o];
-                        v = value_noise_box(px, py, pz, cache + bx[6], bx[0], bx[1], bx[2], bx[3], bx[4], bx[5]);
-                    } else {
-                        const uint32_t* key = src.keys + 3 * o;
-                        v = value_noise(px, py, pz, __ldg(key), __ldg(key + 1), __ldg(key + 2));
-                    }
-                    sum = fmaf(amp, v, sum);
-                    freq *= src.lacunarity;
-                    amp *= src.gain;
-                }
-                Sf[e] = src.amplitude * sum;
-            }
-        }
-    } else {
+    {
         __shared__ BumpSmem bump;
         for (int e = tid; e < Si * Sj; e += 256) {
             const int ii = i0 + e % Si, jj = j0 + e / Si;
@@ -763,16 +632,150 @@ __global__ void __launch_bounds__(256) k_fd_face(LutView out, void* data, shm_so
         }
     }
     __syncthreads();
-    for (int e = tid; e < ti * tj; e += 256) {
-        const int li = e % ti, lj = e / ti;
-        const float* c = Sf + (lj + 1) * Si + (li + 1);  // texel (i0+li, j0+lj) is local sample (li+1, lj+1)
-        float4 v;
-        v.x = c[0] + base;
-        v.y = 0.5f * (c[1] - c[-1]);
-        v.z = 0.5f * (c[Si] - c[-Si]);
-        v.w = 0.25f * ((c[Si + 1] - c[-Si + 1]) - (c[Si - 1] - c[-Si - 1]));
-        store_texel(data, out.dtype, out.layout, Gr, f, j0 + lj, i0 + li, v);
+    fd_records(out, data, Gr, f, i0, j0, ti, tj, Sf, base);
+}
+
+// fBm tables, one CTA per (glyph, face, region of up to T x T texels): the octaves' lattice values are hashed
+// once per region into shared memory, then every margin sample sums its octaves, two samples per
+// thread on float2 pairs.  An octave of frequency f needs the lattice points of [floor(f wmin),
+// floor(f wmax) + 1] per axis; wmin and wmax of the region's directions follow from its chart rectangle
+// (each component of (1, X, Y)/rho is monotone or has its extreme at the smallest |X| and |Y|), widened by
+// 1e-6 against rounding.  Octaves whose box does not fit the cache are hashed per sample.
+// Bound: FP32 issue (about 70 instructions per pair of samples and octave; 73 % of the issue slots).  N = 2048,
+// 8 octaves: 708 -> 470 us, the same values; before, boxes padded by a lattice step on each side left the
+// last octave of 60 % of the regions to per-sample hashing, floor and integer conversions took 12 of the
+// slow conversion operations per pair, and corner indices were clamped.
+template <class Map>
+__global__ void __launch_bounds__(256, 4) k_fbm_face(LutView out, void* data, shm_source src, int T,
+                                                     const __grid_constant__ Map map)
+{
+    extern __shared__ float Sf[];  // [T+2][T+2]
+    __shared__ float2 cache[FBM_CACHE];
+    __shared__ float s_xy[2 * (FBM_T + 2)];
+    __shared__ uint4 s_oct[FBM_MAX_OCT];  // index constant, nx, nxy, boxed
+    __shared__ uint2 s_inv[FBM_MAX_OCT];  // idx / nx = umulhi(idx, .x), idx / nxy = umulhi(idx, .y): idx nxy < 2^32
+    __shared__ int s_box[FBM_MAX_OCT + 1][4];  // x0, y0, z0 and first cache entry (the last row: entries used)
+    int region;
+    const int g = map_block(map, region), f = blockIdx.y;
+    const GlyphRef Gr = glyph_ref(out, g);
+    const int N = Gr.N, P = N + 2;
+    const int nr = (P + T - 1) / T;
+    if (region >= nr * nr) return;
+    const int i0 = (region % nr) * T, j0 = (region / nr) * T;  // first texel of the region
+    const int ti = min(T, P - i0), tj = min(T, P - j0);      // texels in the region
+    const int Si = ti + 2, Sj = tj + 2;                       // samples: texels i0-1 .. i0+ti
+    const int tid = threadIdx.x;
+    const int k = f >> 1;
+    const float sg = (f & 1) ? -1.0f : 1.0f;
+    const Vec3 a = axis_vec(k, sg), bb = axis_vec((k + 1) % 3, 1.0f), cc = axis_vec((k + 2) % 3, 1.0f);
+    // chart coordinates 2u - 1 of the region's sample columns and rows, divided once
+    for (int e = tid; e < Si + Sj; e += 256) {
+        const int g2 = (e < Si) ? 2 * (i0 + e) : 2 * (j0 + e - Si);
+        s_xy[e] = (float)(g2 - 3 - N) / (float)N;
     }
+    __syncthreads();
+    const auto wdir = [&](int li, int lj) {
+        const float X = s_xy[li], Y = s_xy[Si + lj];
+        const float ir = rsqrtf(1.0f + X * X + Y * Y);
+        return Vec3{(a.x + X * bb.x + Y * cc.x) * ir, (a.y + X * bb.y + Y * cc.y) * ir,
+                    (a.z + X * bb.z + Y * cc.z) * ir};
+    };
+    const int octaves = min(src.octaves, FBM_MAX_OCT);
+    if (tid < 32) {
+        // warp 0: lane o boxes octave o
+        const float Xa = s_xy[0], Xb = s_xy[Si - 1], Ya = s_xy[Si], Yb = s_xy[Si + Sj - 1];
+        const auto lo_abs = [](float u, float v) { return u <= 0.0f && v >= 0.0f ? 0.0f : fminf(fabsf(u), fabsf(v)); };
+        const auto hi_abs = [](float u, float v) { return fmaxf(fabsf(u), fabsf(v)); };
+        const float Xn = lo_abs(Xa, Xb), Xx = hi_abs(Xa, Xb), Yn = lo_abs(Ya, Yb), Yx = hi_abs(Ya, Yb);
+        const auto unit = [](float v, float x, float y) { return v * rsqrtf(1.0f + x * x + y * y); };
+        const float kmin = unit(1.0f, Xx, Yx), kmax = unit(1.0f, Xn, Yn);
+        const float bmin = unit(Xa, Xa, Xa < 0.0f ? Yn : Yx), bmax = unit(Xb, Xb, Xb > 0.0f ? Yn : Yx);
+        const float cmin = unit(Ya, Ya < 0.0f ? Xn : Xx, Ya), cmax = unit(Yb, Yb > 0.0f ? Xn : Xx, Yb);
+        float lo[3], hi[3];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            const bool isk = ax == k, isb = ax == (k + 1) % 3;
+            lo[ax] = (isk ? (sg > 0.0f ? kmin : -kmax) : (isb ? bmin : cmin)) - 1e-6f;
+            hi[ax] = (isk ? (sg > 0.0f ? kmax : -kmin) : (isb ? bmax : cmax)) + 1e-6f;
+        }
+        float freq = src.base_freq;
+        for (int o = 0; o < tid && o < octaves; ++o) freq *= src.lacunarity;
+        int x0[3] = {0, 0, 0}, n[3] = {0, 0, 0};
+        int64_t need = (int64_t)FBM_CACHE + 1;
+        if (tid < octaves && freq > 0.0f && freq <= 1.0e5f) {
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) {
+                x0[ax] = (int)floorf(lo[ax] * freq);
+                n[ax] = (int)floorf(hi[ax] * freq) - x0[ax] + 2;
+            }
+            need = (int64_t)n[0] * n[1] * n[2];
+        }
+        const int want = need <= FBM_CACHE ? (int)need : FBM_CACHE + 1;
+        int used = 0, mine = 0;
+        bool boxed = false;
+        for (int o = 0; o < octaves; ++o) {  // in octave order, each one that still fits
+            const int w = __shfl_sync(0xffffffffu, want, o);
+            if (tid == o) mine = used;
+            if (used + w <= FBM_CACHE) {
+                if (tid == o) boxed = true;
+                used += w;
+            }
+        }
+        if (tid < octaves) {
+            const uint32_t nx = n[0], nxy = (uint32_t)n[0] * (uint32_t)n[1];
+            s_oct[tid] = make_uint4((uint32_t)mine - ((uint32_t)x0[0] + FLOOR_MAGIC_BITS) -
+                                        nx * ((uint32_t)x0[1] + FLOOR_MAGIC_BITS) - nxy * ((uint32_t)x0[2] + FLOOR_MAGIC_BITS),
+                                    nx, nxy, boxed ? 1u : 0u);
+            s_inv[tid] = make_uint2(0xffffffffu / max(nx, 2u) + 1u, 0xffffffffu / max(nxy, 2u) + 1u);
+            s_box[tid][0] = x0[0]; s_box[tid][1] = x0[1]; s_box[tid][2] = x0[2];
+            s_box[tid][3] = mine;
+        }
+        if (tid == 0) s_box[octaves][3] = used;
+    }
+    __syncthreads();
+    const int used = s_box[octaves][3];
+    for (int e = tid, o = 0; e < used; e += 256) {
+        while (s_box[o + 1][3] <= e || s_oct[o].w == 0) ++o;  // e < used: ends at the boxed octave that holds e
+        const uint4 oc = s_oct[o];
+        const uint32_t idx = e - s_box[o][3], iz = __umulhi(idx, s_inv[o].y), r = idx - iz * oc.z, iy = __umulhi(r, s_inv[o].x),
+                       ix = r - iy * oc.y;
+        cache[e].x = lattice_value(s_box[o][0] + (int)ix, s_box[o][1] + (int)iy, s_box[o][2] + (int)iz,
+                                   __ldg(src.keys + 3 * o), __ldg(src.keys + 3 * o + 1), __ldg(src.keys + 3 * o + 2));
+    }
+    __syncthreads();
+    // differences along x (the last entry of a row is never a cell's first corner)
+    for (int e = tid; e < used; e += 256) cache[e].y = (e + 1 < used ? cache[e + 1].x : 0.0f) - cache[e].x;
+    __syncthreads();
+    // samples e and e + 256 together (an odd last one twice): per octave one lattice read per corner row
+    const int S = Si * Sj;
+    const uint32_t inv = 0xffffffffu / (uint32_t)Si + 1u;  // e / Si = umulhi(e, inv): e Si < 2^32
+    for (int e = tid; e < S; e += 512) {
+        const int e2 = min(e + 256, S - 1);
+        const int ja = __umulhi(e, inv), jb = __umulhi(e2, inv);
+        const Vec3 wa = wdir(e - ja * Si, ja), wb = wdir(e2 - jb * Si, jb);
+        const float2 wx = make_float2(wa.x, wb.x), wy = make_float2(wa.y, wb.y), wz = make_float2(wa.z, wb.z);
+        float2 sum = bc(0.0f);
+        float freq = src.base_freq, amp = 1.0f;
+        for (int o = 0; o < src.octaves; ++o) {
+            const uint4 oc = o < FBM_MAX_OCT ? s_oct[o] : make_uint4(0, 0, 0, 0);
+            float2 v;
+            if (oc.w) {
+                v = value_noise_lattice2(wx, wy, wz, freq, cache, oc.x, oc.y, oc.z);
+            } else {
+                const uint32_t* key = src.keys + 3 * o;
+                const uint32_t k0 = __ldg(key), k1 = __ldg(key + 1), k2 = __ldg(key + 2);
+                v = make_float2(value_noise(wx.x * freq, wy.x * freq, wz.x * freq, k0, k1, k2),
+                                value_noise(wx.y * freq, wy.y * freq, wz.y * freq, k0, k1, k2));
+            }
+            sum = pfma(bc(amp), v, sum);
+            freq *= src.lacunarity;
+            amp *= src.gain;
+        }
+        Sf[e] = src.amplitude * sum.x;
+        if (e + 256 < S) Sf[e2] = src.amplitude * sum.y;
+    }
+    __syncthreads();
+    fd_records(out, data, Gr, f, i0, j0, ti, tj, Sf, 0.0f);
 }
 
 static int64_t value_tiles(int N)
@@ -787,29 +790,30 @@ cudaError_t launch_fd_build(const LutView& out, void* data, const shm_source& sr
         return for_each_glyph_chunk(sz, value_tiles, [&](unsigned bx, unsigned bz, const auto& map) {
             k_value_build<std::decay_t<decltype(map)>><<<dim3(bx, 6, bz), 256, 0, s>>>(out, data, src, map);
         });
-    {
-        int T = (sz.max_N <= FACE_N_MAX) ? sz.max_N + 2 : REGION_T;
+    int T = (sz.max_N <= FACE_N_MAX) ? sz.max_N + 2 : REGION_T;
+    const bool fbm = src.kind == SHM_SRC_FBM;
+    if (fbm) {
+        T = sz.max_N + 2 < FBM_T ? sz.max_N + 2 : FBM_T;
+    } else {
         if (sz.N_uniform == 0 && T > FACE_SPLIT_T) T = FACE_SPLIT_T;
         if (sz.N_uniform > 0 && T <= FACE_N_MAX + 2 && (T + 2) * (T + 2) * (int)sizeof(float) > FACE_SPLIT_SMEM)
             T = (T + 1) / 2;
-        const int smem = (T + 2) * (T + 2) * (int)sizeof(float);
-        const int mi = sz.N_uniform > 0 ? 0 : 1, fi = src.kind == SHM_SRC_FBM ? 1 : 0;
-        {
-            const void* fn = fi ? (mi == 0 ? (const void*)k_fd_face<true, UniformMap> : (const void*)k_fd_face<true, TileMap>)
-                                : (mi == 0 ? (const void*)k_fd_face<false, UniformMap> : (const void*)k_fd_face<false, TileMap>);
-            cudaError_t e = ensure_dynamic_smem(fn, smem);
-            if (e != cudaSuccess) return e;
-        }
-        auto regions = [T](int N) {
-            const int64_t r = (N + 2 + T - 1) / T;
-            return r * r;
-        };
-        return for_each_glyph_chunk(sz, regions, [&](unsigned bx, unsigned bz, const auto& map) {
-            using M = std::decay_t<decltype(map)>;
-            if (fi) k_fd_face<true, M><<<dim3(bx, 6, bz), 256, smem, s>>>(out, data, src, T, map);
-            else k_fd_face<false, M><<<dim3(bx, 6, bz), 256, smem, s>>>(out, data, src, T, map);
-        });
     }
+    const int smem = (T + 2) * (T + 2) * (int)sizeof(float);
+    const bool uniform = sz.N_uniform > 0;
+    const void* fn = fbm ? (uniform ? (const void*)k_fbm_face<UniformMap> : (const void*)k_fbm_face<TileMap>)
+                         : (uniform ? (const void*)k_fd_face<UniformMap> : (const void*)k_fd_face<TileMap>);
+    const cudaError_t e = ensure_dynamic_smem(fn, smem);
+    if (e != cudaSuccess) return e;
+    auto regions = [T](int N) {
+        const int64_t r = (N + 2 + T - 1) / T;
+        return r * r;
+    };
+    return for_each_glyph_chunk(sz, regions, [&](unsigned bx, unsigned bz, const auto& map) {
+        using M = std::decay_t<decltype(map)>;
+        if (fbm) k_fbm_face<M><<<dim3(bx, 6, bz), 256, smem, s>>>(out, data, src, T, map);
+        else k_fd_face<M><<<dim3(bx, 6, bz), 256, smem, s>>>(out, data, src, T, map);
+    });
 }
 
 // ------------------------------------------------------------------------------------------
