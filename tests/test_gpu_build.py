@@ -338,3 +338,24 @@ def test_sh_eval_direct(S):
     Rr, Gr, Nr = O.sh_eval(L, c.astype(np.float64), dirs, glyph=glyph)
     out = {"R": R, "grad": grad, "normal": normal}
     check_query(out, {"R": Rr, "grad": Gr, "normal": Nr})
+
+
+@pytest.mark.parametrize("octaves,base", [(0, 2.0), (3, 2.0), (8, 2.0), (18, 1.7), (6, -2.0), (2, 3.0e5)])
+@pytest.mark.parametrize("N", [1, 3, 46, 47, 93, 110])
+def test_fbm_regions_match_sampled_values(S, N, octaves, base):
+    """fBm records (regions of up to 48 texels with cached lattice boxes, octaves whose box does not fit or
+    that are past the cached ones, one-texel remainders) against central differences of the fBm value table, whose
+    entries are hashed sample by sample: the product's rounding of one octave is at most 2^-24 f |slope|, the
+    slope of the fade times the lattice difference at most 4, and f falls with the octave as its gain."""
+    keys = torch.from_numpy(I.fbm_keys(7, 18).view(np.int32)).cuda()
+    src = S.Source(kind=S.SHM_SRC_FBM, octaves=octaves, keys=keys, base_freq=base, amplitude=0.5)
+    lut, val = S.alloc_lut(1, N), S.alloc_lut(1, N, layout=S.SHM_LAYOUT_VALUE)
+    S.build_lut(lut, src)
+    S.build_lut(val, src)
+    ref = S.alloc_lut(1, N)
+    S.build_lut(ref, S.Source(kind=S.SHM_SRC_SAMPLES, samples=val.data,
+                              sample_offset=torch.zeros(1, dtype=torch.int64, device="cuda")))
+    tol = 0.5 * (octaves * abs(base) * 3 * 4 * 2.0 ** -24 + 16 * 2.0 ** -24)
+    assert (lut.data - ref.data).abs().max().item() <= tol
+    if base == 3.0e5:
+        assert torch.equal(lut.data, ref.data)

@@ -163,3 +163,24 @@ def test_planet_full_resolution(S):
     ref = O.mip_consistent(f64, r0=1.0)
     got = coarse.data.double().cpu().numpy().reshape(ref.shape)
     _compare(got, ref, np.abs(f64[..., 0]).max())
+
+
+def test_tile_sizes_agree(S):
+    """A pool with one large glyph takes the large tiles for every glyph: its small glyphs' levels equal the
+    small-tile levels of a pool without it bit for bit, and the large glyph's interior records are the means
+    and central differences of its stored values."""
+    Ns = [1040, 24, 10, 2]
+    g = torch.Generator(device="cuda").manual_seed(3)
+    big = S.alloc_lut(4, Ns, r0=np.array([1.0, 0.5, 0.0, -0.25], np.float32))
+    big.data.copy_(torch.randn(big.data.shape, generator=g, device="cuda"))
+    small = S.alloc_lut(3, Ns[1:], r0=np.array([0.5, 0.0, -0.25], np.float32))
+    small.data.copy_(big.data[big.data.numel() - small.data.numel():])
+    a, b = S.build_mip(big, S.mip_like(big)), S.build_mip(small, S.mip_like(small))
+    assert torch.equal(a.data[a.data.numel() - b.data.numel():], b.data)
+    f = big.data[:6 * 1042 * 1042 * 4].view(6, 1042, 1042, 4)[..., 0].double()
+    c = a.data[:6 * 522 * 522 * 4].view(6, 522, 522, 4).double()
+    v = (f[:, 1:-1:2, 1:-1:2] + f[:, 1:-1:2, 2::2] + f[:, 2::2, 1:-1:2] + f[:, 2::2, 2::2]) / 4
+    tol = 4 * 2.0 ** -24 * float(f.abs().max())
+    assert (c[:, 1:-1, 1:-1, 0] - v).abs().max() <= tol
+    assert (c[:, 2:-2, 2:-2, 1] - (v[:, 1:-1, 2:] - v[:, 1:-1, :-2]) / 2).abs().max() <= 2 * tol
+    assert (c[:, 2:-2, 2:-2, 2] - (v[:, 2:, 1:-1] - v[:, :-2, 1:-1]) / 2).abs().max() <= 2 * tol
