@@ -601,8 +601,9 @@ __global__ void __launch_bounds__(256) k_fd_face(LutView out, void* data, shm_so
     float base = 0.0f;
     {
         __shared__ BumpSmem bump;
+        const uint32_t inv = 0xffffffffu / (uint32_t)Si + 1u;  // e / Si = umulhi(e, inv): e Si < 2^32
         for (int e = tid; e < Si * Sj; e += 256) {
-            const int ii = i0 + e % Si, jj = j0 + e / Si;
+            const int je = __umulhi(e, inv), ii = i0 + e - je * Si, jj = j0 + je;
             float v = 0.0f;
             if (src.kind == SHM_SRC_SAMPLES)
                 v = __ldg(src.samples + __ldg(src.sample_offset + g) + ((int64_t)f * S + jj) * S + ii) - Gr.r0;
@@ -620,12 +621,14 @@ __global__ void __launch_bounds__(256) k_fd_face(LutView out, void* data, shm_so
                 for (int e = tid; e < Si * Sj; e += 512) {
                     const int e2 = e + 256;
                     if (e2 < Si * Sj) {
-                        const float2 v = bump_sum2(bump, nb, dir(i0 + e % Si, j0 + e / Si), dir(i0 + e2 % Si, j0 + e2 / Si),
+                        const int ja = __umulhi(e, inv), jb = __umulhi(e2, inv);
+                        const float2 v = bump_sum2(bump, nb, dir(i0 + e - ja * Si, j0 + ja), dir(i0 + e2 - jb * Si, j0 + jb),
                                                    make_float2(Sf[e], Sf[e2]));
                         Sf[e] = v.x;
                         Sf[e2] = v.y;
                     } else {
-                        Sf[e] = bump_sum(bump, nb, dir(i0 + e % Si, j0 + e / Si), Sf[e]);
+                        const int ja = __umulhi(e, inv);
+                        Sf[e] = bump_sum(bump, nb, dir(i0 + e - ja * Si, j0 + ja), Sf[e]);
                     }
                 }
             }
@@ -911,52 +914,69 @@ cudaError_t launch_pack(const LutView& src, const LutView& dst, void* dst_data, 
 // ------------------------------------------------------------------------------------------
 // Bounds: per cell, |r| <= max|r0 + r_ab| + (max|r_u h| + max|r_v h|)/4 + max|r_uv h^2|/16 over the
 // cell's four corners (value weights are >= 0 and sum to 1; sum_a |H^d_a| = s(1-s) <= 1/4).
-constexpr int BOUNDS_PER_BLOCK = 2048;
+//
+// A warp walks a strip of 31 cell columns down up to BOUNDS_ROWS cell rows of a face: per row it loads 32
+// adjacent records once (512 contiguous bytes f32), the right-hand corners come from the next lane and the
+// upper ones from the row before, so each record is read 1.07 times instead of four and no cell index
+// is divided; eight rows are in flight per warp (one at a time: 100 us).  Bound: DRAM (the table once).
+// 512 bump objects, 280 MB: 62 -> 47 us.
+constexpr int BOUNDS_ROWS = 32, BOUNDS_COLS = 31, BOUNDS_WARPS = 8, BOUNDS_BATCH = 8;
 
+struct BoundsUnits {
+    int strips, chunks;
+    __host__ __device__ explicit BoundsUnits(int N)
+        : strips((N + 1 + BOUNDS_COLS - 1) / BOUNDS_COLS), chunks((N + 1 + BOUNDS_ROWS - 1) / BOUNDS_ROWS) {}
+    __host__ __device__ int64_t count() const { return 6LL * strips * chunks; }
+};
+
+// |r0 + r|, |r_u h|, |r_v h|, |r_uv h^2| of texel (i, j), zero beyond the face and for NaN.
 template <int DT, int LAYOUT>
-__device__ __forceinline__ float cell_bound(const LutView& L, const GlyphRef& G, int f, int i, int j)
+__device__ __forceinline__ float4 abs_texel(const LutView& L, const GlyphRef& G, int f, int j, int i)
 {
-    const Corners cr = fetch_corners<DT, LAYOUT>(L.data, G, f, i, j);
-    const float4 v[4] = {cr.c00, cr.c10, cr.c01, cr.c11};
-    float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        m0 = fmaxf(m0, fabsf(G.r0 + v[k].x));
-        m1 = fmaxf(m1, fabsf(v[k].y));
-        m2 = fmaxf(m2, fabsf(v[k].z));
-        m3 = fmaxf(m3, fabsf(v[k].w));
-    }
-    return m0 + 0.25f * (m1 + m2) + 0.0625f * m3;
+    if (i > G.N + 1) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 v = load_texel(L.data, DT, LAYOUT, G, f, j, i);
+    return make_float4(fmaxf(fabsf(G.r0 + v.x), 0.f), fmaxf(fabsf(v.y), 0.f), fmaxf(fabsf(v.z), 0.f), fmaxf(fabsf(v.w), 0.f));
 }
 
 template <int DT, int LAYOUT, class Map>
-__global__ void __launch_bounds__(256) k_bounds(LutView L, float* rmax, const __grid_constant__ Map map)
+__global__ void __launch_bounds__(32 * BOUNDS_WARPS) k_bounds(LutView L, float* rmax, const __grid_constant__ Map map)
 {
-    __shared__ float warp_best[8];
+    __shared__ float warp_best[BOUNDS_WARPS];
     int blk;
     const int g = map_block(map, blk);
     const GlyphRef G = glyph_ref(L, g);
-    const int N = G.N, P = N + 1;
-    const int64_t ncell = 6LL * P * P;
-    const int64_t c_end = min(ncell, (int64_t)(blk + 1) * BOUNDS_PER_BLOCK);
+    const int N = G.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const BoundsUnits U(N);
+    const int64_t unit = (int64_t)blk * BOUNDS_WARPS + warp;
     float best = 0.0f;
-    if (ncell <= 0x7fffffff) {  // 32-bit cell arithmetic (N < 18,900)
-        const uint32_t PP = (uint32_t)P * (uint32_t)P;
-        for (uint32_t c = (uint32_t)blk * BOUNDS_PER_BLOCK + threadIdx.x; c < (uint32_t)c_end; c += blockDim.x) {
-            const uint32_t f = c / PP, rem = c - f * PP, j = rem / (uint32_t)P, i = rem - j * (uint32_t)P;
-            best = fmaxf(best, cell_bound<DT, LAYOUT>(L, G, (int)f, (int)i, (int)j));
-        }
-    } else {
-        for (int64_t c = (int64_t)blk * BOUNDS_PER_BLOCK + threadIdx.x; c < c_end; c += blockDim.x) {
-            const int f = (int)(c / ((int64_t)P * P)), rem = (int)(c % ((int64_t)P * P)), j = rem / P, i = rem % P;
-            best = fmaxf(best, cell_bound<DT, LAYOUT>(L, G, f, i, j));
+    if (unit < U.count()) {  // warp-uniform
+        const int strip = (int)(unit % U.strips), rest = (int)(unit / U.strips);
+        const int f = rest / U.chunks, j0 = (rest % U.chunks) * BOUNDS_ROWS, j1 = min(N + 1, j0 + BOUNDS_ROWS);
+        const int i = strip * BOUNDS_COLS + lane;
+        const bool cell = lane < BOUNDS_COLS && i <= N;
+        const auto row = [&](const float4& c) {  // maxima over texels (i, j), (i + 1, j)
+            return make_float4(fmaxf(c.x, __shfl_down_sync(0xffffffffu, c.x, 1)), fmaxf(c.y, __shfl_down_sync(0xffffffffu, c.y, 1)),
+                               fmaxf(c.z, __shfl_down_sync(0xffffffffu, c.z, 1)), fmaxf(c.w, __shfl_down_sync(0xffffffffu, c.w, 1)));
+        };
+        float4 up = row(abs_texel<DT, LAYOUT>(L, G, f, j0, i));
+        for (int j = j0; j < j1; j += BOUNDS_BATCH) {  // texel rows j + 1 .. j + BOUNDS_BATCH, loaded together
+            float4 v[BOUNDS_BATCH];
+#pragma unroll
+            for (int r = 0; r < BOUNDS_BATCH; ++r) v[r] = abs_texel<DT, LAYOUT>(L, G, f, min(j + r, j1 - 1) + 1, i);
+#pragma unroll
+            for (int r = 0; r < BOUNDS_BATCH; ++r) {
+                const float4 m = row(v[r]);
+                if (cell && j + r < j1)
+                    best = fmaxf(best, fmaxf(up.x, m.x) + 0.25f * (fmaxf(up.y, m.y) + fmaxf(up.z, m.z)) + 0.0625f * fmaxf(up.w, m.w));
+                up = m;
+            }
         }
     }
     for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if ((threadIdx.x & 31) == 0) warp_best[threadIdx.x >> 5] = best;
+    if (lane == 0) warp_best[warp] = best;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) best = fmaxf(best, warp_best[w]);
+        for (int w = 1; w < BOUNDS_WARPS; ++w) best = fmaxf(best, warp_best[w]);
         // non-negative floats order like their bit patterns
         atomicMax(reinterpret_cast<int*>(rmax + g), __float_as_int(best));
     }
@@ -966,18 +986,19 @@ cudaError_t launch_bounds(const LutView& L, float* rmax, const Sizes& sz, cudaSt
 {
     cudaError_t e = cudaMemsetAsync(rmax, 0, sizeof(float) * (size_t)L.n_glyphs, s);
     if (e != cudaSuccess) return e;
-    auto blocks = [](int N) { return (6LL * (N + 1) * (N + 1) + BOUNDS_PER_BLOCK - 1) / BOUNDS_PER_BLOCK; };
+    auto blocks = [](int N) { return (BoundsUnits(N).count() + BOUNDS_WARPS - 1) / BOUNDS_WARPS; };
     return for_each_glyph_chunk(sz, blocks, [&](unsigned bx, unsigned bz, const auto& map) {
         using M = std::decay_t<decltype(map)>;
         const dim3 grid(bx, 1, bz);
+        constexpr int T = 32 * BOUNDS_WARPS;
         if (L.layout == SHM_LAYOUT_TEXEL) {
-            if (L.dtype == SHM_F32) k_bounds<SHM_F32, SHM_LAYOUT_TEXEL, M><<<grid, 256, 0, s>>>(L, rmax, map);
-            else if (L.dtype == SHM_F16) k_bounds<SHM_F16, SHM_LAYOUT_TEXEL, M><<<grid, 256, 0, s>>>(L, rmax, map);
-            else k_bounds<SHM_BF16, SHM_LAYOUT_TEXEL, M><<<grid, 256, 0, s>>>(L, rmax, map);
+            if (L.dtype == SHM_F32) k_bounds<SHM_F32, SHM_LAYOUT_TEXEL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            else if (L.dtype == SHM_F16) k_bounds<SHM_F16, SHM_LAYOUT_TEXEL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            else k_bounds<SHM_BF16, SHM_LAYOUT_TEXEL, M><<<grid, T, 0, s>>>(L, rmax, map);
         } else {
-            if (L.dtype == SHM_F32) k_bounds<SHM_F32, SHM_LAYOUT_CELL, M><<<grid, 256, 0, s>>>(L, rmax, map);
-            else if (L.dtype == SHM_F16) k_bounds<SHM_F16, SHM_LAYOUT_CELL, M><<<grid, 256, 0, s>>>(L, rmax, map);
-            else k_bounds<SHM_BF16, SHM_LAYOUT_CELL, M><<<grid, 256, 0, s>>>(L, rmax, map);
+            if (L.dtype == SHM_F32) k_bounds<SHM_F32, SHM_LAYOUT_CELL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            else if (L.dtype == SHM_F16) k_bounds<SHM_F16, SHM_LAYOUT_CELL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            else k_bounds<SHM_BF16, SHM_LAYOUT_CELL, M><<<grid, T, 0, s>>>(L, rmax, map);
         }
     });
 }
