@@ -32,8 +32,8 @@ constexpr int SSHAPES[N_SSHAPES] = {512, 1024, 256};
 
 // STD: the usual output set (R, gradient and normal; no chart derivatives, no cell indices), so the
 // per-query output checks drop out of the loop.
-template <int DT, int SBLOCK, bool STD>
-__global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArgs a, uint32_t table_bytes, int nbuf)
+template <int DT, int SBLOCK, bool STD, int NBUF>
+__global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArgs a, uint32_t table_bytes)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_abort;
@@ -84,21 +84,21 @@ __global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArg
     while (part.a < part.b) {
         const int g = part.g;
         const int64_t s1 = part.b;
-        const stage::Part next = stage::next_part(a.seg, G, a.Q, g + 1, start, end);
-        const bool more = next.a < next.b;
-        if (tid == 0 && more && nbuf == 2) copy(next.g, buf ^ 1);
-        const unsigned char* table = tables + buf * table_bytes;
         // first direction of this thread while the copy runs
         int64_t q = part.a + tid;
         float d0 = 0.f, d1 = 0.f, d2 = 0.f;
         if (q < s1) { d0 = __ldcs(a.dirs + 3 * q); d1 = __ldcs(a.dirs + 3 * q + 1); d2 = __ldcs(a.dirs + 3 * q + 2); }
+        const stage::Part next = stage::next_part(a.seg, G, a.Q, g + 1, start, end);
+        const bool more = next.a < next.b;
+        if (NBUF == 2 && tid == 0 && more) copy(next.g, buf ^ 1);
+        const unsigned char* table = NBUF == 2 ? tables + buf * table_bytes : tables;
         if (!stage::bar_wait(bar + 8 * buf, (phase >> buf) & 1, stage::WAIT_NS)) s_abort = 1;
         __syncthreads();
         if (s_abort) {
             status |= SHM_DEV_TIMEOUT;
             if (tid == 0) {
                 stage::bar_wait(bar + 8 * buf, (phase >> buf) & 1, stage::DRAIN_NS);
-                if (more && nbuf == 2) stage::bar_wait(bar + 8 * (buf ^ 1), (phase >> (buf ^ 1)) & 1, stage::DRAIN_NS);
+                if (NBUF == 2 && more) stage::bar_wait(bar + 8 * (buf ^ 1), (phase >> (buf ^ 1)) & 1, stage::DRAIN_NS);
             }
             break;
         }
@@ -135,31 +135,36 @@ __global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArg
             d0 = n0; d1 = n1; d2 = n2;
         }
         __syncthreads();  // every read of this table is done before the next copy lands
-        if (nbuf == 2) buf ^= 1;
+        if (NBUF == 2) buf ^= 1;
         else if (tid == 0 && more) copy(next.g, 0);
         part = next;
     }
     report_status(a.dev_status, status);
 }
 
+template <int DT, int SBLOCK, bool STD, int NBUF>
+cudaError_t launch_staged_n(const QueryArgs& a, uint32_t table_bytes, cudaStream_t s)
+{
+    const void* fn = (const void*)k_query_staged<DT, SBLOCK, STD, NBUF>;
+    const int smem = stage::TABLE_OFFSET + NBUF * (int)table_bytes;
+    cudaError_t e = ensure_dynamic_smem(fn, smem);
+    if (e != cudaSuccess) return e;
+    int resident = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, fn, SBLOCK, smem) != cudaSuccess || resident < 1)
+        resident = 1;
+    const int64_t blocks = stage::units_for(a.Q, a.L.n_glyphs, table_bytes / stage::QUERY_BYTES,
+                                            (int64_t)sm_count() * resident);
+    k_query_staged<DT, SBLOCK, STD, NBUF><<<(unsigned)blocks, SBLOCK, smem, s>>>(a, table_bytes);
+    return cudaGetLastError();
+}
+
 template <int DT, int SBLOCK, bool STD>
 cudaError_t launch_staged_o(const QueryArgs& a, uint32_t table_bytes, cudaStream_t s)
 {
     // a second buffer takes the next glyph's table while this one is queried, where two CTAs per SM
-    // still fit
-    const int nbuf = 2 * (int64_t)table_bytes <= STAGED_TABLE_MAX_BYTES ? 2 : 1;
-    const int smem = stage::TABLE_OFFSET + nbuf * (int)table_bytes;
-    cudaError_t e = ensure_dynamic_smem((const void*)k_query_staged<DT, SBLOCK, STD>, smem);
-    if (e != cudaSuccess) return e;
-    int resident = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_query_staged<DT, SBLOCK, STD>, SBLOCK, smem) !=
-            cudaSuccess ||
-        resident < 1)
-        resident = 1;
-    const int64_t blocks = stage::units_for(a.Q, a.L.n_glyphs, table_bytes / stage::QUERY_BYTES,
-                                            (int64_t)sm_count() * resident);
-    k_query_staged<DT, SBLOCK, STD><<<(unsigned)blocks, SBLOCK, smem, s>>>(a, table_bytes, nbuf);
-    return cudaGetLastError();
+    // still fit (a template: with one buffer its table is at a fixed address)
+    return 2 * (int64_t)table_bytes <= STAGED_TABLE_MAX_BYTES ? launch_staged_n<DT, SBLOCK, STD, 2>(a, table_bytes, s)
+                                                              : launch_staged_n<DT, SBLOCK, STD, 1>(a, table_bytes, s);
 }
 
 template <int DT, int SBLOCK>

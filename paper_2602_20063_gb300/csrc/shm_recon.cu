@@ -97,13 +97,13 @@ __global__ void __launch_bounds__(RS_BLOCK, 2) k_recon_staged(QueryArgs a, uint3
     if (tid == 0 && part.a < part.b) copy(part.g, 0);
     while (part.a < part.b) {
         const int g = part.g;
+        int64_t q = part.a + tid;
+        float d0 = 0.f, d1 = 0.f, d2 = 0.f;
+        if (q < part.b) { d0 = __ldcs(a.dirs + 3 * q); d1 = __ldcs(a.dirs + 3 * q + 1); d2 = __ldcs(a.dirs + 3 * q + 2); }
         const stage::Part next = stage::next_part(a.seg, G, a.Q, g + 1, start, end);
         const bool more = next.a < next.b;
         if (tid == 0 && more && nbuf == 2) copy(next.g, buf ^ 1);
         copy_rest(g, buf);
-        int64_t q = part.a + tid;
-        float d0 = 0.f, d1 = 0.f, d2 = 0.f;
-        if (q < part.b) { d0 = __ldcs(a.dirs + 3 * q); d1 = __ldcs(a.dirs + 3 * q + 1); d2 = __ldcs(a.dirs + 3 * q + 2); }
         if (!stage::bar_wait(bar + 8 * buf, (phase >> buf) & 1, stage::WAIT_NS)) s_abort = 1;
         __syncthreads();
         if (s_abort) {

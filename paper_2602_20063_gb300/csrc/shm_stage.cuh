@@ -87,20 +87,35 @@ __device__ __forceinline__ int64_t seg_at(const int64_t* seg, int64_t Q, int g)
     return min(max(__ldg(seg + g), (int64_t)0), Q);
 }
 
-// The path position at cost D (a whole warp calls it; 32 probes per round).
+// Cost of the path up to glyph g, and up to the start of unit u of `units`.
+__device__ __forceinline__ int64_t cost_of(const int64_t* seg, int64_t Q, int64_t w, int g)
+{
+    return seg_at(seg, Q, g) - seg_at(seg, Q, 0) + w * g;
+}
+
+__device__ __forceinline__ int64_t unit_cost(const int64_t* seg, int G, int64_t Q, int64_t w, int64_t u, int64_t units)
+{
+    const int64_t total = cost_of(seg, Q, w, G);
+    return total / units * u + total % units * u / units;
+}
+
+// The path position at cost D (a whole warp calls it; 32 probes per round, so two or three dependent
+// loads; a CTA has nothing else to do before its first copy).
 __device__ __forceinline__ Pos path_at(const int64_t* seg, int G, int64_t Q, int64_t w, int64_t D)
 {
     const int lane = threadIdx.x & 31;
     const int64_t lo = seg_at(seg, Q, 0);
     int g = 0, n = G + 1;  // the largest g in [0, G] with cost(g) = seg[g] - seg[0] + w g <= D
+    int64_t s = lo;        // seg[g]
     while (n > 1) {
         const int step = (n + 31) / 32, at = lane * step;
-        const unsigned m = __ballot_sync(0xffffffffu, at < n && seg_at(seg, Q, g + at) - lo + w * (g + at) <= D);
+        const int64_t v = at < n ? seg_at(seg, Q, g + at) : INT64_MAX / 2;
+        const unsigned m = __ballot_sync(0xffffffffu, at < n && v - lo + w * (g + at) <= D);
         const int k = 31 - __clz((int)(m | 1u));
+        s = __shfl_sync(0xffffffffu, v, k);
         g += k * step;
         n = min(step, n - k * step);
     }
-    const int64_t s = seg_at(seg, Q, g);
     return Pos{g, min(Q, s + max((int64_t)0, D - (s - lo + w * g) - w))};
 }
 
@@ -114,18 +129,6 @@ __device__ __forceinline__ Part next_part(const int64_t* seg, int G, int64_t Q, 
         if (a < b) return Part{g, a, b};
     }
     return Part{G, 0, 0};
-}
-
-// Cost of the path up to glyph g, and up to the start of unit u of `units`.
-__device__ __forceinline__ int64_t cost_of(const int64_t* seg, int64_t Q, int64_t w, int g)
-{
-    return seg_at(seg, Q, g) - seg_at(seg, Q, 0) + w * g;
-}
-
-__device__ __forceinline__ int64_t unit_cost(const int64_t* seg, int G, int64_t Q, int64_t w, int64_t u, int64_t units)
-{
-    const int64_t total = cost_of(seg, Q, w, G);
-    return total / units * u + total % units * u / units;
 }
 
 // This CTA's unit of the path: start and end positions through shared memory (every thread calls it).
