@@ -141,17 +141,25 @@ def _io_ptr(t: Optional[torch.Tensor]):
     return C.c_void_p(t.data_ptr())
 
 
+# The current stream's handle without a Stream object (0.2 us instead of 3 us a call) where torch has it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return C.c_void_p(stream.cuda_stream)
+    if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+        return C.c_void_p(_raw_stream(_raw_device()))
+    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
 def _io_empty(shape, dtype, like: torch.Tensor) -> torch.Tensor:
     """An output buffer next to `like`: on its device, or page-locked host memory when `like` is
     page-locked host memory (the kernels write it directly)."""
-    if like.device.type == "cpu":
-        return torch.empty(shape, dtype=dtype, pin_memory=True)
-    return torch.empty(shape, dtype=dtype, device=like.device)
+    if like.is_cuda:
+        return torch.empty(shape, dtype=dtype, device=like.device)
+    return torch.empty(shape, dtype=dtype, pin_memory=True)
 
 
 def _need(t: Optional[torch.Tensor], dtype, shape=None, name="tensor"):
@@ -256,6 +264,10 @@ def like_lut(L: Lut, dtype: int = None, layout: int = None, r0="same", zero=Fals
 
 
 # ------------------------------------------------------------------------------------------- query
+_QUERY_OUT = {"R": (1, torch.float32), "grad": (3, torch.float32), "normal": (3, torch.float32),
+              "chart": (2, torch.float32), "fij": (3, torch.int32)}
+
+
 def query(lut: Lut, dirs: torch.Tensor, glyph: torch.Tensor = None, seg: torch.Tensor = None,
           want=("R", "grad", "normal"), out: dict = None, dev_status: torch.Tensor = None, stream=None) -> dict:
     """shm_query: returns a dict of the requested outputs among R, grad, normal, chart, fij."""
@@ -264,10 +276,10 @@ def query(lut: Lut, dirs: torch.Tensor, glyph: torch.Tensor = None, seg: torch.T
     _need(glyph, torch.int32, (Q,), "glyph")
     _need(seg, torch.int64, (lut.n_glyphs + 1,), "seg")
     out = {} if out is None else out
-    shapes = {"R": (Q,), "grad": (Q, 3), "normal": (Q, 3), "chart": (Q, 2), "fij": (Q, 3)}
     for k in want:
         if k not in out:
-            out[k] = _io_empty(shapes[k], torch.int32 if k == "fij" else torch.float32, dirs)
+            width, dtype = _QUERY_OUT[k]
+            out[k] = _io_empty((Q, width) if width > 1 else (Q,), dtype, dirs)
     st = lib().shm_query(C.byref(lut.c()), Q, _io_ptr(dirs), _io_ptr(glyph), _io_ptr(seg), _io_ptr(out.get("R")),
                          _io_ptr(out.get("grad")), _io_ptr(out.get("normal")), _io_ptr(out.get("chart")),
                          _io_ptr(out.get("fij")), _io_ptr(dev_status), _stream(stream))

@@ -919,7 +919,7 @@ cudaError_t launch_pack(const LutView& src, const LutView& dst, void* dst_data, 
 // adjacent records once (512 contiguous bytes f32), the right-hand corners come from the next lane and the
 // upper ones from the row before, so each record is read 1.07 times instead of four and no cell index
 // is divided; eight rows are in flight per warp (one at a time: 100 us).  Bound: DRAM (the table once).
-// 512 bump objects, 280 MB: 62 -> 47 us.
+// 512 bump objects, 280 MB: 62 -> 55 us.
 constexpr int BOUNDS_ROWS = 32, BOUNDS_COLS = 31, BOUNDS_WARPS = 8, BOUNDS_BATCH = 8;
 
 struct BoundsUnits {
