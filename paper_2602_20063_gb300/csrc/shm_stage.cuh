@@ -56,18 +56,28 @@ __device__ __forceinline__ void init(uint32_t bar)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// Thread 0: copy `bytes` (a multiple of 16, 16-byte aligned source) into shared memory at dst,
-// completing on `bar`.  Earlier generic-proxy reads of the destination are ordered before it.
-__device__ __forceinline__ void issue(uint32_t bar, uint32_t dst, const unsigned char* src, uint32_t bytes)
+// Thread 0: `bar` completes when `bytes` have arrived.  Earlier generic-proxy accesses of the destination
+// are ordered before the copies that follow.
+__device__ __forceinline__ void expect(uint32_t bar, uint32_t bytes)
 {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-    for (uint32_t off = 0; off < bytes; off += BULK_PIECE) {
-        const uint32_t n = min(BULK_PIECE, bytes - off);
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(dst + off), "l"(src + off), "r"(n), "r"(bar)
-                     : "memory");
-    }
+}
+
+// Thread 0: copy `bytes` (a multiple of 16; 16-byte aligned addresses) into shared memory, counted on `bar`.
+__device__ __forceinline__ void copy(uint32_t bar, uint32_t dst, const void* src, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
+// Thread 0: copy `bytes` (a multiple of 16, 16-byte aligned source) into shared memory at dst,
+// completing on `bar`.
+__device__ __forceinline__ void issue(uint32_t bar, uint32_t dst, const unsigned char* src, uint32_t bytes)
+{
+    expect(bar, bytes);
+    for (uint32_t off = 0; off < bytes; off += BULK_PIECE) copy(bar, dst + off, src + off, min(BULK_PIECE, bytes - off));
 }
 
 // Position on the path: query q of glyph g (g = G: past the last one).

@@ -163,3 +163,24 @@ def test_binned_planet_full_size(S):
     maxG = np.linalg.norm(Gr, axis=1).max()
     assert np.abs(R - Rr).max() <= 1e-5 * np.abs(Rr).max()
     assert np.abs(G - Gr).max() <= 1e-4 * maxG + 3 * N * 2e-8
+
+
+@pytest.mark.parametrize("Q", [4095, 4096, 4097, 3 * 4096, 700 * 4096 + 17])
+@pytest.mark.parametrize("kind", ["uniform", "one_bin", "unaligned"])
+def test_binned_blocks(S, Q, kind):
+    """Full and partial blocks, several blocks per CTA, directions of a single bin (most runs empty, one as
+    long as its block), directions and outputs that bulk copies and vector stores cannot reach."""
+    lut = _glyph(23, N=48, L=4)
+    L, _ = upload_pool(S, [lut])
+    g = torch.Generator(device="cuda").manual_seed(Q)
+    d = torch.randn((Q + 1, 3), generator=g, device="cuda")
+    if kind == "one_bin":
+        d = d.mul_(0.001).add_(torch.tensor([1.0, 0.2, 0.3], device="cuda"))
+    d = d.view(-1)[1:1 + 3 * Q].view(Q, 3) if kind == "unaligned" else d[:Q]
+    ws = S.query_binned_workspace(L, Q, 20000)
+    out = {}
+    if kind == "unaligned":
+        for k, n in (("grad", 3), ("normal", 3)):
+            out[k] = torch.empty(n * Q + 1, device="cuda")[1:].view(Q, 3)
+    out = S.query_binned(L, d, ws, band_bytes=20000, want=WANT, out=out)
+    _equal(out, S.query(L, d, want=WANT))
