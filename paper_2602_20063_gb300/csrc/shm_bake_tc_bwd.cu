@@ -10,45 +10,51 @@ namespace tc {
 // with a CTA's group of up to 128 glyphs on the MMA M side (rows beyond the group hold stale data and
 // are never stored; see plan() for the group size) and the coefficients on N (K padded to
 // Kp <= 128).  Operands:
-//   A = dlut tiles [R glyphs x 16 c], loaded raw by TMA (64-byte swizzle) and split in place by
-//       six converter warps into tf32 hi = x truncated (overwriting the raw tile) and
-//       lo = tf32_rna(x - hi);
+//   A = dlut tiles [R glyphs x 32 c], loaded raw by TMA (128-byte swizzle) and split by four warps,
+//       one glyph row per thread, into tf32 hi = x truncated and lo = tf32_rna(x - hi), which go to
+//       TMEM: the MMAs read A from there;
 //   B = the transposed tf32 split of the basis, hiS / loS (part of shm_sh_basis's buffer), stored as
-//       one contiguous [Kp][16 c] slab per stage with its rows already in the 64-byte swizzled order
-//       that a tensor load would produce, so each stage's B tile is one plain bulk copy (a tensor
-//       load of [Kp][16] from a [Kp][4T] array would be Kp separate 64-byte pieces).
+//       one contiguous [Kp][16 c] slab per 16 columns with its rows already in the 64-byte swizzled
+//       order that a tensor load would produce, so each B tile is one plain bulk copy (a tensor load
+//       of [Kp][16] from a [Kp][4T] array would be Kp separate 64-byte pieces).
 // D = A_hi B_hi + A_hi B_lo + A_lo B_hi (3xTF32, as the forward bake), in two MMAs per K step: B_hi
 // and B_lo lie back to back in a stage, so A_hi [B_hi; B_lo] is one MMA of N = 2 Kp whose columns
 // [0, Kp) take A_hi B_hi and [Kp, 2 Kp) A_hi B_lo, and A_lo B_hi adds into [0, Kp); the drain warps
-// add both halves (TMEM: two buffers of 2 Kp columns).  Two MMA instructions instead of three per
-// K step at the same tensor work: 0.962 -> 0.870 ms on the glyph field, the MMA issuer being one of
-// the two roles that set the pace; the split, the other, runs on six warps (0.870 -> 0.853 ms).
+// add both halves.
+// What bounds it: HBM reads of dlut (455 MB in 67 us at 4,096 glyphs, N = 32) and, with hi and lo in
+// shared memory, that memory's port (78 KB of traffic per 8 KB of A: raw in, out, hi and lo in, and
+// out again for the MMAs; 46 KB with A in TMEM) and the per-stage work of the roles, which are serial
+// chains of waits.  A training step (query, its reverse, this kernel, the bake; 4,096 glyphs, N = 32,
+// L = 8) took 867 us with 16-column stages split in shared memory by six warps; 837 with two slabs a
+// stage; 834 with A in TMEM, 802 when the drain's sums stopped taking registers from the other roles
+// and ring positions were counted instead of divided, 797 without an L2 prefetch of dlut (160 KB of
+// loads in flight need none).  At 16,384 glyphs this kernel went from 853 us to about 380 (floor 267).
+// Tried: 1 / 4 slabs a stage 852 / 935 (the serial chain; too few TMEM slots); one accumulator and more
+// slots 802; stores to TMEM waited for a stage later 800-811.
 // Accuracy: the error of the tensor cores' float32 accumulation grew with the length of the sum
 // kept in one TMEM accumulator (measured: 4.6e-5 of the largest entry after 434 stages, against
 // 7.9e-6 for a plain float32 sum).  So the MMAs accumulate CH stages at a time into one of two
 // TMEM buffers, and four drain warps add each finished chunk into float32 registers (one glyph row
 // per thread, Kp values) while the MMAs fill the other buffer.
-// Latency: seven 28 KB stages, and the producer prefetches dlut into L2 in boxes of 1 KB per glyph
-// row (16 stages), two boxes ahead of the shared-memory loads: the rows of a tile lie 4T x 4 B apart,
-// so 64-byte pieces per row and stage would reach DRAM as scattered small requests.
+// TMEM (512 columns): two accumulators of 2 Kp columns, then as many split stages of 64 columns as
+// fit; at Kp = 128 one accumulator, else no column were left (each chunk's drain then holds up the MMAs).
 // The c range may be split over the S CTAs of a thread-block cluster (small glyph counts); at the
 // end every CTA writes its register sums to shared memory and each CTA sums a slice of them over
 // the cluster's ranks in rank order through distributed shared memory, so the result does not
 // depend on timing (deterministic, no atomics, no workspace).
 //   warp 0 lane 0: TMA producer   warp 1: TMEM allocation, lane 0 issues the MMAs
-//   warps 4-7: drain (TMEM lane quadrant = warp % 4) and epilogue   warps 2-3, 8-11: tf32 split
+//   warps 4-7: drain and its partial sums   warps 8-11: tf32 split   (TMEM lane quadrant = warp % 4)
 // Every mbarrier wait is bounded (1 s) and raises SHM_DEV_TIMEOUT on expiry; the cluster barriers
 // are reached by every thread of every CTA the same number of times, aborted or not.
 namespace bwd {
 
 constexpr int MG = 128;                       // glyph rows (MMA M)
-constexpr uint32_t A_TILE = MG * KC * 4;      // 8 KB
 constexpr int KPMAX = 128;                    // register sums per drain thread
-constexpr int CH = 16;                        // stages per TMEM chunk
-constexpr int PFW = 16;                       // stages per L2 prefetch box (256 c: 1 KB of each glyph row)
-constexpr int PFA = 2;                        // prefetch boxes ahead of the shared-memory loads
+constexpr int SUB = 2;                        // 16-column slabs per stage (a row of A: 128 bytes)
+constexpr uint32_t A_BYTES = MG * SUB * KC * 4;  // 16 KB
+constexpr int CH = 16 / SUB;                  // stages per TMEM chunk (256 columns)
 constexpr int THREADS = 384;
-constexpr int SPLIT_T = 192;                  // tf32-split threads: warps 2-3 and 8-11
+constexpr int SPLIT_T = 128;                  // tf32-split threads: warps 8-11, one glyph row each
 constexpr uint32_t STAGE_CAP = 196 * 1024;    // shared memory for the stages (and the partials after them)
 constexpr uint32_t BAR_BYTES = 1024;
 constexpr int MAXSTAGE = 8;
@@ -61,9 +67,11 @@ struct Args {
     int R;         // glyph rows per group (<= MG; the MMA's rows beyond R are never stored)
     int groups;
     int S;         // CTAs per cluster (splits of the c range)
-    int NC;        // stages over the whole c range
+    int NC;        // slabs over the whole c range
     int nstage;    // pipeline depth
-    uint32_t b_bytes, stage_bytes;
+    int nacc;      // accumulators in TMEM
+    int nslot;     // split A stages in TMEM
+    uint32_t b_bytes, stage_bytes;  // one B tile; a stage: A, then B hi and B lo of each slab
     float* dcoeffs;
     int32_t* dev_status;
 };
@@ -102,30 +110,50 @@ __device__ __forceinline__ float ld_dsmem(uint32_t local_addr, uint32_t rank)
     return v;
 }
 
-__device__ __forceinline__ void tma_prefetch_l2(const CUtensorMap* map, int x, int y)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"((uint64_t)map), "r"(x),
-                 "r"(y)
-                 : "memory");
-}
-
 __device__ __forceinline__ uint32_t idesc(int NB)
 {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(NB >> 3) << 17) | ((uint32_t)(MG >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_tf32_n(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc)
+// D += A B with A in TMEM (lane = row, one column per k) and B in shared memory.
+__device__ __forceinline__ void mma_tf32_n(uint32_t d, uint32_t a, uint64_t b, uint32_t id, uint32_t acc)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n"
-        ::"r"(d), "l"(a), "l"(b), "r"(id), "r"(acc)
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}\n"
+        ::"r"(d), "r"(a), "l"(b), "r"(id), "r"(acc)
         : "memory");
 }
 
+// 32 columns of this warp's 32 TMEM lanes
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
+        ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
+          "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
+          "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]),
+          "r"(taddr)
+        : "memory");
+}
+
+// Position in a ring of n buffers and the parity of its current pass.
+struct Ring {
+    int i, n;
+    uint32_t ph;
+    __device__ __forceinline__ explicit Ring(int n_) : i(0), n(n_), ph(0) {}
+    __device__ __forceinline__ void next()
+    {
+        if (++i == n) { i = 0; ph ^= 1; }
+    }
+};
+
 __global__ void __launch_bounds__(THREADS, 1)
-    k_sh_gemm_bwd_tc(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mApf, Args a)
+    k_sh_gemm_bwd_tc(const __grid_constant__ CUtensorMap mA, Args a)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -142,14 +170,15 @@ __global__ void __launch_bounds__(THREADS, 1)
     const uint32_t rank = cluster_rank();
     const int g_base = (blockIdx.x / a.S) * a.R;
     const int c0 = (int)(((int64_t)a.NC * rank) / a.S), c1 = (int)(((int64_t)a.NC * (rank + 1)) / a.S);
-    const int nst = c1 - c0;
+    const int nsl = c1 - c0;                     // slabs of this CTA
+    const int nst = (nsl + SUB - 1) / SUB;       // stages, the last one with fewer slabs perhaps
     const int nchunk = (nst + CH - 1) / CH;
     const uint32_t ID = idesc(a.Kp), ID2 = idesc(2 * a.Kp);
 
-    auto stA = [&](int st) { return stages + (size_t)st * a.stage_bytes; };
-    auto stAlo = [&](int st) { return stages + (size_t)st * a.stage_bytes + A_TILE; };
-    auto stBh = [&](int st) { return stages + (size_t)st * a.stage_bytes + 2 * A_TILE; };
-    auto stBl = [&](int st) { return stages + (size_t)st * a.stage_bytes + 2 * A_TILE + a.b_bytes; };
+    const auto slabs_of = [&](int it) { return min(SUB, nsl - it * SUB); };
+    // stage st: A raw, then B hi and B lo of slab u back to back
+    const auto stA = [&](int st) { return stages + (size_t)st * a.stage_bytes; };
+    const auto stB = [&](int st, int u) { return smem_u32(stA(st)) + A_BYTES + (uint32_t)u * 2 * a.b_bytes; };
 
     if (threadIdx.x == 0) {
         for (int st = 0; st < a.nstage; ++st) {
@@ -176,26 +205,28 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tmem_holder;
-    float acc[KPMAX];  // drain warps: the glyph row's running sums
-#pragma unroll
-    for (int i = 0; i < KPMAX; ++i) acc[i] = 0.0f;
+    const uint32_t tmem_a = tmem + (uint32_t)(a.nacc * 2 * a.Kp);  // then nslot split stages of 32 SUB columns
+    float* P = reinterpret_cast<float*>(stages);  // [128][Kp + 1] partial sums of this CTA, after the last MMA
+    const int PS = a.Kp + 1;
 
     if (warp == 0 && lane == 0) {
         // ---------------------------------------------------------------- TMA producer
-        for (int p = 0; p < PFA && p * PFW < nst; ++p) tma_prefetch_l2(&mApf, (c0 + p * PFW) * KC, g_base);
         int it = 0;
-        for (; it < nst; ++it) {
-            const int st = it % a.nstage;
-            const uint32_t ph = (uint32_t)(it / a.nstage) & 1;
+        Ring r(a.nstage);
+        for (; it < nst; ++it, r.next()) {
+            const int st = r.i;
+            const uint32_t ph = r.ph;
             if (!mbar_wait(empty0 + 8 * st, ph ^ 1, abort_flag, WAIT_LIMIT_NS)) break;
-            if (it % PFW == 0 && it + PFA * PFW < nst) tma_prefetch_l2(&mApf, (c0 + it + PFA * PFW) * KC, g_base);
             const uint32_t fb = full0 + 8 * st;
-            const int c = (c0 + it) * KC;
-            mbar_expect_tx(fb, (uint32_t)a.R * KC * 4 + 2 * a.b_bytes);
-            tma_load_2d(smem_u32(stA(st)), &mA, c, g_base, fb);
-            const size_t slab = (size_t)(c0 + it) * a.Kp * KC;
-            bulk_load(smem_u32(stBh(st)), a.hiS + slab, a.b_bytes, fb);
-            bulk_load(smem_u32(stBl(st)), a.loS + slab, a.b_bytes, fb);
+            const int m = slabs_of(it);
+            // the box is SUB slabs wide also where the range ends with fewer (columns past it are not used)
+            mbar_expect_tx(fb, (uint32_t)a.R * SUB * KC * 4 + (uint32_t)m * 2 * a.b_bytes);
+            tma_load_2d(smem_u32(stA(st)), &mA, (c0 + it * SUB) * KC, g_base, fb);
+            for (int u = 0; u < m; ++u) {
+                const size_t slab = (size_t)(c0 + it * SUB + u) * a.Kp * KC;
+                bulk_load(stB(st, u), a.hiS + slab, a.b_bytes, fb);
+                bulk_load(stB(st, u) + a.b_bytes, a.loS + slab, a.b_bytes, fb);
+            }
         }
         if (it < nst) {
             // aborted: the last load issued into each stage must land before the shared memory is reused
@@ -211,26 +242,30 @@ __global__ void __launch_bounds__(THREADS, 1)
         // ---------------------------------------------------------------- MMA issuer
         bool ok = true, any = false;
         int it = 0;
+        Ring rs(a.nstage), ra(a.nslot);
         for (int j = 0; j < nchunk && ok; ++j) {
-            const int b = j & 1;
-            if (!mbar_wait(cempty0 + 8 * b, ((uint32_t)(j >> 1) & 1) ^ 1, abort_flag, WAIT_LIMIT_NS)) { ok = false; break; }
+            const int b = j % a.nacc;
+            if (!mbar_wait(cempty0 + 8 * b, ((uint32_t)(j / a.nacc) & 1) ^ 1, abort_flag, WAIT_LIMIT_NS)) { ok = false; break; }
             fence_after();
             const uint32_t d = tmem + (uint32_t)(b * 2 * a.Kp);
             const int jend = min(nst, (j + 1) * CH);
-            for (; it < jend; ++it) {
-                const int st = it % a.nstage;
-                const uint32_t ph = (uint32_t)(it / a.nstage) & 1;
+            for (; it < jend; ++it, rs.next(), ra.next()) {
+                const int st = rs.i;
+                const uint32_t ph = rs.ph;
                 if (!mbar_wait(conv0 + 8 * st, ph, abort_flag, WAIT_LIMIT_NS)) { ok = false; break; }
                 fence_after();
-                const uint32_t ah = smem_u32(stA(st)), al = smem_u32(stAlo(st));
-                const uint32_t bh = smem_u32(stBh(st));
+                const int m = slabs_of(it);
+                for (int u = 0; u < m; ++u) {
+                    const uint32_t ah = tmem_a + (uint32_t)((ra.i * SUB + u) * 32), al = ah + 16;
+                    const uint32_t bh = stB(st, u);
 #pragma unroll
-                for (int kk = 0; kk < KC / 8; ++kk) {
-                    const uint32_t o = kk * 32;
-                    // columns [0, Kp): A_hi B_hi (+ A_lo B_hi below); [Kp, 2 Kp): A_hi B_lo, one MMA of
-                    // N = 2 Kp over the stage's B_hi and B_lo slabs, which lie back to back
-                    mma_tf32_n(d, sdesc(ah + o), sdesc(bh + o), ID2, (it != j * CH || kk != 0) ? 1u : 0u);
-                    mma_tf32_n(d, sdesc(al + o), sdesc(bh + o), ID, 1);
+                    for (int kk = 0; kk < KC / 8; ++kk) {
+                        const uint32_t o = kk * 32;  // bytes of 8 k in B; A: 8 columns
+                        // columns [0, Kp): A_hi B_hi (+ A_lo B_hi below); [Kp, 2 Kp): A_hi B_lo, one MMA of
+                        // N = 2 Kp over the slab's B_hi and B_lo, which lie back to back
+                        mma_tf32_n(d, ah + kk * 8, sdesc(bh + o), ID2, (it != j * CH || u != 0 || kk != 0) ? 1u : 0u);
+                        mma_tf32_n(d, al + kk * 8, sdesc(bh + o), ID, 1);
+                    }
                 }
                 any = true;
                 mma_commit(empty0 + 8 * st);
@@ -243,34 +278,56 @@ __global__ void __launch_bounds__(THREADS, 1)
             while (!mbar_try_wait(drain, 0) && globaltimer() - t0 < DRAIN_LIMIT_NS) {
             }
         }
-    } else if (warp >= 8 || warp == 2 || warp == 3) {
+    } else if (warp >= 8) {
         // ---------------------------------------------------------------- tf32 split of each stage
-        const int t = warp >= 8 ? threadIdx.x - 256 : threadIdx.x + 64;  // warps 8-11: 0-127, warps 2-3: 128-191
-        constexpr int n4 = (int)(A_TILE / 16);
-        for (int it = 0; it < nst; ++it) {
-            const int st = it % a.nstage;
-            const uint32_t ph = (uint32_t)(it / a.nstage) & 1;
-            if (!mbar_wait(full0 + 8 * st, ph, abort_flag, WAIT_LIMIT_NS)) break;
-            float4* hi = reinterpret_cast<float4*>(stA(st));
-            float4* lo = reinterpret_cast<float4*>(stAlo(st));
+        // thread = glyph row = TMEM lane; a stage's hi and lo go to 32 columns of TMEM per slab
+        const int wq = warp & 3, row = 32 * wq + lane;
+        const uint32_t lanes = (uint32_t)(32 * wq) << 16;
+        Ring rs(a.nstage), ra(a.nslot), rp(a.nstage);
+        for (int it = 0; it < nst; ++it, rs.next(), ra.next()) {
+            float4 v[SUB][4];
+            bool ok = mbar_wait(full0 + 8 * rs.i, rs.ph, abort_flag, WAIT_LIMIT_NS);
+            const uint8_t* src = stA(rs.i) + row * (SUB * KC * 4);
 #pragma unroll
-            for (int i = t; i < n4; i += SPLIT_T) {
-                const float4 x = hi[i];
-                float4 h, l;
-                h.x = tf32_trunc(x.x); h.y = tf32_trunc(x.y); h.z = tf32_trunc(x.z); h.w = tf32_trunc(x.w);
-                l.x = tf32_rna(x.x - h.x); l.y = tf32_rna(x.y - h.y); l.z = tf32_rna(x.z - h.z); l.w = tf32_rna(x.w - h.w);
-                hi[i] = h;
-                lo[i] = l;
+            for (int u = 0; u < SUB; ++u)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    v[u][q] = *reinterpret_cast<const float4*>(src + 16 * ((4 * u + q) ^ (row & 7)));
+            if (it >= a.nslot) {  // the MMAs that read this TMEM slot before
+                ok = ok && mbar_wait(empty0 + 8 * rp.i, rp.ph, abort_flag, WAIT_LIMIT_NS);
+                rp.next();
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_arrive(conv0 + 8 * st);
+            if (!__all_sync(0xFFFFFFFFu, ok)) break;
+            fence_after();
+#pragma unroll
+            for (int u = 0; u < SUB; ++u) {
+                uint32_t r[32];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float x[4] = {v[u][q].x, v[u][q].y, v[u][q].z, v[u][q].w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float h = tf32_trunc(x[e]);
+                        r[4 * q + e] = __float_as_uint(h);
+                        r[16 + 4 * q + e] = __float_as_uint(tf32_rna(x[e] - h));
+                    }
+                }
+                tmem_st32(tmem_a + lanes + (uint32_t)((ra.i * SUB + u) * 32), r);
+            }
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            fence_before();
+            mbar_arrive(conv0 + 8 * rs.i);
         }
     } else if (warp >= 4) {
         // ---------------------------------------------------------------- drain: chunk sums -> registers
         const int wq = warp & 3;
-        for (int j = 0; j < nchunk; ++j) {
-            const int b = j & 1;
-            if (!mbar_wait(cfull0 + 8 * b, (uint32_t)(j >> 1) & 1, abort_flag, WAIT_LIMIT_NS)) break;
+        float acc[KPMAX];  // the glyph row's running sums
+#pragma unroll
+        for (int i = 0; i < KPMAX; ++i) acc[i] = 0.0f;
+        int j = 0;
+        for (; j < nchunk; ++j) {
+            const int b = j % a.nacc;
+            if (!mbar_wait(cfull0 + 8 * b, (uint32_t)(j / a.nacc) & 1, abort_flag, WAIT_LIMIT_NS)) break;
             fence_after();
 #pragma unroll
             for (int cc = 0; cc < KPMAX; cc += 32) {
@@ -288,18 +345,17 @@ __global__ void __launch_bounds__(THREADS, 1)
             fence_before();
             mbar_arrive(cempty0 + 8 * b);
         }
+        // all MMAs of this CTA are done, so every stage has been loaded, split and read
+        if (j == nchunk) {
+            const int row = 32 * wq + lane;
+#pragma unroll
+            for (int i = 0; i < KPMAX; ++i)
+                if (i < a.Kp) P[row * PS + i] = acc[i];
+        }
     }
     __syncthreads();
     // ---------------------------------------------------------------- epilogue: cluster reduction
     const bool aborted = *abort_flag != 0;
-    float* P = reinterpret_cast<float*>(stages);  // [128][Kp + 1] partial sums of this CTA
-    const int PS = a.Kp + 1;
-    if (warp >= 4 && warp < 8 && !aborted) {
-        const int row = 32 * (warp & 3) + lane;
-#pragma unroll
-        for (int i = 0; i < KPMAX; ++i)
-            if (i < a.Kp) P[row * PS + i] = acc[i];
-    }
     cluster_sync();
     const uint32_t P_s = smem_u32(P);
     const int E = a.R * a.K;
@@ -341,12 +397,11 @@ __global__ void k_split_basis_t(const float* __restrict__ full, int K, int Kp, i
     }
 }
 
-// 2-D map over a row-major [rows][M4] f32 array, boxes of [box_rows][box_c]: the operand loads use
-// box_c = 16 with the 64-byte swizzle of the MMA descriptors; the L2 prefetch boxes are unswizzled.
-static bool make_map_c(CUtensorMap* m, const float* base, int rows, int M4, int box_rows, int box_c = KC,
-                       bool swizzle = true)
+// 2-D map over a row-major [rows][M4] f32 array, boxes of [box_rows][32] in the 128-byte swizzle (row
+// reads without bank conflicts).
+static bool make_map_c(CUtensorMap* m, const float* base, int rows, int M4, int box_rows)
 {
-    return encode_map_2d(m, base, M4, rows, box_c, box_rows, swizzle ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+    return encode_map_2d(m, base, M4, rows, SUB * KC, box_rows, CU_TENSOR_MAP_SWIZZLE_128B,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 
@@ -373,10 +428,13 @@ static bool plan(int G, int K, int Kp, int M4, int sms, int max_cluster, Args* o
     a.NC = (M4 + KC - 1) / KC;
     if (a.S > a.NC) a.S = a.NC;
     a.b_bytes = (uint32_t)Kp * KC * 4;
-    a.stage_bytes = 2 * A_TILE + 2 * a.b_bytes;
+    a.stage_bytes = A_BYTES + SUB * 2 * a.b_bytes;
     a.nstage = (int)(STAGE_CAP / a.stage_bytes);
     if (a.nstage > MAXSTAGE) a.nstage = MAXSTAGE;
     if (a.nstage < 2) return false;
+    a.nacc = 4 * a.Kp + 2 * 32 * SUB <= 512 ? 2 : 1;
+    a.nslot = (512 - a.nacc * 2 * a.Kp) / (32 * SUB);
+    if (a.nslot > a.nstage) a.nslot = a.nstage;
     if ((uint64_t)MG * (Kp + 1) * 4 > (uint64_t)a.nstage * a.stage_bytes) return false;  // partials fit
     *out = a;
     return true;
@@ -435,9 +493,8 @@ cudaError_t launch_sh_build_bwd_tc(int N, int G, int L, const float* dlut, const
     }
     Args a;
     if (!plan(G, K, Kp, M4, sm_count(), max_cluster, &a)) return cudaErrorNotSupported;
-    CUtensorMap mA, mApf;
-    if (((uintptr_t)hiS & 15u) != 0 || !make_map_c(&mA, dlut, G, M4, a.R) ||
-        !make_map_c(&mApf, dlut, G, M4, a.R, PFW * tc::KC, false))
+    CUtensorMap mA;
+    if (((uintptr_t)hiS & 15u) != 0 || !make_map_c(&mA, dlut, G, M4, a.R))
         return cudaErrorNotSupported;
     a.hiS = hiS;
     a.loS = loS;
@@ -455,6 +512,6 @@ cudaError_t launch_sh_build_bwd_tc(int N, int G, int L, const float* dlut, const
     attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_sh_gemm_bwd_tc, mA, mApf, a);
+    return cudaLaunchKernelEx(&cfg, k_sh_gemm_bwd_tc, mA, a);
 }
 }  // namespace shm

@@ -168,6 +168,23 @@ def test_build_backward_glyph_group_sizing(S, per_sm):
         assert np.abs(dcn[r] - oref).max() <= 2e-5 * np.abs(oref).max(), r
 
 
+@pytest.mark.parametrize("N,L,G", [(1, 9, 2), (33, 10, 129), (21, 9, 700), (12, 8, 1300), (14, 5, 1), (9, 3, 9800)])
+def test_build_backward_tensor_memory_slots(S, N, L, G):
+    """The tensor-core adjoint at each padded coefficient count (32, 64, 96, 128: six to two split stages in
+    tensor memory, and one accumulator instead of two at 128), odd and even slab counts per cluster rank, sums
+    shorter than a stage and longer than several chunks: every glyph against the float64 contraction of the
+    same float32 operands, 2e-5 of the largest entry."""
+    T = 6 * (N + 2) ** 2
+    K = (L + 1) ** 2
+    g = torch.Generator(device="cuda").manual_seed(100 * N + L)
+    D = S.alloc_lut(G, N)
+    D.data.copy_(torch.randn(D.data.numel(), device="cuda", generator=g))
+    basis = S.sh_basis(N, L)
+    dc = S.build_lut_backward(D, L, basis)
+    ref = D.data.view(G, T * 4).double() @ basis[:K * T * 4].view(K, T * 4).double().T
+    assert float((dc.double() - ref).abs().max()) <= 2e-5 * float(ref.abs().max())
+
+
 @pytest.mark.parametrize("G,N", [(1, 10), (300, 9), (257, 17)])
 def test_bake_snapshot_and_gradient_in_place(G, N):
     """sh_bake_fn's table is a snapshot (a later bake into the lut leaves it alone) with the lut's records,
