@@ -28,7 +28,7 @@ namespace tc {
 // L = 8) took 867 us with 16-column stages split in shared memory by six warps; 837 with two slabs a
 // stage; 834 with A in TMEM, 802 when the drain's sums stopped taking registers from the other roles
 // and ring positions were counted instead of divided, 797 without an L2 prefetch of dlut (160 KB of
-// loads in flight need none).  At 16,384 glyphs this kernel went from 853 us to about 380 (floor 267).
+// loads in flight need none).  At 16,384 glyphs this kernel went from 852 us to 597 (floor 267).
 // Tried: 1 / 4 slabs a stage 852 / 935 (the serial chain; too few TMEM slots); one accumulator and more
 // slots 802; stores to TMEM waited for a stage later 800-811.
 // Accuracy: the error of the tensor cores' float32 accumulation grew with the length of the sum

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(1024) k_zero_cut(const int64_t* seg, int G, in
 }
 
 template <int DT, bool FIT, bool SET>
-__global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uint32_t table_bytes, int nbuf)
+__global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uint32_t table_bytes, int nbuf, bool whole)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_abort;
@@ -219,12 +219,18 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
     }
     const int64_t w = table_bytes / BWD_PATH_BYTES;
     stage::Pos start, end;
-    stage::unit_of(a.seg, G, a.Q, w, s_unit, start, end);  // its barrier also publishes the mbarriers
+    if (whole) {  // grid: one CTA per glyph
+        start = stage::Pos{(int)blockIdx.x, 0};
+        end = stage::Pos{(int)blockIdx.x, a.Q};
+        __syncthreads();
+    } else {
+        stage::unit_of(a.seg, G, a.Q, w, s_unit, start, end);  // its barrier also publishes the mbarriers
+    }
 
     // SET: glyphs z .. are still to be zeroed (those wholly inside this unit, through glyph `last`)
     int z = start.g;
-    int64_t D0 = 0, D1 = 0;
-    if (SET) {
+    int64_t D0 = INT64_MIN, D1 = INT64_MAX;
+    if (SET && !whole) {
         D0 = stage::unit_cost(a.seg, G, a.Q, w, blockIdx.x, gridDim.x);
         D1 = stage::unit_cost(a.seg, G, a.Q, w, blockIdx.x + 1, gridDim.x);
     }
@@ -307,13 +313,20 @@ static cudaError_t launch_bwd_staged_ft(const BackwardArgs& a, uint32_t table_by
     cudaError_t e = ensure_dynamic_smem((const void*)k_query_bwd_staged<DT, FIT, SET>, smem);
     if (e != cudaSuccess) return e;
     const int64_t w = table_bytes / BWD_PATH_BYTES;
-    const int64_t blocks = stage::units_for(a.Q, a.L.n_glyphs, w, (int64_t)sm_count() * 2);
-    if (SET && blocks > 1) {
+    // Many glyphs, one table buffer: a CTA per glyph, which nothing cuts and which the hardware hands out as
+    // SMs come free.  Neighbouring glyphs are then in flight together (16,384 x 4,096 queries, even, N = 32:
+    // 2,055 us in cut units, 1,962 for strided glyphs, 1,727 so; 4,096 x 2,048: 352, 328, 297; uneven, in a
+    // training step: 795 -> 794).  Below 24 glyphs an SM the last uneven glyph shows (700 glyphs, N = 30:
+    // 321 -> 357), and with two buffers the unit hides the next table's copy (1,000 uneven glyphs of N = 20,
+    // in a training step: 376 -> 582).
+    const bool whole = nbuf == 1 && a.L.n_glyphs >= 24 * sm_count();
+    const int64_t blocks = whole ? a.L.n_glyphs : stage::units_for(a.Q, a.L.n_glyphs, w, (int64_t)sm_count() * 2);
+    if (SET && !whole && blocks > 1) {
         const int P = a.L.N_uniform + 2;
         k_zero_cut<<<(unsigned)(blocks - 1), 1024, 0, s>>>(a.seg, a.L.n_glyphs, a.Q, w, blocks,
                                                            reinterpret_cast<float4*>(a.dlut), 6 * P * P);
     }
-    k_query_bwd_staged<DT, FIT, SET><<<(unsigned)blocks, SBB, smem, s>>>(a, table_bytes, nbuf);
+    k_query_bwd_staged<DT, FIT, SET><<<(unsigned)blocks, SBB, smem, s>>>(a, table_bytes, nbuf, whole);
     return cudaGetLastError();
 }
 

@@ -235,3 +235,30 @@ def test_written_gradient_equals_accumulated(S, mode, dtype, N):
     assert ((x - r).abs().amax(0) <= 2e-6 * r.abs().amax(0)).all()
     if mode == "det":
         assert torch.equal(ref.data, got.data)
+
+
+@pytest.mark.parametrize("extra", [-1, 0, 7])
+def test_many_glyphs_one_cta_each(S, extra):
+    """From 24 glyphs per SM (tables too large for two buffers) the staged pass takes one CTA per glyph instead
+    of cut units: on both sides of that line, accumulated and written gradients of uneven segments (empty and
+    tiny ones, queries before and after all segments) equal the per-query pass with glyph ids."""
+    G, N = 24 * torch.cuda.get_device_properties(0).multi_processor_count + extra, 23
+    counts = [(g * 613) % 2100 * (g % 11 != 3) + g % 3 for g in range(G)]
+    seg, glyph, Q = _segments(counts, 33, 50)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    lut = S.alloc_lut(G, N)
+    lut.data.copy_(1.0 + 0.1 * torch.randn(lut.data.shape, generator=g, device="cuda"))
+    d = torch.nn.functional.normalize(torch.randn(Q, 3, generator=g, device="cuda"), dim=1)
+    up = [torch.randn(s, generator=g, device="cuda") for s in ((Q,), (Q, 3), (Q, 3))]
+    kw = dict(gR=up[0], ggrad=up[1], gnormal=up[2])
+    ref, acc, got = S.like_lut(lut, zero=True), S.like_lut(lut, zero=True), S.like_lut(lut)
+    got.data.fill_(float("nan"))
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    a = S.query_backward(lut, d, ref, glyph=_t(glyph), **kw)
+    for out, over in ((acc, False), (got, True)):
+        b = S.query_backward(lut, d, out, seg=_t(seg), overwrite=over, dev_status=st, **kw)
+        ok = torch.isfinite(a)
+        assert torch.equal(ok, torch.isfinite(b)) and float((a[ok] - b[ok]).abs().max()) <= 2e-6 * float(a[ok].abs().max())
+        r, x = ref.data.view(-1, 4).double(), out.data.view(-1, 4).double()
+        assert ((x - r).abs().amax(0) <= 2e-6 * r.abs().amax(0)).all()
+    assert st.item() == S.SHM_DEV_BOUNDS
