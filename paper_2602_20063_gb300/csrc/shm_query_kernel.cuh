@@ -27,9 +27,11 @@ constexpr QShape QSHAPES[N_QSHAPES] = {{512, 8}, {256, 16}, {1024, 4}, {256, 8}}
 // Work is handed out per CTA in contiguous chunks (up to 4,096 queries by default), so that for
 // per-glyph query segments a CTA serves whole glyphs and the glyph's table stays in that SM's L1 (two
 // CTAs per SM keep two tables of up to ~110 KB resident) instead of being pulled into several SMs.
-// Without segments a chunk is one round of BLOCK queries: there is no glyph to keep, a small batch
-// spreads over every SM (65,536 queries: 128 CTAs instead of 16, kernel 18 -> 5 us) and a large one has
-// no last wave of eight rounds (4K planet view, f16 cells, 4.6 M queries: 71 -> 60 us).
+// Without segments, and where a glyph has many chunks of queries, there is no glyph to keep: chunks of
+// one round up to CHUNK_WAVES chunks per CTA, longer ones above.  A small batch then spreads over every
+// SM (65,536 queries: 128 CTAs instead of 16, kernel 18 -> 5 us), a middling one has no last wave of
+// eight rounds (planet view, f16 cells, 4.6 M queries: 71 -> 60 us), and a large one keeps the longer
+// runs of neighbouring queries.
 //
 // VEC (all of dirs / grad / normal 16-byte aligned): for a full warp round (32 queries) the 384 B
 // of directions are read with 24 128-bit loads and the 384 B of gradients and of normals are
@@ -61,7 +63,7 @@ __global__ void __launch_bounds__(QBLOCK, (QueryOccupancy<RECON, QBLOCK>::min_bl
     int i = 0;
     // glyph of this lane's first query and the end of its segment (one search per warp and chunk)
     int g = 0;
-    int64_t seg_end = INT64_MAX;
+    int64_t seg_end = a.seg ? INT64_MIN : INT64_MAX;
     // direction of the first round: vector (full round) or scalar
     float4 pv = make_float4(0.f, 0.f, 0.f, 0.f);
     float n0 = 0.f, n1 = 0.f, n2 = 0.f;
@@ -77,7 +79,8 @@ __global__ void __launch_bounds__(QBLOCK, (QueryOccupancy<RECON, QBLOCK>::min_bl
     load_dirs(qw);
 #pragma unroll 1
     while (qw < a.Q) {
-        if (a.seg && i == 0) {
+        // a chunk that goes on in the same segment needs no search
+        if (a.seg && i == 0 && __any_sync(0xffffffffu, qw + lane >= seg_end || g < 0)) {
             g = (qw < __ldg(a.seg)) ? -1 : seg_find_warp(a.seg, G, qw);
             seg_end = (g >= 0 && g < G) ? __ldg(a.seg + g + 1) : 0;
         }
@@ -168,6 +171,11 @@ __global__ void __launch_bounds__(QBLOCK, (QueryOccupancy<RECON, QBLOCK>::min_bl
     report_status(a.dev_status, status);
 }
 
+// chunks per CTA below which chunks get shorter (f32, start of the range to its end: 4K planet view 68 -> 58
+// us; 64 glyphs of 20,391 queries, N = 47, 40 -> 31; 25 of 179,818, N = 30 in cells, 83.3 -> 82.1)
+constexpr int CHUNK_WAVES = 16, SEG_WAVES = 4;
+constexpr int64_t LONG_GLYPH = 16384;  // mean queries per glyph: four chunks of 4,096
+
 template <int DT, int LAYOUT, bool VEC, int RECON, int QBLOCK, int QIT>
 cudaError_t launch_fwd_v(const QueryArgs& a, cudaStream_t s)
 {
@@ -183,8 +191,10 @@ cudaError_t launch_fwd_v(const QueryArgs& a, cudaStream_t s)
     }
     const int64_t cap = (int64_t)sm_count() * resident;
     const int64_t total = (a.Q + QBLOCK - 1) / QBLOCK;
-    int64_t rounds = a.seg ? (total + cap - 1) / cap : 1;
+    const bool short_glyphs = a.seg && a.Q / LONG_GLYPH < a.L.n_glyphs;
+    int64_t rounds = short_glyphs ? (total + cap - 1) / cap : total / ((a.seg ? SEG_WAVES : CHUNK_WAVES) * cap);
     if (rounds > QIT) rounds = QIT;
+    if (rounds < 1) rounds = 1;
     int64_t blocks = (total + rounds - 1) / rounds;
     if (blocks > cap) blocks = cap;
     k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK><<<(unsigned)blocks, QBLOCK, 0, s>>>(a, (int)rounds);

@@ -154,11 +154,13 @@ __device__ __forceinline__ void unit_of(const int64_t* seg, int G, int64_t Q, in
     end = sh[1];
 }
 
-// Host: units for Q queries over G glyphs, at most `cap` (the CTAs that run at once).
+// Host: units for Q queries over G glyphs, at most `cap` (the CTAs that run at once); just under one
+// glyph each becomes one glyph each, which leaves even segments uncut.
 inline int64_t units_for(int64_t Q, int64_t G, int64_t w, int64_t cap)
 {
     const int64_t n = (Q + w * G) / (UNIT_MIN + (w < UNIT_MIN ? w : UNIT_MIN)) + 1;
-    return n < cap ? n : cap;
+    const int64_t m = n < cap ? n : cap;
+    return m > G && m - G <= m / 32 ? G : m;
 }
 
 template <int DT>

@@ -75,3 +75,27 @@ def test_split_value_tables_equal_per_query(S, method, N, dtype):
     for k in want:
         assert torch.equal(got[k].view(torch.int32), ref[k].view(torch.int32)), k
     assert st[0].item() == st[1].item() != 0
+
+
+@pytest.mark.parametrize("lens", [[3000000, 0, 7, 1700000, 0, 511], [40000] * 9 + [1, 0, 0, 90001], [5000000] * 2])
+@pytest.mark.parametrize("N,layout", [(47, 0), (9, 1)])
+def test_long_unstaged_segments_equal_per_query(S, N, layout, lens):
+    """Segments of many chunks on tables that are not staged (one to eight rounds a chunk, no search where a
+    segment goes on): bit-identical to the same queries with glyph ids."""
+    n = np.asarray(lens)
+    G, lead, tail = len(n), 600, 75
+    seg = np.concatenate([[0], np.cumsum(n)]).astype(np.int64) + lead
+    Q = int(seg[-1]) + tail
+    ids = np.full(Q, -1, dtype=np.int32)
+    ids[lead:Q - tail] = np.repeat(np.arange(G), n)
+    g = torch.Generator(device="cuda").manual_seed(N)
+    lut = S.alloc_lut(G, N, 0, layout)
+    lut.data.copy_(1.0 + 0.1 * torch.randn(lut.data.shape, generator=g, device="cuda"))
+    d = torch.nn.functional.normalize(torch.randn(Q, 3, generator=g, device="cuda"), dim=1)
+    want = ("R", "grad", "normal", "chart", "fij")
+    st = torch.zeros(2, dtype=torch.int32, device="cuda")
+    ref = S.query(lut, d, glyph=torch.from_numpy(ids).cuda(), want=want, dev_status=st[:1])
+    got = S.query(lut, d, seg=torch.from_numpy(seg).cuda(), want=want, dev_status=st[1:])
+    for k in want:
+        assert torch.equal(got[k].view(torch.int32), ref[k].view(torch.int32)), k
+    assert st[0].item() == st[1].item() == S.SHM_DEV_BOUNDS
