@@ -849,7 +849,7 @@ class Planet:
             self.config["random_queries"] = {"path": "direct (shm_query in query order)"}
         self.config["l2_fetch_granularity"] = self.pick_l2_granularity(self.l2g_choice)
         self.launches_per_step = ((1 if (self.dtype == 0 and self.layout == 0) else 2) + 1 +
-                                  (5 if self.random_mode == "binned" else 1))
+                                  (3 if self.random_mode == "binned" else 1))
 
     def query_random(self, out, stream=None, dirs=None, ws=None):
         d = self.dr if dirs is None else dirs
@@ -958,7 +958,7 @@ class Planet:
             "query_random": {"bound": "hbm", "algorithmic": self.Qr * per_q, "unit": "GB/s", "peak": peaks["hbm_gbs"],
                              "per_unit": f"{per_q} B/query: 4 corner records ({rec} B, the paper's 16-scalar "
                                          "accounting) + 12 B direction + 28 B outputs, no reuse assumed"
-                                         + ("; timed: the whole binned query (count, scan, partition, query in "
+                                         + ("; timed: the whole binned query (partition, query in "
                                             "partitioned order, gradient/normal back in query order)"
                                             if self.random_mode == "binned" else ""),
                              "files": rfiles},

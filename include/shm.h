@@ -140,19 +140,19 @@ shm_status shm_tune_reset(void);
  * §4.10 queried at uniformly random directions).  Same per-query results as shm_query with
  * glyph = seg = NULL (every query on glyph 0): R [Q], grad [Q][3], normal [Q][3] and the chart
  * derivatives chart [Q][2] (R_u, R_v), each may be NULL, in query order, bit-identical to
- * shm_query's.  Work: the queries are partitioned by the table region their 2x2 footprint reads
+ * shm_query's.  Work: the queries are partitioned, within blocks, by the table region their 2x2 footprint reads
  * -- face and band of cell rows, a band holding about band_bytes of records (0 = 32 MiB) -- the
  * query runs over the partitioned batch so that the bands in flight stay resident in L2, and the
- * results return to query order.  The partition is stable and computed on the device; nothing is
- * synchronised with the host.
+ * results return to query order.  The partition is computed on the device; nothing is synchronised
+ * with the host.
  *   - lut: any dtype, texel or cell layout, uniform resolution (N_uniform > 0, else
  *     SHM_ERR_UNSUPPORTED); only glyph 0 is read.
  *   - ws: device workspace of at least shm_query_binned_workspace_bytes(lut, Q, band_bytes)
- *     (about 25 B per query: the partitioned directions, intermediate R / R_u / R_v, one bin byte
- *     per query and per-tile counts), else SHM_ERR_WORKSPACE.  Its contents need no clearing and
+ *     (about 25 B per query: the partitioned directions, replaced by R / R_u / R_v, one bin byte
+ *     per query, per-block offsets and counters), else SHM_ERR_WORKSPACE.  Its contents need no clearing and
  *     are scratch after the call; two calls that overlap on the GPU must not share it.
  *   - dirs and the outputs follow shm_query's rules (device or page-locked host memory); the
- *     directions are read three times, so device memory is the fast case.
+ *     directions are read twice, so device memory is the fast case.
  *   - band_bytes < 0 or Q < 0: SHM_ERR_INVALID_ARG. */
 int64_t shm_query_binned_workspace_bytes(const shm_lut* lut, int64_t Q, int64_t band_bytes);
 /* Bins (6 faces x bands) the partition uses for (lut, band_bytes); *band_rows (host, may be NULL)
