@@ -20,8 +20,13 @@
 // L = 16, 2^22 queries: 3,777 -> 236 us (a thread per query with its Legendre table in local memory and
 // about 60 instructions per term before), about half of the FP32 rate of its 1,160 multiply-adds per
 // query; the error against 64 bits fell from 6.2e-7 to 5.0e-7 of the gradient.
-// k_sh_eval_ids: per-query glyphs; the coefficients are gathered, each once (the derivative by its own
-// recurrence), one query per thread.
+// Where fewer than EV_SHORT queries of a glyph are left, scaling its coefficients and a slab of mostly idle
+// lanes cost more than the queries: 32 queries then go a lane each (ev_one), lanes on glyphs of their own, and
+// runs of empty segments are searched over.  100,000 glyphs of L = 8, 1 / 2 / 4 queries each: 304 / 232 / 233 -> 26 /
+// 25 / 41 us (a thread per query before 45 / 83 / 123); 50,000 of 8: 120 -> 41; two segments among 200,000 empty ones
+// 16.4 ms -> 15 us.  With 16 queries each a slab takes 109 us for 800,000 queries, the lanes no less.
+// k_sh_eval_ids: per-query glyphs; ev_one for every query: the coefficients are gathered, each once (the
+// derivative by its own recurrence).
 #include <math.h>
 
 #include "shm_internal.h"
@@ -34,6 +39,7 @@ constexpr int EV_LMAX = 20;
 constexpr int EV_TERMS = (EV_LMAX + 1) * (EV_LMAX + 2) / 2;
 constexpr int EV_BLOCK = 128;
 constexpr int EV_WARPS = EV_BLOCK / 32;
+constexpr int EV_SHORT = 16;  // fewer queries of a glyph than this go a thread each
 constexpr int EV_RES = 4;  // CTAs per SM: 121 registers, no spills (five with 96 registers spill: 264 us)
 
 // Constants of the terms (M, l), l = M..L, in the order the families run.
@@ -193,6 +199,78 @@ __device__ __forceinline__ void ev_slab(const EvArgs& a, const float4* co, const
     }
 }
 
+// One query on glyph g (any int), a thread by itself: the coefficients are gathered, each once, and the
+// derivative runs by its own recurrence.  Lanes of a warp may be on different glyphs.
+__device__ __forceinline__ void ev_one(const EvArgs& a, const EvTable& T, int64_t q, int g, uint32_t& status)
+{
+    const int L = a.L, K = (L + 1) * (L + 1);
+    const float d0 = __ldg(a.dirs + 3 * q), d1 = __ldg(a.dirs + 3 * q + 1), d2 = __ldg(a.dirs + 3 * q + 2);
+    const float n2 = d0 * d0 + d1 * d1 + d2 * d2;
+    bool ok = (g >= 0 && g < a.G);
+    if (!ok) status |= SHM_DEV_BOUNDS;
+    if (ok && !ev_valid(n2)) { ok = false; status |= SHM_DEV_NONFINITE; }
+    if (!ok) {
+        ev_store_nan(a, q);
+        return;
+    }
+    const float il = rsqrtf(n2);
+    const Vec3 w{d0 * il, d1 * il, d2 * il};
+    const float* c = a.coeffs + (int64_t)g * K;
+    float C = 1.0f, S = 0.0f, R = 0.0f, gx = 0.0f, gy = 0.0f, gz = 0.0f;
+    int t = 0;
+    for (int M = 0; M <= L; ++M) {
+        float p1 = 1.0f, p2 = 0.0f, e1 = 0.0f, e2 = 0.0f;  // p and dp/dz of degrees l-1 and l-2
+        float U = 0.0f, V = 0.0f, Uz = 0.0f, Vz = 0.0f;
+        for (int l = M; l <= L; ++l, ++t) {
+            float p = 1.0f, e = 0.0f;
+            if (l > M) {
+                const float nbt = T.nbeta[t];
+                p = fmaf(w.z, p1, nbt * p2);
+                e = fmaf(w.z, e1, fmaf(nbt, e2, p1));
+                p2 = p1; e2 = e1;
+                p1 = p; e1 = e;
+            }
+            const float kc = T.kc[t];
+            const float cc = kc * __ldg(c + l * l + l + M), cs = kc * __ldg(c + l * l + l - M);
+            U = fmaf(cc, p, U);
+            V = fmaf(cs, p, V);
+            Uz = fmaf(cc, e, Uz);
+            Vz = fmaf(cs, e, Vz);
+        }
+        const float fm = (float)M;
+        if (M > 0) {
+            gx = fmaf(fm, C * U + S * V, gx);
+            gy = fmaf(fm, C * V - S * U, gy);
+            const float Cn = w.x * C - w.y * S;
+            S = w.x * S + w.y * C;
+            C = Cn;
+        }
+        R += C * U + S * V;
+        gz += C * Uz + S * Vz;
+    }
+    ev_finish(a, q, d0, d1, d2, w, R, gx, gy, gz);
+}
+
+// Glyph of each lane's query q0 + lane, given the glyph g of q0 (0 <= g < G, seg[g] <= q0): the number of
+// segment ends at or before it, counted over the next 32 ends held one per lane; a lane whose query lies
+// past all 32 (runs of empty segments) searches by itself.  Every lane calls it.
+__device__ __forceinline__ int ev_lane_glyph(const int64_t* seg, int G, int g, int64_t q0, int lane)
+{
+    const int64_t q = q0 + lane;
+    const int64_t end = g + 1 + lane <= G ? __ldg(seg + g + 1 + lane) : INT64_MAX;
+    int k = 0;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1)
+        if (__shfl_sync(0xffffffffu, end, k + s - 1) <= q) k += s;
+    if (__shfl_sync(0xffffffffu, end, k) > q) return g + k;
+    int lo = g + k + 1, hi = G + 1;  // seg[lo] <= q
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(seg + mid) <= q) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 // Warp w of W takes queries [Q w / W, Q (w + 1) / W) and walks the glyphs they belong to.
 __global__ void __launch_bounds__(EV_BLOCK, EV_RES) k_sh_eval_seg(EvArgs a, const __grid_constant__ EvTable T)
 {
@@ -213,8 +291,9 @@ __global__ void __launch_bounds__(EV_BLOCK, EV_RES) k_sh_eval_seg(EvArgs a, cons
     while (q < qe) {
         int64_t e = qe;  // end of glyph g's queries within the warp's range
         if (a.seg) {
-            if (g >= 0)
-                while (g < a.G && q >= __ldg(a.seg + g + 1)) ++g;
+            // the next segment holds q but for empty ones, which are searched over instead of walked
+            if (g >= 0 && g < a.G && q >= __ldg(a.seg + g + 1) && (++g < a.G) && q >= __ldg(a.seg + g + 1))
+                g = seg_find_warp(a.seg, a.G, q);
             e = g >= a.G ? qe : min(qe, __ldg(a.seg + g + 1));
         }
         if (g < 0 || g >= a.G) {
@@ -223,6 +302,14 @@ __global__ void __launch_bounds__(EV_BLOCK, EV_RES) k_sh_eval_seg(EvArgs a, cons
                 if (q + lane < e) ev_store_nan(a, q + lane);
             q = e;
             g = g < 0 ? 0 : g;
+            continue;
+        }
+        if (e - q < EV_SHORT) {
+            // 32 queries, each lane on its own glyph
+            const int gl = a.seg ? ev_lane_glyph(a.seg, a.G, g, q, lane) : g;
+            if (q + lane < qe) ev_one(a, T, q + lane, gl, status);
+            g = __shfl_sync(0xffffffffu, gl, 31);
+            q += 32;
             continue;
         }
         const float* c = a.coeffs + (int64_t)g * K;
@@ -255,56 +342,9 @@ __global__ void __launch_bounds__(EV_BLOCK, EV_RES) k_sh_eval_seg(EvArgs a, cons
 
 __global__ void __launch_bounds__(EV_BLOCK) k_sh_eval_ids(EvArgs a, const __grid_constant__ EvTable T)
 {
-    const int L = a.L, K = (L + 1) * (L + 1);
     uint32_t status = 0;
-    for (int64_t q = (int64_t)blockIdx.x * EV_BLOCK + threadIdx.x; q < a.Q; q += (int64_t)gridDim.x * EV_BLOCK) {
-        const int g = __ldg(a.glyph + q);
-        const float d0 = __ldg(a.dirs + 3 * q), d1 = __ldg(a.dirs + 3 * q + 1), d2 = __ldg(a.dirs + 3 * q + 2);
-        const float n2 = d0 * d0 + d1 * d1 + d2 * d2;
-        bool ok = (g >= 0 && g < a.G);
-        if (!ok) status |= SHM_DEV_BOUNDS;
-        if (ok && !ev_valid(n2)) { ok = false; status |= SHM_DEV_NONFINITE; }
-        if (!ok) {
-            ev_store_nan(a, q);
-            continue;
-        }
-        const float il = rsqrtf(n2);
-        const Vec3 w{d0 * il, d1 * il, d2 * il};
-        const float* c = a.coeffs + (int64_t)g * K;
-        float C = 1.0f, S = 0.0f, R = 0.0f, gx = 0.0f, gy = 0.0f, gz = 0.0f;
-        int t = 0;
-        for (int M = 0; M <= L; ++M) {
-            float p1 = 1.0f, p2 = 0.0f, e1 = 0.0f, e2 = 0.0f;  // p and dp/dz of degrees l-1 and l-2
-            float U = 0.0f, V = 0.0f, Uz = 0.0f, Vz = 0.0f;
-            for (int l = M; l <= L; ++l, ++t) {
-                float p = 1.0f, e = 0.0f;
-                if (l > M) {
-                    const float nbt = T.nbeta[t];
-                    p = fmaf(w.z, p1, nbt * p2);
-                    e = fmaf(w.z, e1, fmaf(nbt, e2, p1));
-                    p2 = p1; e2 = e1;
-                    p1 = p; e1 = e;
-                }
-                const float kc = T.kc[t];
-                const float cc = kc * __ldg(c + l * l + l + M), cs = kc * __ldg(c + l * l + l - M);
-                U = fmaf(cc, p, U);
-                V = fmaf(cs, p, V);
-                Uz = fmaf(cc, e, Uz);
-                Vz = fmaf(cs, e, Vz);
-            }
-            const float fm = (float)M;
-            if (M > 0) {
-                gx = fmaf(fm, C * U + S * V, gx);
-                gy = fmaf(fm, C * V - S * U, gy);
-                const float Cn = w.x * C - w.y * S;
-                S = w.x * S + w.y * C;
-                C = Cn;
-            }
-            R += C * U + S * V;
-            gz += C * Uz + S * Vz;
-        }
-        ev_finish(a, q, d0, d1, d2, w, R, gx, gy, gz);
-    }
+    for (int64_t q = (int64_t)blockIdx.x * EV_BLOCK + threadIdx.x; q < a.Q; q += (int64_t)gridDim.x * EV_BLOCK)
+        ev_one(a, T, q, __ldg(a.glyph + q), status);
     report_status(a.dev_status, status);
 }
 

@@ -77,3 +77,19 @@ def check_query(out_gpu, ref, tol_scale=1.0, mask=None):
         err = np.abs(Nn - ref["normal"]).max(1)
         assert np.all((err <= bound)[mask]), (err / bound)[mask].max()
     return eR / maxR, eG / maxG
+
+
+def best_us(fn, windows=7, passes=10):
+    """Device time of one call of fn in us: the smallest mean over windows of back-to-back calls."""
+    for _ in range(3):
+        fn()
+    best = float("inf")
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    for _ in range(windows):
+        e0.record()
+        for _ in range(passes):
+            fn()
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, e0.elapsed_time(e1) * 1000 / passes)
+    return best
