@@ -915,12 +915,19 @@ cudaError_t launch_pack(const LutView& src, const LutView& dst, void* dst_data, 
 // Bounds: per cell, |r| <= max|r0 + r_ab| + (max|r_u h| + max|r_v h|)/4 + max|r_uv h^2|/16 over the
 // cell's four corners (value weights are >= 0 and sum to 1; sum_a |H^d_a| = s(1-s) <= 1/4).
 //
-// A warp walks a strip of 31 cell columns down up to BOUNDS_ROWS cell rows of a face: per row it loads 32
-// adjacent records once (512 contiguous bytes f32), the right-hand corners come from the next lane and the
-// upper ones from the row before, so each record is read 1.07 times instead of four and no cell index
-// is divided; eight rows are in flight per warp (one at a time: 100 us).  Bound: DRAM (the table once).
-// 512 bump objects, 280 MB: 62 -> 55 us.
+// Two forms.  k_bounds_strips: a warp walks a strip of 31 cell columns down up to BOUNDS_ROWS cell rows of a
+// face: per row it loads 32 adjacent records once (512 contiguous bytes), the right-hand corners come from the
+// next lane and the upper ones from the row before, so each record is read 1.07 times instead of four and no
+// cell index is divided; eight rows are in flight per warp (one at a time: 100 us).  Bound: DRAM (the table once).
+// k_bounds_cells: a thread per cell reads its four corners, which L1 serves after the first.
+// The strips are for float32 texel tables of at least BOUNDS_STRIP_N: below, most of a strip's lanes and of its
+// batches of rows lie past the face, and records of 8 B or whole cells leave it too few bytes in flight.
+// Strips against cells in us: one f32 texel table of N = 2048 / 1024 / 512 68 / 20.5 / 11.9 against 96.6 / 26.3 /
+// 14.9; 600 of N = 80 73 against 90, 1,000 of N = 64 101 against 96.5, 4,096 of N = 32 154 against 107, 20,000 of N = 8 140 against 58; f16 N = 2048
+// 110 against 80, f32 cells 237 against 222.
 constexpr int BOUNDS_ROWS = 32, BOUNDS_COLS = 31, BOUNDS_WARPS = 8, BOUNDS_BATCH = 8;
+constexpr int BOUNDS_STRIP_N = 80;
+constexpr int BOUNDS_CELLS = 2048;  // cells per CTA of k_bounds_cells
 
 struct BoundsUnits {
     int strips, chunks;
@@ -929,19 +936,31 @@ struct BoundsUnits {
     __host__ __device__ int64_t count() const { return 6LL * strips * chunks; }
 };
 
+// Largest bound of a CTA's threads into rmax[g]; every thread calls it.
+__device__ __forceinline__ void bounds_max(float best, float* rmax, int g)
+{
+    __shared__ float warp_best[BOUNDS_WARPS];
+    for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if ((threadIdx.x & 31) == 0) warp_best[threadIdx.x >> 5] = best;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < BOUNDS_WARPS; ++w) best = fmaxf(best, warp_best[w]);
+        // non-negative floats order like their bit patterns
+        atomicMax(reinterpret_cast<int*>(rmax + g), __float_as_int(best));
+    }
+}
+
 // |r0 + r|, |r_u h|, |r_v h|, |r_uv h^2| of texel (i, j), zero beyond the face and for NaN.
-template <int DT, int LAYOUT>
 __device__ __forceinline__ float4 abs_texel(const LutView& L, const GlyphRef& G, int f, int j, int i)
 {
     if (i > G.N + 1) return make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 v = load_texel(L.data, DT, LAYOUT, G, f, j, i);
+    const float4 v = load_texel(L.data, SHM_F32, SHM_LAYOUT_TEXEL, G, f, j, i);
     return make_float4(fmaxf(fabsf(G.r0 + v.x), 0.f), fmaxf(fabsf(v.y), 0.f), fmaxf(fabsf(v.z), 0.f), fmaxf(fabsf(v.w), 0.f));
 }
 
-template <int DT, int LAYOUT, class Map>
-__global__ void __launch_bounds__(32 * BOUNDS_WARPS) k_bounds(LutView L, float* rmax, const __grid_constant__ Map map)
+template <class Map>
+__global__ void __launch_bounds__(32 * BOUNDS_WARPS) k_bounds_strips(LutView L, float* rmax, const __grid_constant__ Map map)
 {
-    __shared__ float warp_best[BOUNDS_WARPS];
     int blk;
     const int g = map_block(map, blk);
     const GlyphRef G = glyph_ref(L, g);
@@ -962,7 +981,7 @@ __global__ void __launch_bounds__(32 * BOUNDS_WARPS) k_bounds(LutView L, float* 
         for (int j = j0; j < j1; j += BOUNDS_BATCH) {  // texel rows j + 1 .. j + BOUNDS_BATCH, loaded together
             float4 v[BOUNDS_BATCH];
 #pragma unroll
-            for (int r = 0; r < BOUNDS_BATCH; ++r) v[r] = abs_texel<DT, LAYOUT>(L, G, f, min(j + r, j1 - 1) + 1, i);
+            for (int r = 0; r < BOUNDS_BATCH; ++r) v[r] = abs_texel(L, G, f, min(j + r, j1 - 1) + 1, i);
 #pragma unroll
             for (int r = 0; r < BOUNDS_BATCH; ++r) {
                 const float4 m = row(v[r]);
@@ -972,33 +991,77 @@ __global__ void __launch_bounds__(32 * BOUNDS_WARPS) k_bounds(LutView L, float* 
             }
         }
     }
-    for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if (lane == 0) warp_best[warp] = best;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < BOUNDS_WARPS; ++w) best = fmaxf(best, warp_best[w]);
-        // non-negative floats order like their bit patterns
-        atomicMax(reinterpret_cast<int*>(rmax + g), __float_as_int(best));
+    bounds_max(best, rmax, g);
+}
+
+template <int DT, int LAYOUT>
+__device__ __forceinline__ float cell_bound(const LutView& L, const GlyphRef& G, int f, int i, int j)
+{
+    const Corners cr = fetch_corners<DT, LAYOUT>(L.data, G, f, i, j);
+    const float4 v[4] = {cr.c00, cr.c10, cr.c01, cr.c11};
+    float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        m0 = fmaxf(m0, fabsf(G.r0 + v[k].x));
+        m1 = fmaxf(m1, fabsf(v[k].y));
+        m2 = fmaxf(m2, fabsf(v[k].z));
+        m3 = fmaxf(m3, fabsf(v[k].w));
     }
+    return m0 + 0.25f * (m1 + m2) + 0.0625f * m3;
+}
+
+template <int DT, int LAYOUT, class Map>
+__global__ void __launch_bounds__(32 * BOUNDS_WARPS) k_bounds_cells(LutView L, float* rmax, const __grid_constant__ Map map)
+{
+    int blk;
+    const int g = map_block(map, blk);
+    const GlyphRef G = glyph_ref(L, g);
+    const int N = G.N, P = N + 1;
+    const int64_t ncell = 6LL * P * P;
+    const int64_t c0 = (int64_t)blk * BOUNDS_CELLS, c_end = min(ncell, c0 + BOUNDS_CELLS);
+    float best = 0.0f;
+    if (ncell <= 0x7fffffff) {  // 32-bit cell arithmetic (N < 18,900)
+        const uint32_t PP = (uint32_t)P * (uint32_t)P;
+        for (uint32_t c = (uint32_t)c0 + threadIdx.x; c < (uint32_t)c_end; c += blockDim.x) {
+            const uint32_t f = c / PP, rem = c - f * PP, j = rem / (uint32_t)P, i = rem - j * (uint32_t)P;
+            best = fmaxf(best, cell_bound<DT, LAYOUT>(L, G, (int)f, (int)i, (int)j));
+        }
+    } else {
+        for (int64_t c = c0 + threadIdx.x; c < c_end; c += blockDim.x) {
+            const int f = (int)(c / ((int64_t)P * P)), rem = (int)(c % ((int64_t)P * P)), j = rem / P, i = rem % P;
+            best = fmaxf(best, cell_bound<DT, LAYOUT>(L, G, f, i, j));
+        }
+    }
+    bounds_max(best, rmax, g);
 }
 
 cudaError_t launch_bounds(const LutView& L, float* rmax, const Sizes& sz, cudaStream_t s)
 {
     cudaError_t e = cudaMemsetAsync(rmax, 0, sizeof(float) * (size_t)L.n_glyphs, s);
     if (e != cudaSuccess) return e;
-    auto blocks = [](int N) { return (BoundsUnits(N).count() + BOUNDS_WARPS - 1) / BOUNDS_WARPS; };
+    constexpr int T = 32 * BOUNDS_WARPS;
+    // a pool's glyphs of either kind in a launch of their own
+    const bool strips = L.dtype == SHM_F32 && L.layout == SHM_LAYOUT_TEXEL;
+    const auto by_strips = [strips](int N) { return strips && N >= BOUNDS_STRIP_N; };
+    if (by_strips(sz.max_N)) {
+        const auto blocks = [&](int N) { return by_strips(N) ? (BoundsUnits(N).count() + BOUNDS_WARPS - 1) / BOUNDS_WARPS : 0; };
+        e = for_each_glyph_chunk(sz, blocks, [&](unsigned bx, unsigned bz, const auto& map) {
+            k_bounds_strips<<<dim3(bx, 1, bz), T, 0, s>>>(L, rmax, map);
+        });
+        if (e != cudaSuccess) return e;
+    }
+    const auto blocks = [&](int N) { return by_strips(N) ? 0 : (6LL * (N + 1) * (N + 1) + BOUNDS_CELLS - 1) / BOUNDS_CELLS; };
     return for_each_glyph_chunk(sz, blocks, [&](unsigned bx, unsigned bz, const auto& map) {
         using M = std::decay_t<decltype(map)>;
         const dim3 grid(bx, 1, bz);
-        constexpr int T = 32 * BOUNDS_WARPS;
         if (L.layout == SHM_LAYOUT_TEXEL) {
-            if (L.dtype == SHM_F32) k_bounds<SHM_F32, SHM_LAYOUT_TEXEL, M><<<grid, T, 0, s>>>(L, rmax, map);
-            else if (L.dtype == SHM_F16) k_bounds<SHM_F16, SHM_LAYOUT_TEXEL, M><<<grid, T, 0, s>>>(L, rmax, map);
-            else k_bounds<SHM_BF16, SHM_LAYOUT_TEXEL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            if (L.dtype == SHM_F32) k_bounds_cells<SHM_F32, SHM_LAYOUT_TEXEL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            else if (L.dtype == SHM_F16) k_bounds_cells<SHM_F16, SHM_LAYOUT_TEXEL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            else k_bounds_cells<SHM_BF16, SHM_LAYOUT_TEXEL, M><<<grid, T, 0, s>>>(L, rmax, map);
         } else {
-            if (L.dtype == SHM_F32) k_bounds<SHM_F32, SHM_LAYOUT_CELL, M><<<grid, T, 0, s>>>(L, rmax, map);
-            else if (L.dtype == SHM_F16) k_bounds<SHM_F16, SHM_LAYOUT_CELL, M><<<grid, T, 0, s>>>(L, rmax, map);
-            else k_bounds<SHM_BF16, SHM_LAYOUT_CELL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            if (L.dtype == SHM_F32) k_bounds_cells<SHM_F32, SHM_LAYOUT_CELL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            else if (L.dtype == SHM_F16) k_bounds_cells<SHM_F16, SHM_LAYOUT_CELL, M><<<grid, T, 0, s>>>(L, rmax, map);
+            else k_bounds_cells<SHM_BF16, SHM_LAYOUT_CELL, M><<<grid, T, 0, s>>>(L, rmax, map);
         }
     });
 }

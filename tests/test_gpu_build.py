@@ -16,7 +16,7 @@ import torch
 
 import oracle as O
 import shm_inputs as I
-from gpu_common import check_query, shm, upload_pool
+from gpu_common import best_us, check_query, shm, upload_pool
 
 pytestmark = pytest.mark.gpu
 
@@ -359,3 +359,61 @@ def test_fbm_regions_match_sampled_values(S, N, octaves, base):
     assert (lut.data - ref.data).abs().max().item() <= tol
     if base == 3.0e5:
         assert torch.equal(lut.data, ref.data)
+
+
+def _torch_bounds(rec, N, r0):
+    """Largest cell bound of records [6][N+2][N+2][4] in float64."""
+    v = rec.double().abs()
+    v[..., 0] = (rec[..., 0].double() + r0).abs()
+    m = torch.maximum(torch.maximum(v[:, :-1, :-1], v[:, :-1, 1:]), torch.maximum(v[:, 1:, :-1], v[:, 1:, 1:]))
+    return float((m[..., 0] + 0.25 * (m[..., 1] + m[..., 2]) + 0.0625 * m[..., 3]).max())
+
+
+@pytest.mark.parametrize("dtype,layout", [(0, 0), (1, 0), (2, 0), (0, 1), (1, 1)])
+def test_bounds_large_and_mixed(S, dtype, layout):
+    """Bounds of faces of several strips and row chunks (float32 texels from N = 80) and of every other pool (a
+    thread per cell), in a pool that mixes both and in uniform pools: the largest cell in each face corner, edge
+    and in the middle in turn, against float64; four roundings of a float32 sum."""
+    Ns = [1, 16, 30, 31, 79, 80, 92, 93, 128, 250]
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r0 = np.linspace(-0.5, 0.5, len(Ns)).astype(np.float32)
+    src = S.alloc_lut(len(Ns), Ns, r0=r0)
+    src.data.copy_(torch.randn(src.data.shape, generator=g, device="cuda"))
+    recs, at = [], 0
+    for k, N in enumerate(Ns):
+        n = 6 * (N + 2) ** 2
+        recs.append(src.data.view(-1, 4)[at:at + n].view(6, N + 2, N + 2, 4))
+        at += n
+        P = N + 2
+        spot = [(0, 0), (0, P - 1), (P - 1, 0), (P - 1, P - 1), (P // 2, P - 1), (31 % P, 32 % P), (33 % P, 30 % P),
+                (P - 1, 62 % P), (64 % P, 93 % P), (P // 2, P // 2)][k]
+        recs[k][k % 6, spot[0], spot[1], k % 4] = 40.0 + k
+
+    def pool(idx):
+        uniform = len(set(Ns[i] for i in idx)) == 1
+        one = S.alloc_lut(len(idx), Ns[idx[0]] if uniform else [Ns[i] for i in idx], r0=r0[list(idx)])
+        one.data.copy_(torch.cat([recs[i].reshape(-1) for i in idx]))
+        dst = S.like_lut(one, dtype=dtype, layout=layout)
+        S.pack_lut(one, dst)
+        back = S.like_lut(one)
+        S.pack_lut(dst, back)
+        got, at = S.lut_bounds(dst).cpu().numpy(), 0
+        for i, x in zip(idx, got):
+            n = 6 * (Ns[i] + 2) ** 2
+            ref = _torch_bounds(back.data.view(-1, 4)[at:at + n].view(6, Ns[i] + 2, Ns[i] + 2, 4), Ns[i], float(r0[i]))
+            at += n
+            assert abs(x - ref) <= 4 * 2.0 ** -24 * ref, (Ns[i], x, ref)
+
+    pool(range(len(Ns)))
+    for i in range(len(Ns)):
+        pool([i, i])
+
+
+def test_bounds_half_tables_cost_no_more(S):
+    """16-bit tables hold half the bytes of float32 ones: their bounds take at most 1.5 times as long."""
+    t = {}
+    for dtype in (0, 1):
+        lut = S.alloc_lut(2048, 32, dtype)
+        lut.data.zero_()
+        t[dtype] = best_us(lambda: S.lut_bounds(lut))
+    assert t[1] <= 1.5 * t[0], t
