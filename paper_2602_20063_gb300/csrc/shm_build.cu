@@ -417,8 +417,12 @@ __device__ __forceinline__ float2 value_noise_lattice2(float2 x, float2 y, float
 // ------------------------------------------------------------------------------------------
 // Sampled sources: value tables (k_value_build) and finite-difference records (k_fd_face).
 constexpr int FS = 18, MAX_BUMPS_SMEM = 128;
-constexpr int FBM_T = 48;        // region edge of the fBm bake: 64 / 48 / 32 texels measured 470 / 474 / 590 us at
-                                 // N = 2048, 160 / 154 / 186 at N = 1024 (larger regions miss the cache there)
+// Longest region edge of the fBm bake: 64 / 48 / 32 texels measured 470 / 474 / 590 us at N = 2048, 160 / 154 / 186 at
+// N = 1024 (larger regions miss the cache there).  A face is cut into equal regions of at most that: 48 + 2 texels
+// for N = 48 took 60 us (64 glyphs, six octaves), 2 x 25 take 49 and the whole face 38.  Faces of up to FBM_WHOLE
+// texels stay whole where there are enough of them for every SM (16 glyphs: whole 20.5 us, cut 16.5).
+constexpr int FBM_T = 48;
+constexpr int FBM_WHOLE = 66;
 constexpr int FBM_CACHE = 5376;  // lattice entries of the octaves' boxes per CTA (42 KB, four CTAs per SM)
 constexpr int FBM_MAX_OCT = 16;  // octaves whose boxes may be cached
 
@@ -654,7 +658,7 @@ __global__ void __launch_bounds__(256, 4) k_fbm_face(LutView out, void* data, sh
 {
     extern __shared__ float Sf[];  // [T+2][T+2]
     __shared__ float2 cache[FBM_CACHE];
-    __shared__ float s_xy[2 * (FBM_T + 2)];
+    __shared__ float s_xy[2 * (FBM_WHOLE + 2)];
     __shared__ uint4 s_oct[FBM_MAX_OCT];  // index constant, nx, nxy, boxed
     __shared__ uint2 s_inv[FBM_MAX_OCT];  // idx / nx = umulhi(idx, .x), idx / nxy = umulhi(idx, .y): idx nxy < 2^32
     __shared__ int s_box[FBM_MAX_OCT + 1][4];  // x0, y0, z0 and first cache entry (the last row: entries used)
@@ -662,10 +666,10 @@ __global__ void __launch_bounds__(256, 4) k_fbm_face(LutView out, void* data, sh
     const int g = map_block(map, region), f = blockIdx.y;
     const GlyphRef Gr = glyph_ref(out, g);
     const int N = Gr.N, P = N + 2;
-    const int nr = (P + T - 1) / T;
+    const int nr = (P + T - 1) / T, Te = (P + nr - 1) / nr;  // regions of Te x Te texels, the last ones of a row shorter
     if (region >= nr * nr) return;
-    const int i0 = (region % nr) * T, j0 = (region / nr) * T;  // first texel of the region
-    const int ti = min(T, P - i0), tj = min(T, P - j0);      // texels in the region
+    const int i0 = (region % nr) * Te, j0 = (region / nr) * Te;  // first texel of the region
+    const int ti = min(Te, P - i0), tj = min(Te, P - j0);      // texels in the region
     const int Si = ti + 2, Sj = tj + 2;                       // samples: texels i0-1 .. i0+ti
     const int tid = threadIdx.x;
     const int k = f >> 1;
@@ -796,7 +800,8 @@ cudaError_t launch_fd_build(const LutView& out, void* data, const shm_source& sr
     int T = (sz.max_N <= FACE_N_MAX) ? sz.max_N + 2 : REGION_T;
     const bool fbm = src.kind == SHM_SRC_FBM;
     if (fbm) {
-        T = sz.max_N + 2 < FBM_T ? sz.max_N + 2 : FBM_T;
+        const int P = sz.max_N + 2;
+        T = P <= FBM_T || (P <= FBM_WHOLE && 6LL * sz.G >= sm_count()) ? P : FBM_T;
     } else {
         if (sz.N_uniform == 0 && T > FACE_SPLIT_T) T = FACE_SPLIT_T;
         if (sz.N_uniform > 0 && T <= FACE_N_MAX + 2 && (T + 2) * (T + 2) * (int)sizeof(float) > FACE_SPLIT_SMEM)
@@ -977,7 +982,7 @@ __global__ void __launch_bounds__(32 * BOUNDS_WARPS) k_bounds_strips(LutView L, 
             return make_float4(fmaxf(c.x, __shfl_down_sync(0xffffffffu, c.x, 1)), fmaxf(c.y, __shfl_down_sync(0xffffffffu, c.y, 1)),
                                fmaxf(c.z, __shfl_down_sync(0xffffffffu, c.z, 1)), fmaxf(c.w, __shfl_down_sync(0xffffffffu, c.w, 1)));
         };
-        float4 up = row(abs_texel<DT, LAYOUT>(L, G, f, j0, i));
+        float4 up = row(abs_texel(L, G, f, j0, i));
         for (int j = j0; j < j1; j += BOUNDS_BATCH) {  // texel rows j + 1 .. j + BOUNDS_BATCH, loaded together
             float4 v[BOUNDS_BATCH];
 #pragma unroll

@@ -417,3 +417,26 @@ def test_bounds_half_tables_cost_no_more(S):
         lut.data.zero_()
         t[dtype] = best_us(lambda: S.lut_bounds(lut))
     assert t[1] <= 1.5 * t[0], t
+
+
+def test_fbm_cost_grows_with_the_texels(S):
+    """A face just above the region edge costs no more per texel than one just below it (1.2 times at most)."""
+    keys = torch.from_numpy(I.fbm_keys(7, 6).view(np.int32)).cuda()
+    t = {}
+    for N in (46, 48):
+        lut = S.alloc_lut(64, N)
+        src = S.Source(kind=S.SHM_SRC_FBM, octaves=6, keys=keys)
+        t[N] = best_us(lambda: S.build_lut(lut, src)) / (N + 2) ** 2
+    assert t[48] <= 1.2 * t[46], t
+
+
+@pytest.mark.parametrize("N", [47, 62, 64, 65])
+def test_fbm_whole_and_cut_faces_agree(S, N):
+    """Many glyphs keep faces of up to 66 texels whole, few cut them into equal regions: the same records bit for
+    bit (every octave's frequency is a power of two, so boxed and hashed octaves round alike)."""
+    src = S.Source(kind=S.SHM_SRC_FBM, octaves=7, keys=torch.from_numpy(I.fbm_keys(7, 7).view(np.int32)).cuda())
+    one, many = S.alloc_lut(1, N), S.alloc_lut(60, N)
+    S.build_lut(one, src)
+    S.build_lut(many, src)
+    assert torch.isfinite(one.data).all()
+    assert torch.equal(many.data.view(60, -1), one.data.expand(60, -1))
