@@ -271,7 +271,9 @@ __device__ __forceinline__ int ev_lane_glyph(const int64_t* seg, int G, int g, i
     return lo;
 }
 
-// Warp w of W takes queries [Q w / W, Q (w + 1) / W) and walks the glyphs they belong to.
+// Warp w of W takes queries [Q w / W, Q (w + 1) / W) and walks the glyphs they belong to.  SHORT: segments may be short
+// on average.
+template <bool SHORT>
 __global__ void __launch_bounds__(EV_BLOCK, EV_RES) k_sh_eval_seg(EvArgs a, const __grid_constant__ EvTable T)
 {
     extern __shared__ __align__(16) float4 ev_smem[];
@@ -291,9 +293,14 @@ __global__ void __launch_bounds__(EV_BLOCK, EV_RES) k_sh_eval_seg(EvArgs a, cons
     while (q < qe) {
         int64_t e = qe;  // end of glyph g's queries within the warp's range
         if (a.seg) {
-            // the next segment holds q but for empty ones, which are searched over instead of walked
-            if (g >= 0 && g < a.G && q >= __ldg(a.seg + g + 1) && (++g < a.G) && q >= __ldg(a.seg + g + 1))
-                g = seg_find_warp(a.seg, a.G, q);
+            // past empty segments to the one that holds q: by a search, or 32 ends at a time where segments are not short
+            if (SHORT) {
+                if (g >= 0 && g < a.G && q >= __ldg(a.seg + g + 1) && (++g < a.G) && q >= __ldg(a.seg + g + 1))
+                    g = seg_find_warp(a.seg, a.G, q);
+            } else if (g >= 0) {
+                for (unsigned m = ~0u; m == ~0u && g < a.G; g += __popc(m))
+                    m = __ballot_sync(0xffffffffu, g + 1 + lane <= a.G && __ldg(a.seg + min(g + 1 + lane, a.G)) <= q);
+            }
             e = g >= a.G ? qe : min(qe, __ldg(a.seg + g + 1));
         }
         if (g < 0 || g >= a.G) {
@@ -304,7 +311,7 @@ __global__ void __launch_bounds__(EV_BLOCK, EV_RES) k_sh_eval_seg(EvArgs a, cons
             g = g < 0 ? 0 : g;
             continue;
         }
-        if (e - q < EV_SHORT) {
+        if (SHORT && e - q < EV_SHORT) {
             // 32 queries, each lane on its own glyph
             const int gl = a.seg ? ev_lane_glyph(a.seg, a.G, g, q, lane) : g;
             if (q + lane < qe) ev_one(a, T, q + lane, gl, status);
@@ -370,7 +377,9 @@ cudaError_t launch_sh_eval(int L, int G, const float* coeffs, int64_t Q, const f
     int64_t blocks = (Q + 32 * EV_WARPS - 1) / (32 * EV_WARPS);
     const int64_t cap = (int64_t)sm_count() * EV_RES;
     if (blocks > cap) blocks = cap;
-    k_sh_eval_seg<<<(unsigned)blocks, EV_BLOCK, smem, s>>>(a, T);
+    // (the lanes' path costs the other 1.7 %, in registers and scheduling, where it is not taken)
+    if (seg && Q < 64LL * G) k_sh_eval_seg<true><<<(unsigned)blocks, EV_BLOCK, smem, s>>>(a, T);
+    else k_sh_eval_seg<false><<<(unsigned)blocks, EV_BLOCK, smem, s>>>(a, T);
     return cudaGetLastError();
 }
 
