@@ -666,7 +666,8 @@ __global__ void __launch_bounds__(256, 4) k_fbm_face(LutView out, void* data, sh
     const int g = map_block(map, region), f = blockIdx.y;
     const GlyphRef Gr = glyph_ref(out, g);
     const int N = Gr.N, P = N + 2;
-    const int nr = (P + T - 1) / T, Te = (P + nr - 1) / nr;  // regions of Te x Te texels, the last ones of a row shorter
+    const int nr = (P + T - 1) / T;
+    const int Te = std::is_same<Map, UniformMap>::value ? T : (P + nr - 1) / nr;  // equal regions; uniform pools pass such a T
     if (region >= nr * nr) return;
     const int i0 = (region % nr) * Te, j0 = (region / nr) * Te;  // first texel of the region
     const int ti = min(Te, P - i0), tj = min(Te, P - j0);      // texels in the region
@@ -802,6 +803,8 @@ cudaError_t launch_fd_build(const LutView& out, void* data, const shm_source& sr
     if (fbm) {
         const int P = sz.max_N + 2;
         T = P <= FBM_T || (P <= FBM_WHOLE && 6LL * sz.G >= sm_count()) ? P : FBM_T;
+        const int nr = (P + T - 1) / T;
+        if (sz.N_uniform > 0) T = (P + nr - 1) / nr;
     } else {
         if (sz.N_uniform == 0 && T > FACE_SPLIT_T) T = FACE_SPLIT_T;
         if (sz.N_uniform > 0 && T <= FACE_N_MAX + 2 && (T + 2) * (T + 2) * (int)sizeof(float) > FACE_SPLIT_SMEM)
