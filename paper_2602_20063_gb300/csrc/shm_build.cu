@@ -1048,15 +1048,24 @@ cudaError_t launch_bounds(const LutView& L, float* rmax, const Sizes& sz, cudaSt
     cudaError_t e = cudaMemsetAsync(rmax, 0, sizeof(float) * (size_t)L.n_glyphs, s);
     if (e != cudaSuccess) return e;
     constexpr int T = 32 * BOUNDS_WARPS;
-    // a pool's glyphs of either kind in a launch of their own
-    const bool strips = L.dtype == SHM_F32 && L.layout == SHM_LAYOUT_TEXEL;
-    const auto by_strips = [strips](int N) { return strips && N >= BOUNDS_STRIP_N; };
-    if (by_strips(sz.max_N)) {
+    // A pool's glyphs of either kind in a launch of their own (one kernel with both forms has the strips' 64 registers and
+    // took 89 us where two launches take 80, for 128 each of N = 16, 32, 64, 128); where faces below N = 48 hold at most an
+    // eighth of the texels, strips for all (77).
+    const bool strips = L.dtype == SHM_F32 && L.layout == SHM_LAYOUT_TEXEL && sz.max_N >= BOUNDS_STRIP_N;
+    int64_t small = 0, all = 0;
+    for (int g = 0; strips && sz.N_host && g < sz.G; ++g) {
+        const int64_t texels = (int64_t)(sz.N_host[g] + 2) * (sz.N_host[g] + 2);
+        all += texels;
+        small += sz.N_host[g] < 48 ? texels : 0;
+    }
+    const int least = sz.N_host && 8 * small <= all ? 1 : BOUNDS_STRIP_N;
+    const auto by_strips = [=](int N) { return strips && N >= least; };
+    if (strips) {
         const auto blocks = [&](int N) { return by_strips(N) ? (BoundsUnits(N).count() + BOUNDS_WARPS - 1) / BOUNDS_WARPS : 0; };
         e = for_each_glyph_chunk(sz, blocks, [&](unsigned bx, unsigned bz, const auto& map) {
             k_bounds_strips<<<dim3(bx, 1, bz), T, 0, s>>>(L, rmax, map);
         });
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || least == 1 || sz.N_uniform > 0) return e;
     }
     const auto blocks = [&](int N) { return by_strips(N) ? 0 : (6LL * (N + 1) * (N + 1) + BOUNDS_CELLS - 1) / BOUNDS_CELLS; };
     return for_each_glyph_chunk(sz, blocks, [&](unsigned bx, unsigned bz, const auto& map) {

@@ -404,7 +404,8 @@ def test_bounds_large_and_mixed(S, dtype, layout):
             at += n
             assert abs(x - ref) <= 4 * 2.0 ** -24 * ref, (Ns[i], x, ref)
 
-    pool(range(len(Ns)))
+    pool(range(len(Ns)))    # few texels in small faces: one form for all
+    pool([1, 2, 3, 5])      # many: each glyph its own
     for i in range(len(Ns)):
         pool([i, i])
 
