@@ -27,11 +27,15 @@ constexpr QShape QSHAPES[N_QSHAPES] = {{512, 8}, {256, 16}, {1024, 4}, {256, 8}}
 // Work is handed out per CTA in contiguous chunks (up to 4,096 queries by default), so that for
 // per-glyph query segments a CTA serves whole glyphs and the glyph's table stays in that SM's L1 (two
 // CTAs per SM keep two tables of up to ~110 KB resident) instead of being pulled into several SMs.
-// Without segments, and where a glyph has many chunks of queries, there is no glyph to keep: chunks of
-// one round up to CHUNK_WAVES chunks per CTA, longer ones above.  A small batch then spreads over every
-// SM (65,536 queries: 128 CTAs instead of 16, kernel 18 -> 5 us), a middling one has no last wave of
-// eight rounds (planet view, f16 cells, 4.6 M queries: 71 -> 60 us), and a large one keeps the longer
-// runs of neighbouring queries.
+// Without segments there is no glyph to keep.  Chunks of one round then spread a small batch over every SM
+// (65,536 queries: 128 CTAs instead of 16, kernel 18 -> 5 us) and spare a middling one its last wave of eight
+// rounds (4K planet view, 2.7 M queries in f32 texels / f16 cells: 68 / 70 us in long chunks, 58 / 60 so; 8K view 202 /
+// 206 and 193 / 198).  Long chunks keep a large one's CTAs on longer runs of addresses: above SHORT_ROUNDS rounds a
+// CTA, 2^26 random queries take 1,150 us long and 1,201 short at N = 64, 3,199 and 3,298 at N = 2048.  Long and
+// one-round loops are instantiations of their own: one loop with the round count at run time spilled and
+// took 1,222 us for the former.
+// Segments: chunks no longer than keeps every CTA busy where glyphs are short, and SEG_WAVES chunks per CTA where a
+// glyph has many (64 glyphs of 20,391 queries, N = 47: 35 us in chunks of eight rounds, 29 to 32 so).
 //
 // VEC (all of dirs / grad / normal 16-byte aligned): for a full warp round (32 queries) the 384 B
 // of directions are read with 24 128-bit loads and the 384 B of gradients and of normals are
@@ -45,9 +49,12 @@ struct QueryOccupancy {
     static constexpr int min_blocks = (RECON >= SHM_RECON_BICUBIC) ? 1 : (QBLOCK >= 1024 ? 1 : 1024 / QBLOCK);
 };
 
-template <int DT, int LAYOUT, bool VEC, int RECON, int QBLOCK = 512>
+// QIT: rounds of QBLOCK queries per chunk (0: `rounds`).  The next round's directions load under this round's
+// table fetch: those of the same chunk, or of the CTA's next one where chunks are one round (QIT == 1).
+template <int DT, int LAYOUT, bool VEC, int RECON, int QBLOCK = 512, int QIT = 8>
 __global__ void __launch_bounds__(QBLOCK, (QueryOccupancy<RECON, QBLOCK>::min_blocks)) k_query_fwd(QueryArgs a, int rounds)
 {
+    if (QIT > 0) rounds = QIT;
     __shared__ __align__(16) float sbuf[QBLOCK / 32][96];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* wb = sbuf[warp];
@@ -55,16 +62,12 @@ __global__ void __launch_bounds__(QBLOCK, (QueryOccupancy<RECON, QBLOCK>::min_bl
     uint32_t status = 0;
     const float qnan = __int_as_float(0x7fc00000);
     const float4* dirs4 = reinterpret_cast<const float4*>(a.dirs);
+    const int64_t step = (int64_t)gridDim.x * QBLOCK * rounds;
 
-    // round i of the chunk at c0; the next round (of this chunk or of the CTA's next one) is known one
-    // round ahead, so its directions are always loaded under this round's table fetch
-    int64_t c0 = (int64_t)blockIdx.x * QBLOCK * rounds;
-    int64_t qw = c0 + warp * 32;
-    int i = 0;
-    // glyph of this lane's first query and the end of its segment (one search per warp and chunk)
+    // glyph of this lane's first query and the end of its segment
     int g = 0;
     int64_t seg_end = a.seg ? INT64_MIN : INT64_MAX;
-    // direction of the first round: vector (full round) or scalar
+    // directions of the coming round: vector (full round) or scalar
     float4 pv = make_float4(0.f, 0.f, 0.f, 0.f);
     float n0 = 0.f, n1 = 0.f, n2 = 0.f;
     const auto load_dirs = [&](int64_t qn) {
@@ -76,128 +79,149 @@ __global__ void __launch_bounds__(QBLOCK, (QueryOccupancy<RECON, QBLOCK>::min_bl
             n2 = __ldcs(a.dirs + 3 * (qn + lane) + 2);
         }
     };
-    load_dirs(qw);
+    int64_t c0 = (int64_t)blockIdx.x * QBLOCK * rounds;
+    if (QIT == 1) load_dirs(c0 + warp * 32);
 #pragma unroll 1
-    while (qw < a.Q) {
-        // a chunk that goes on in the same segment needs no search
-        if (a.seg && i == 0 && __any_sync(0xffffffffu, qw + lane >= seg_end || g < 0)) {
-            g = (qw < __ldg(a.seg)) ? -1 : seg_find_warp(a.seg, G, qw);
+    for (; c0 + warp * 32 < a.Q; c0 += step) {
+        const int64_t qw0 = c0 + warp * 32;
+        // one search per warp and chunk; a chunk that goes on in the same segment needs none
+        if (a.seg && __any_sync(0xffffffffu, qw0 + lane >= seg_end || g < 0)) {
+            g = (qw0 < __ldg(a.seg)) ? -1 : seg_find_warp(a.seg, G, qw0);
             seg_end = (g >= 0 && g < G) ? __ldg(a.seg + g + 1) : 0;
         }
-        int64_t qn = qw + QBLOCK;
-        if (++i == rounds) {
-            i = 0;
-            c0 += (int64_t)gridDim.x * QBLOCK * rounds;
-            qn = c0 + warp * 32;
-        }
-        const bool full = VEC && (qw + 32 <= a.Q);
-        const int64_t q = qw + lane;
-        float d0, d1, d2;
-        if (full) {
-            // re-distribute the warp's 24 float4 of directions: lane L takes floats 3L..3L+2
-            if (lane < 24) reinterpret_cast<float4*>(wb)[lane] = pv;
-            __syncwarp();
-            d0 = wb[3 * lane]; d1 = wb[3 * lane + 1]; d2 = wb[3 * lane + 2];
-            __syncwarp();
-        } else {
-            if (q >= a.Q) break;
-            d0 = n0; d1 = n1; d2 = n2;
-        }
-        load_dirs(qn);
-        int gq = 0;
-        if (a.glyph) {
-            gq = __ldg(a.glyph + q);
-        } else if (a.seg) {
-            if (q >= seg_end || g < 0) {
-                if (g < 0 && q >= __ldg(a.seg)) g = 0;
-                while (g >= 0 && g < G && q >= __ldg(a.seg + g + 1)) ++g;
-                seg_end = (g >= 0 && g < G) ? __ldg(a.seg + g + 1) : INT64_MAX;
-            }
-            gq = g;
-        }
-        bool valid = true;
-        if (gq < 0 || gq >= G) { valid = false; status |= SHM_DEV_BOUNDS; }
-        QueryResult r;
-        Chart c;
-        if (valid) {
-            const GlyphRef Gr = glyph_ref(a.L, gq);
-            if constexpr (RECON < 0) valid = query_one<DT, LAYOUT>(a.L, Gr, d0, d1, d2, r, c);
-            else valid = recon_one<RECON, DT>(a.L, Gr, d0, d1, d2, r, c);
-            if (!valid) status |= SHM_DEV_NONFINITE;
-        }
-        if (!valid) {
-            r.R = r.Ru = r.Rv = qnan;
-            r.grad = Vec3{qnan, qnan, qnan};
-            r.f = r.i = r.j = -1;
-        }
-        const Vec3 n = (a.normal && valid) ? surface_normal(d0, d1, d2, r.R, r.grad) : Vec3{qnan, qnan, qnan};
-        if (a.R) __stcs(a.R + q, r.R);
-        if (full) {
-            if (a.grad) {
-                wb[3 * lane] = r.grad.x; wb[3 * lane + 1] = r.grad.y; wb[3 * lane + 2] = r.grad.z;
+        if (QIT != 1) load_dirs(qw0);
+#pragma unroll 1
+        for (int it = 0; it < rounds; ++it) {
+            const int64_t qw = qw0 + (int64_t)it * QBLOCK;
+            if (QIT != 1 && qw >= a.Q) break;
+            const bool full = VEC && (qw + 32 <= a.Q);
+            const int64_t q = qw + lane;
+            float d0, d1, d2;
+            if (full) {
+                // re-distribute the warp's 24 float4 of directions: lane L takes floats 3L..3L+2
+                if (lane < 24) reinterpret_cast<float4*>(wb)[lane] = pv;
                 __syncwarp();
-                if (lane < 24) __stcs(reinterpret_cast<float4*>(a.grad) + (3 * qw) / 4 + lane, reinterpret_cast<const float4*>(wb)[lane]);
+                d0 = wb[3 * lane]; d1 = wb[3 * lane + 1]; d2 = wb[3 * lane + 2];
                 __syncwarp();
+            } else {
+                if (q >= a.Q) break;
+                d0 = n0; d1 = n1; d2 = n2;
             }
-            if (a.normal) {
-                wb[3 * lane] = n.x; wb[3 * lane + 1] = n.y; wb[3 * lane + 2] = n.z;
-                __syncwarp();
-                if (lane < 24) __stcs(reinterpret_cast<float4*>(a.normal) + (3 * qw) / 4 + lane, reinterpret_cast<const float4*>(wb)[lane]);
-                __syncwarp();
+            // the next round's directions: their latency overlaps the table fetch below
+            if (QIT == 1) load_dirs(qw + step);
+            else if (it + 1 < rounds) load_dirs(qw + QBLOCK);
+            int gq = 0;
+            if (a.glyph) {
+                gq = __ldg(a.glyph + q);
+            } else if (a.seg) {
+                if (q >= seg_end || g < 0) {
+                    if (g < 0 && q >= __ldg(a.seg)) g = 0;
+                    while (g >= 0 && g < G && q >= __ldg(a.seg + g + 1)) ++g;
+                    seg_end = (g >= 0 && g < G) ? __ldg(a.seg + g + 1) : INT64_MAX;
+                }
+                gq = g;
             }
-        } else {
-            if (a.grad) {
-                a.grad[3 * q] = r.grad.x;
-                a.grad[3 * q + 1] = r.grad.y;
-                a.grad[3 * q + 2] = r.grad.z;
+            bool valid = true;
+            if (gq < 0 || gq >= G) { valid = false; status |= SHM_DEV_BOUNDS; }
+            QueryResult r;
+            Chart c;
+            if (valid) {
+                const GlyphRef Gr = glyph_ref(a.L, gq);
+                if constexpr (RECON < 0) valid = query_one<DT, LAYOUT>(a.L, Gr, d0, d1, d2, r, c);
+                else valid = recon_one<RECON, DT>(a.L, Gr, d0, d1, d2, r, c);
+                if (!valid) status |= SHM_DEV_NONFINITE;
             }
-            if (a.normal) {
-                a.normal[3 * q] = n.x;
-                a.normal[3 * q + 1] = n.y;
-                a.normal[3 * q + 2] = n.z;
+            if (!valid) {
+                r.R = r.Ru = r.Rv = qnan;
+                r.grad = Vec3{qnan, qnan, qnan};
+                r.f = r.i = r.j = -1;
+            }
+            const Vec3 n = (a.normal && valid) ? surface_normal(d0, d1, d2, r.R, r.grad) : Vec3{qnan, qnan, qnan};
+            if (a.R) __stcs(a.R + q, r.R);
+            if (full) {
+                if (a.grad) {
+                    wb[3 * lane] = r.grad.x; wb[3 * lane + 1] = r.grad.y; wb[3 * lane + 2] = r.grad.z;
+                    __syncwarp();
+                    if (lane < 24) __stcs(reinterpret_cast<float4*>(a.grad) + (3 * qw) / 4 + lane, reinterpret_cast<const float4*>(wb)[lane]);
+                    __syncwarp();
+                }
+                if (a.normal) {
+                    wb[3 * lane] = n.x; wb[3 * lane + 1] = n.y; wb[3 * lane + 2] = n.z;
+                    __syncwarp();
+                    if (lane < 24) __stcs(reinterpret_cast<float4*>(a.normal) + (3 * qw) / 4 + lane, reinterpret_cast<const float4*>(wb)[lane]);
+                    __syncwarp();
+                }
+            } else {
+                if (a.grad) {
+                    a.grad[3 * q] = r.grad.x;
+                    a.grad[3 * q + 1] = r.grad.y;
+                    a.grad[3 * q + 2] = r.grad.z;
+                }
+                if (a.normal) {
+                    a.normal[3 * q] = n.x;
+                    a.normal[3 * q + 1] = n.y;
+                    a.normal[3 * q + 2] = n.z;
+                }
+            }
+            if (a.chart) {
+                a.chart[2 * q] = r.Ru;
+                a.chart[2 * q + 1] = r.Rv;
+            }
+            if (a.fij) {
+                a.fij[3 * q] = r.f;
+                a.fij[3 * q + 1] = r.i;
+                a.fij[3 * q + 2] = r.j;
             }
         }
-        if (a.chart) {
-            a.chart[2 * q] = r.Ru;
-            a.chart[2 * q + 1] = r.Rv;
-        }
-        if (a.fij) {
-            a.fij[3 * q] = r.f;
-            a.fij[3 * q + 1] = r.i;
-            a.fij[3 * q + 2] = r.j;
-        }
-        qw = qn;
     }
     report_status(a.dev_status, status);
 }
 
-// chunks per CTA below which chunks get shorter (f32, start of the range to its end: 4K planet view 68 -> 58
-// us; 64 glyphs of 20,391 queries, N = 47, 40 -> 31; 25 of 179,818, N = 30 in cells, 83.3 -> 82.1)
-constexpr int CHUNK_WAVES = 16, SEG_WAVES = 4;
-constexpr int64_t LONG_GLYPH = 16384;  // mean queries per glyph: four chunks of 4,096
+// Rounds per CTA up to which chunks are one round; chunks per CTA that long segments keep; mean queries per glyph of
+// a long segment (four chunks of 4,096).
+constexpr int SHORT_ROUNDS = 96, SEG_WAVES = 4;
+constexpr int64_t LONG_GLYPH = 16384;
 
 template <int DT, int LAYOUT, bool VEC, int RECON, int QBLOCK, int QIT>
-cudaError_t launch_fwd_v(const QueryArgs& a, cudaStream_t s)
+int query_resident()
 {
-    // one persistent wave: SMs x resident blocks per SM
     static int resident = 0;
     if (resident == 0) {
         int r = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK>, QBLOCK,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK, QIT>, QBLOCK,
                                                           0) != cudaSuccess ||
             r < 1)
             r = QueryOccupancy<RECON, QBLOCK>::min_blocks;
         resident = r;
     }
-    const int64_t cap = (int64_t)sm_count() * resident;
-    const int64_t total = (a.Q + QBLOCK - 1) / QBLOCK;
-    const bool short_glyphs = a.seg && a.Q / LONG_GLYPH < a.L.n_glyphs;
-    int64_t rounds = short_glyphs ? (total + cap - 1) / cap : total / ((a.seg ? SEG_WAVES : CHUNK_WAVES) * cap);
-    if (rounds > QIT) rounds = QIT;
-    if (rounds < 1) rounds = 1;
-    int64_t blocks = (total + rounds - 1) / rounds;
-    if (blocks > cap) blocks = cap;
-    k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK><<<(unsigned)blocks, QBLOCK, 0, s>>>(a, (int)rounds);
+    return resident;
+}
+
+template <int DT, int LAYOUT, bool VEC, int RECON, int QBLOCK, int QIT>
+cudaError_t launch_fwd_v(const QueryArgs& a, cudaStream_t s)
+{
+    // one persistent wave: SMs x resident blocks per SM
+    const int64_t cap = (int64_t)sm_count() * query_resident<DT, LAYOUT, VEC, RECON, QBLOCK, QIT>();
+    const int64_t total = (a.Q + QBLOCK - 1) / QBLOCK;  // rounds
+    const auto blocks = [&](int64_t rounds) {
+        const int64_t n = (total + rounds - 1) / rounds;
+        return (unsigned)(n < cap ? n : cap);
+    };
+    if constexpr (!VEC) {
+        if (a.seg) {
+            const bool short_glyphs = a.Q / LONG_GLYPH < a.L.n_glyphs;
+            int64_t rounds = short_glyphs ? (total + cap - 1) / cap : total / (SEG_WAVES * cap);
+            if (rounds < 1) rounds = 1;
+            if (rounds < QIT) {
+                k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK, 0><<<blocks(rounds), QBLOCK, 0, s>>>(a, (int)rounds);
+                return cudaGetLastError();
+            }
+        }
+    }
+    if (!a.seg && total <= SHORT_ROUNDS * cap)
+        k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK, 1><<<blocks(1), QBLOCK, 0, s>>>(a, 1);
+    else
+        k_query_fwd<DT, LAYOUT, VEC, RECON, QBLOCK, QIT><<<blocks(QIT), QBLOCK, 0, s>>>(a, QIT);
     return cudaGetLastError();
 }
 

@@ -232,3 +232,35 @@ def test_staged_glyph_field_size(S):
     b = S.query(lut, dirs, glyph=glyph, want=("R", "grad", "normal", "fij"))
     for k in a:
         assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("which", ["tiny", "short", "limit", "long"])
+@pytest.mark.parametrize("layout", [0, 1])
+def test_launch_forms_agree(S, which, layout):
+    """The per-query kernel's forms (chunks of one round, of eight, of a count set at run time for segments)
+    give the same bits: batches on both sides of the line between short and long chunks (96 rounds of 512
+    queries for each of two CTAs per SM) and much smaller ones, without selection, with ids and with one
+    segment that leaves queries on both sides outside; aligned and unaligned buffers, ragged ends."""
+    line = 96 * 2 * torch.cuda.get_device_properties(0).multi_processor_count * 512
+    Q = {"tiny": 77, "short": 200003, "limit": line, "long": line + 4801}[which]
+    N = 47 if layout == 0 else 9  # tables that a segment does not stage
+    g = torch.Generator(device="cuda").manual_seed(Q)
+    lut = S.alloc_lut(1, N, 0, layout, r0=[0.25])
+    lut.data.copy_(1.0 + 0.1 * torch.randn(lut.data.shape, generator=g, device="cuda"))
+    d = torch.nn.functional.normalize(torch.randn((Q, 3), generator=g, device="cuda"), dim=1)
+    d[Q // 2] = 0.0
+    want = ("R", "grad", "normal")
+    ref = S.query(lut, d, want=want)
+    same = lambda a, b: torch.equal(a.view(torch.int32), b.view(torch.int32))
+    shifted = torch.empty(3 * Q + 1, device="cuda")[1:].view(Q, 3).copy_(d)
+    out = S.query(lut, shifted, want=want)
+    assert all(same(ref[k], out[k]) for k in want)
+    out = S.query(lut, d, glyph=torch.zeros(Q, dtype=torch.int32, device="cuda"), want=want)
+    assert all(same(ref[k], out[k]) for k in want)
+    a, b = 5, Q - 3
+    out = S.query(lut, d, seg=torch.tensor([a, b], device="cuda"), want=want)
+    for k in want:
+        assert same(ref[k][a:b], out[k][a:b]) and torch.isnan(out[k][:a]).all() and torch.isnan(out[k][b:]).all()
+    pick = torch.randint(0, Q, (4096,), generator=g, device="cuda")
+    few = S.query(lut, d[pick].contiguous(), want=want)
+    assert all(same(ref[k][pick], few[k]) for k in want)
