@@ -56,7 +56,6 @@ struct Args {
     LutView view;         // output table (any dtype / layout) for the generic epilogue
     void* data;
     int direct;           // 1: f32 texel layout, uniform N, write out[g*M + c]
-    int twice;            // direct: the same boxes also go to a second table
     int32_t* dev_status;
 };
 
@@ -89,6 +88,8 @@ __device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uin
         : "memory");
 }
 
+// TWICE: the output boxes also go to a second table, mOut2.
+template <bool TWICE>
 __global__ void __launch_bounds__(256, 1)
     k_sh_gemm_tc(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
                  const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl,
@@ -241,7 +242,7 @@ __global__ void __launch_bounds__(256, 1)
                     epi_bar();
                     if (issuer) {
                         tma_store_2d(&mOut, smem_u32(buf), mt * TM, g0);  // clipped at M columns, G rows
-                        if (a.twice) tma_store_2d(&mOut2, smem_u32(buf), mt * TM, g0);
+                        if (TWICE) tma_store_2d(&mOut2, smem_u32(buf), mt * TM, g0);
                         bulk_commit();
                     }
                     ++box;
@@ -357,14 +358,14 @@ cudaError_t launch_sh_build_tc(const LutView& out, void* data, int L, const floa
     a.data = data;
     a.out = reinterpret_cast<float*>(data);
     a.direct = direct ? 1 : 0;
-    a.twice = copy ? 1 : 0;
     a.dev_status = dev_status;
-    e = ensure_dynamic_smem((const void*)tc::k_sh_gemm_tc, (int)tc::SMEM_BYTES);
+    const auto kernel = copy ? tc::k_sh_gemm_tc<true> : tc::k_sh_gemm_tc<false>;
+    e = ensure_dynamic_smem((const void*)kernel, (int)tc::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     const int tiles = ((M + tc::TM - 1) / tc::TM) * ((G + tc::TN - 1) / tc::TN);
     int grid = sm_count();
     if (grid > tiles) grid = tiles;
-    tc::k_sh_gemm_tc<<<grid, 256, tc::SMEM_BYTES, s>>>(mAh, mAl, mBh, mBl, mOut, mOut2, a);
+    kernel<<<grid, 256, tc::SMEM_BYTES, s>>>(mAh, mAl, mBh, mBl, mOut, mOut2, a);
     return cudaGetLastError();
 }
 
