@@ -211,3 +211,42 @@ def test_bake_snapshot_and_gradient_in_place(G, N):
         assert torch.equal(dense, torch.autograd.grad(t0, c[0], other, retain_graph=True)[0])
     ones = torch.autograd.grad(t0.sum(), c[0], retain_graph=True)[0]
     assert torch.equal(ones, torch.autograd.grad(t0, c[0], torch.ones_like(g))[0])
+
+
+def test_first_call_of_a_thread_takes_the_tensor_cores():
+    """The driver's tensor-map call needs a context on its thread, which one that has made no runtime call yet (an
+    autograd worker) lacks: there too the bake and its adjoint give the tensor cores' bits, not the CUDA cores'."""
+    import threading
+    S = shm()
+    G, N, L = 200, 20, 6
+    g = torch.Generator(device="cuda").manual_seed(1)
+    basis = S.sh_basis(N, L)
+    src = S.Source(kind=S.SHM_SRC_SH, L=L, coeffs=torch.randn((G, (L + 1) ** 2), generator=g, device="cuda"), basis=basis)
+    lut, D = S.alloc_lut(G, N), S.alloc_lut(G, N)
+    D.data.copy_(torch.randn(D.data.shape, generator=g, device="cuda"))
+    ws = S.build_workspace(lut, src)
+    s = torch.cuda.current_stream()
+    dc = torch.empty((G, (L + 1) ** 2), device="cuda")
+    S.build_lut(lut, src, ws=ws)
+    table, ref, other = lut.data.clone(), S.build_lut_backward(D, L, basis), S.build_lut_backward(D, L, basis, cuda_cores=True)
+    S.build_lut(lut, src)
+    assert not torch.equal(lut.data, table) and not torch.equal(ref, other)
+    errors = []
+
+    def run(fn):
+        def body():
+            try:
+                fn()
+            except Exception as e:  # noqa: BLE001
+                errors.append(e)
+        t = threading.Thread(target=body)
+        t.start()
+        t.join()
+
+    lut.data.zero_()
+    torch.cuda.synchronize()
+    run(lambda: S.build_lut(lut, src, ws=ws, stream=s))
+    run(lambda: S.build_lut_backward(D, L, basis, stream=s, out=dc))
+    torch.cuda.synchronize()
+    assert not errors, errors
+    assert torch.equal(lut.data, table) and torch.equal(dc, ref)
