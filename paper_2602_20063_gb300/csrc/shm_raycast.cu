@@ -103,28 +103,51 @@ __device__ __forceinline__ uint32_t pack_tiles(bool on, int x0, int x1, int y0, 
 
 __host__ __device__ __forceinline__ bool tiles_fit_bytes(int W, int H) { return W <= 256 * RT && H <= 256 * RT; }
 
-// Front-to-back rank of every object, one warp per object: its lanes count the keys before it.  The
-// object's tile rectangle goes with it, so that the tiles do not work it out again (8,160 tiles by 512
-// objects: k_bin_tiles 27 -> 12.5 us; this kernel, a thread per object before, 9 -> 7.5 us).
-__global__ void __launch_bounds__(RANK_BLOCK) k_rank_objects(const shm_object* __restrict__ objs, int n, shm_camera cam,
-                                                             int32_t* order, uint32_t* rects)
+// Front-to-back rank of every object: its lanes count the keys before it.  The object's tile rectangle goes with
+// it, so that the tiles do not work it out again (8,160 tiles by 512 objects: k_bin_tiles 27 -> 12.5 us; this kernel,
+// a thread per object before, 9 -> 7.5 us).  Up to RANK_DIRECT objects a warp ranks one and forms the others' keys
+// itself; beyond, where n^2 records of 24 bytes no longer come from L1, the keys are formed once (k_rank_keys, into
+// the region of the tiles' lists, which are written later) and a warp ranks RANK_OBJS objects per reading of them.
+constexpr int RANK_DIRECT = 4096, RANK_OBJS = 4;
+
+__global__ void __launch_bounds__(RANK_BLOCK) k_rank_keys(const shm_object* __restrict__ objs, int n, shm_camera cam, float* keys)
 {
-    const int i = (int)(((int64_t)blockIdx.x * RANK_BLOCK + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (i >= n) return;  // warp-uniform
-    const shm_object o = objs[i];
-    const float ki = rank_key(o, cam);
-    int rank = 0;
-    for (int j = lane; j < n; j += 32) {
-        const float kj = rank_key(objs[j], cam);
-        rank += (kj < ki) || (kj == ki && j < i);
+    const int i = blockIdx.x * RANK_BLOCK + threadIdx.x;
+    if (i < n) keys[i] = rank_key(objs[i], cam);
+}
+
+template <bool KEYS>
+__global__ void __launch_bounds__(RANK_BLOCK) k_rank_objects(const shm_object* __restrict__ objs, int n, shm_camera cam,
+                                                             const float* keys, int32_t* order, uint32_t* rects)
+{
+    constexpr int M = KEYS ? RANK_OBJS : 1;
+    const int64_t first = (((int64_t)blockIdx.x * RANK_BLOCK + threadIdx.x) >> 5) * M;
+    const int lane = threadIdx.x & 31;
+    if (first >= n) return;  // warp-uniform
+    const int i0 = (int)first;
+    const auto key = [&](int j) { return KEYS ? keys[j] : rank_key(objs[j], cam); };
+    float ki[M];
+    int rank[M];
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        ki[m] = key(min(i0 + m, n - 1));
+        rank[m] = 0;
     }
-    rank = __reduce_add_sync(0xffffffffu, rank);
-    if (lane == 0) {
-        order[rank] = i;
+#pragma unroll KEYS ? 4 : 1
+    for (int j = lane; j < n; j += 32) {
+        const float kj = key(j);
+#pragma unroll
+        for (int m = 0; m < M; ++m) rank[m] += (kj < ki[m]) || (kj == ki[m] && j < i0 + m);
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        const int i = i0 + m, r = __reduce_add_sync(0xffffffffu, rank[m]);
+        if (lane != m || i >= n) continue;
+        order[r] = i;
         if (tiles_fit_bytes(cam.W, cam.H)) {
             int x0 = 0, x1 = 0, y0 = 0, y1 = 0;
-            const bool on = sphere_rect(o, cam, x0, x1, y0, y1);
-            rects[rank] = pack_tiles(on, x0, x1, y0, y1);
+            const bool on = sphere_rect(objs[i], cam, x0, x1, y0, y1);
+            rects[r] = pack_tiles(on, x0, x1, y0, y1);
         }
     }
 }
@@ -443,8 +466,16 @@ cudaError_t launch_raycast(const LutView& L, const shm_object* objs, int n_obj, 
     if (e != cudaSuccess) return e;
     if (n_obj > 0) {
         uint32_t* rects = (uint32_t*)(base + w.rect_off);
-        k_rank_objects<<<(unsigned)(((int64_t)n_obj * 32 + RANK_BLOCK - 1) / RANK_BLOCK), RANK_BLOCK, 0, s>>>(objs, n_obj, cam,
-                                                                                                           order, rects);
+        if (n_obj <= RANK_DIRECT) {
+            k_rank_objects<false><<<(unsigned)(((int64_t)n_obj * 32 + RANK_BLOCK - 1) / RANK_BLOCK), RANK_BLOCK, 0, s>>>(
+                objs, n_obj, cam, nullptr, order, rects);
+        } else {
+            float* keys = reinterpret_cast<float*>(lists);  // 4 n_obj bytes at least: a list of n_obj entries per tile
+            k_rank_keys<<<(unsigned)((n_obj + RANK_BLOCK - 1) / RANK_BLOCK), RANK_BLOCK, 0, s>>>(objs, n_obj, cam, keys);
+            const int64_t warps = ((int64_t)n_obj + RANK_OBJS - 1) / RANK_OBJS;
+            k_rank_objects<true><<<(unsigned)((warps * 32 + RANK_BLOCK - 1) / RANK_BLOCK), RANK_BLOCK, 0, s>>>(
+                objs, n_obj, cam, keys, order, rects);
+        }
         k_bin_tiles<<<(unsigned)(((int64_t)tiles * 32 + 255) / 256), 256, 0, s>>>(objs, n_obj, cam, order, rects, counts,
                                                                                    lists);
     } else {

@@ -252,3 +252,61 @@ def test_value_only_raycast_rejects_unknown_method(S):
     eye, fwd, right, up = camera_frame((0.0, 0.0, 4.0))
     with pytest.raises(S.ShmError, match="invalid"):
         S.raycast(L, objs, 1, S.make_camera(eye, fwd, right, up, 40.0, 16, 16), S.make_raycast_params(recon=7))
+
+
+def _frame(S, centres, W, H, eye=(0.0, 0.0, 40.0), fov=40.0):
+    lut = S.alloc_lut(1, 8, r0=[1.0], zero=True)
+    n = len(centres)
+    e, fwd, right, up = camera_frame(eye)
+    return S.raycast(lut, S.objects_tensor(centres, np.ones(n), np.ones(n), np.zeros(n, int)), n,
+                     S.make_camera(e, fwd, right, up, fov, W, H), S.make_raycast_params())
+
+
+@pytest.mark.parametrize("n", [4096, 4097, 9001])
+def test_many_objects_in_depth_order(S, n):
+    """Up to 4,096 objects each warp forms the keys it ranks against, beyond they are formed once: overlapping
+    spheres at many depths (equal ones among them: the lower index is in front) between objects behind the
+    camera give the frame of the visible ones alone."""
+    rng = np.random.default_rng(n)
+    seen = np.sort(rng.choice(n, 300, replace=False))
+    near = np.stack([rng.uniform(-9, 9, 300), rng.uniform(-6, 6, 300), np.round(rng.uniform(-9, 9, 300), 0)], 1)
+    near[7] = near[3]  # the same sphere twice
+    centres = np.tile([0.0, 0.0, 900.0], (n, 1)) + rng.uniform(-50, 50, (n, 3))
+    centres[seen] = near
+    full, part = _frame(S, centres, 320, 200), _frame(S, near, 320, 200)
+    ids = part["obj_id"].long()
+    assert (ids >= 0).float().mean() > 0.2
+    mapped = torch.where(ids >= 0, torch.from_numpy(seen).cuda()[ids.clamp(min=0)], ids)
+    assert torch.equal(full["obj_id"].long(), mapped)
+    for k in ("rgba", "depth", "normal"):
+        assert torch.equal(full[k].view(torch.int32), part[k].view(torch.int32)), k
+
+
+def test_image_wider_than_packed_tiles(S):
+    """Above 4,096 pixels a side the tiles work out the objects' rectangles themselves: bump objects across an
+    image of 4,300 x 32, sampled pixels against the oracle, bars of the full-size grid."""
+    n, W, H, fov = 8, 4300, 32, 0.5
+    luts, Ns = _scene(n, 320)
+    centres = np.stack([np.linspace(-4.2, 4.2, n), 0.3 * np.sin(np.arange(n)), np.linspace(-0.5, 0.5, n)], 1)
+    r0 = np.ones(n, np.float32)
+    L, stored = upload_pool(S, luts, r0=r0)
+    rmax = S.lut_bounds(L).cpu().numpy()
+    eye, fwd, right, up = camera_frame((0.0, 0.0, 8.0))
+    out = S.raycast(L, S.objects_tensor(centres, 0.5 * np.ones(n), 0.5 * rmax, np.arange(n)), n,
+                    S.make_camera(eye, fwd, right, up, fov, W, H), S.make_raycast_params())
+    rng = np.random.default_rng(5)
+    px, py = rng.integers(0, W, 400).astype(np.int32), rng.integers(0, H, 400).astype(np.int32)
+    pool = stored.reshape(-1, 4)
+    off, Nn = O.make_pool(luts)[1:]
+    rmax_o = np.array([O.lut_bound(pool[off[k]:off[k] + 6 * (Nn[k] + 2) ** 2].reshape(6, Nn[k] + 2, Nn[k] + 2, 4),
+                                   int(Nn[k]), 1.0) for k in range(n)]) * 0.5
+    ref = O.raycast(pool, off, Nn, centres, 0.5 * np.ones(n), rmax_o, np.arange(n),
+                    O.make_camera(eye, fwd, right, up, fov, W, H), O.make_raycast_params(), px=px, py=py,
+                    r0=r0.astype(np.float64))
+    ids = out["obj_id"].cpu().numpy()[py, px]
+    depth = out["depth"].double().cpu().numpy()[py, px]
+    amb = ref["margin"] < 1e-4 * rmax_o.max()
+    assert np.all((ids == ref["obj_id"])[~amb])
+    hit = (ids >= 0) & ~amb
+    assert hit.sum() > 50 and (ids < 0).sum() > 20 and len(set(ids[hit])) == n
+    assert (np.abs(depth[hit] - ref["depth"][hit]) / ref["depth"][hit]).max() <= 2e-5
