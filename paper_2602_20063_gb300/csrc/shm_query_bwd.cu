@@ -86,16 +86,25 @@ __device__ __forceinline__ void add_loss(float* loss, float v)
     }
 }
 
-// CTA of the per-query pass, and the most consecutive rounds of 32 queries per warp.  Its warps' queries lie
-// side by side (4,096 of them), so a glyph's records are reused in L1, while all CTAs together still work
-// on few glyphs, whose tables and gradients (836 KB each at N = 64) must stay in L2: fit workload 502 ->
-// 470 us; CTAs of 256 threads 488; a contiguous range of glyphs per CTA 770 to 1,800 (L2 thrashes).
-constexpr int BBLOCK = 1024;
+// CTA of the per-query pass, and the most consecutive rounds of 32 queries per warp.  The fused fit takes CTAs of
+// 1,024 threads, whose warps' queries lie side by side (4,096 of them), so a glyph's records are reused in L1, while
+// all CTAs together still work on few glyphs, whose tables and gradients (836 KB each at N = 64) must stay in L2:
+// fit workload 502 -> 470 us; CTAs of 256 threads 488; a contiguous range of glyphs per CTA 770 to 1,800 (L2
+// thrashes).  Upstream gradients bring 28 B more per query, and there the large CTAs' common pace loses: 256 threads
+// (four CTAs per SM) against 1,024 take 38.8 / 42.7 us for 10^6 queries of one glyph of N = 64, 233.8 / 239.8 for 4,096
+// each of 1,000, 68.4 / 73.7 for 2 M queries of 100 glyphs of N = 32 by ids.
+template <bool FIT>
+struct BwdCta {
+    static constexpr int threads = FIT ? 1024 : 256;
+    static constexpr int resident = FIT ? 1 : 4;
+    static constexpr int per_sm = FIT ? 1 : 8;  // CTAs launched per SM at most
+};
 constexpr int BROUNDS = 4;
 
 template <int DT, int LAYOUT, bool FIT>
-__global__ void __launch_bounds__(BBLOCK, 1) k_query_bwd(BackwardArgs a, int rounds)
+__global__ void __launch_bounds__(BwdCta<FIT>::threads, BwdCta<FIT>::resident) k_query_bwd(BackwardArgs a, int rounds)
 {
+    constexpr int BBLOCK = BwdCta<FIT>::threads;
     float loss_acc = 0.0f;
     const int lane = threadIdx.x & 31;
     const int64_t chunk = 32 * rounds;
@@ -338,17 +347,23 @@ static cudaError_t launch_bwd_staged(const BackwardArgs& a, uint32_t table_bytes
                  : launch_bwd_staged_ft<DT, false, false>(a, table_bytes, s);
 }
 
+template <int DT, int LAYOUT, bool FIT>
+static cudaError_t launch_bwd_f(const BackwardArgs& a, cudaStream_t s)
+{
+    using Cta = BwdCta<FIT>;
+    const int64_t at_once = (int64_t)sm_count() * Cta::resident * Cta::threads, cap = (int64_t)sm_count() * Cta::per_sm;
+    int64_t rounds = (a.Q + at_once - 1) / at_once;  // small batches: every SM first
+    if (rounds > BROUNDS) rounds = BROUNDS;
+    int64_t blocks = (a.Q + Cta::threads * rounds - 1) / (Cta::threads * rounds);
+    if (blocks > cap) blocks = cap;
+    k_query_bwd<DT, LAYOUT, FIT><<<(unsigned)blocks, Cta::threads, 0, s>>>(a, (int)rounds);
+    return cudaGetLastError();
+}
+
 template <int DT, int LAYOUT>
 static cudaError_t launch_bwd_t(const BackwardArgs& a, cudaStream_t s)
 {
-    const int64_t cap = sm_count();
-    int64_t rounds = (a.Q + cap * BBLOCK - 1) / (cap * BBLOCK);  // small batches: every SM first
-    if (rounds > BROUNDS) rounds = BROUNDS;
-    int64_t blocks = (a.Q + BBLOCK * rounds - 1) / (BBLOCK * rounds);
-    if (blocks > cap) blocks = cap;
-    if (a.fit) k_query_bwd<DT, LAYOUT, true><<<(unsigned)blocks, BBLOCK, 0, s>>>(a, (int)rounds);
-    else k_query_bwd<DT, LAYOUT, false><<<(unsigned)blocks, BBLOCK, 0, s>>>(a, (int)rounds);
-    return cudaGetLastError();
+    return a.fit ? launch_bwd_f<DT, LAYOUT, true>(a, s) : launch_bwd_f<DT, LAYOUT, false>(a, s);
 }
 
 cudaError_t launch_query_bwd(const BackwardArgs& a, cudaStream_t s)
