@@ -179,22 +179,25 @@ __device__ __forceinline__ void zero_slab(float4* slab, int records, int tid, in
 
 // Block b zeroes the slab of the glyph that the boundary between units b and b + 1 cuts, unless an
 // earlier boundary cuts it too.
-__global__ void __launch_bounds__(1024) k_zero_cut(const int64_t* seg, int G, int64_t Q, int64_t w, int64_t units,
-                                                   float4* dlut, int records)
+__global__ void __launch_bounds__(1024) k_zero_cut(const __grid_constant__ stage::Path path, float4* dlut, int records)
 {
-    __shared__ int s_g;
-    if (threadIdx.x < 32) {
-        const int64_t D = stage::unit_cost(seg, G, Q, w, blockIdx.x + 1, units), before = stage::unit_cost(seg, G, Q, w, blockIdx.x, units);
-        const int g = stage::path_at(seg, G, Q, w, D).g;
-        const bool cut = g < G && stage::cost_of(seg, Q, w, g) < D && stage::cost_of(seg, Q, w, g) >= before;
-        if (threadIdx.x == 0) s_g = cut ? g : -1;
+    __shared__ stage::Pos s_cut[2];
+    const int warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        const stage::Pos p = path.at(blockIdx.x + warp);
+        if ((threadIdx.x & 31) == 0) s_cut[warp] = p;
     }
     __syncthreads();
-    if (s_g >= 0) zero_slab(dlut + (int64_t)s_g * records, records, threadIdx.x, 1024);
+    const stage::Pos before = s_cut[0], cut = s_cut[1];
+    if (cut.g >= path.G) return;
+    const int64_t s0 = stage::seg_at(path.seg, path.Q, cut.g);
+    if (cut.q <= s0 || (before.g == cut.g && before.q > s0)) return;
+    zero_slab(dlut + (int64_t)cut.g * records, records, threadIdx.x, 1024);
 }
 
 template <int DT, bool FIT, bool SET>
-__global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uint32_t table_bytes, int nbuf, bool whole)
+__global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uint32_t table_bytes, int nbuf,
+                                                             const __grid_constant__ stage::Path path, bool whole)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_abort;
@@ -226,26 +229,20 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
         stage::init(bar + 8);
         s_abort = 0;
     }
-    const int64_t w = table_bytes / BWD_PATH_BYTES;
     stage::Pos start, end;
     if (whole) {  // grid: one CTA per glyph
         start = stage::Pos{(int)blockIdx.x, 0};
         end = stage::Pos{(int)blockIdx.x, a.Q};
         __syncthreads();
     } else {
-        stage::unit_of(a.seg, G, a.Q, w, s_unit, start, end);  // its barrier also publishes the mbarriers
+        path.unit(s_unit, start, end);  // its barrier also publishes the mbarriers
     }
 
-    // SET: glyphs z .. are still to be zeroed (those wholly inside this unit, through glyph `last`)
+    // SET: glyphs z .. are still to be zeroed: those wholly inside this unit, through glyph `last`
     int z = start.g;
-    int64_t D0 = INT64_MIN, D1 = INT64_MAX;
-    if (SET && !whole) {
-        D0 = stage::unit_cost(a.seg, G, a.Q, w, blockIdx.x, gridDim.x);
-        D1 = stage::unit_cost(a.seg, G, a.Q, w, blockIdx.x + 1, gridDim.x);
-    }
     const auto zero_through = [&](int last) {
         for (; z <= last && z < G; ++z)
-            if (stage::cost_of(a.seg, a.Q, w, z) >= D0 && stage::cost_of(a.seg, a.Q, w, z + 1) <= D1)
+            if ((z > start.g || start.q <= stage::seg_at(a.seg, a.Q, z)) && (z < end.g || end.q >= stage::seg_at(a.seg, a.Q, z + 1)))
                 zero_slab(reinterpret_cast<float4*>(a.dlut) + (int64_t)z * records, records, tid, SBB);
     };
     const auto copy = [&](int g, int buf) {
@@ -329,13 +326,13 @@ static cudaError_t launch_bwd_staged_ft(const BackwardArgs& a, uint32_t table_by
     // 321 -> 357), and with two buffers the unit hides the next table's copy (1,000 uneven glyphs of N = 20,
     // in a training step: 376 -> 582).
     const bool whole = nbuf == 1 && a.L.n_glyphs >= 24 * sm_count();
-    const int64_t blocks = whole ? a.L.n_glyphs : stage::units_for(a.Q, a.L.n_glyphs, w, (int64_t)sm_count() * 2);
-    if (SET && !whole && blocks > 1) {
+    const int64_t units = stage::units_for(a.Q, a.L.n_glyphs, w, (int64_t)sm_count() * 2);
+    const stage::Path path(a.seg, a.L.n_glyphs, a.Q, w, units);
+    if (SET && !whole && units > 1) {
         const int P = a.L.N_uniform + 2;
-        k_zero_cut<<<(unsigned)(blocks - 1), 1024, 0, s>>>(a.seg, a.L.n_glyphs, a.Q, w, blocks,
-                                                           reinterpret_cast<float4*>(a.dlut), 6 * P * P);
+        k_zero_cut<<<(unsigned)(units - 1), 1024, 0, s>>>(path, reinterpret_cast<float4*>(a.dlut), 6 * P * P);
     }
-    k_query_bwd_staged<DT, FIT, SET><<<(unsigned)blocks, SBB, smem, s>>>(a, table_bytes, nbuf, whole);
+    k_query_bwd_staged<DT, FIT, SET><<<(unsigned)(whole ? a.L.n_glyphs : units), SBB, smem, s>>>(a, table_bytes, nbuf, path, whole);
     return cudaGetLastError();
 }
 

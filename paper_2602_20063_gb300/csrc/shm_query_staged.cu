@@ -33,7 +33,7 @@ constexpr int SSHAPES[N_SSHAPES] = {512, 1024, 256};
 // STD: the usual output set (R, gradient and normal; no chart derivatives, no cell indices), so the
 // per-query output checks drop out of the loop.
 template <int DT, int SBLOCK, bool STD, int NBUF>
-__global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArgs a, uint32_t table_bytes)
+__global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArgs a, uint32_t table_bytes, const __grid_constant__ stage::Path path)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_abort;
@@ -69,9 +69,8 @@ __global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArg
         stage::init(bar + 8);
         s_abort = 0;
     }
-    const int64_t w = table_bytes / stage::QUERY_BYTES;
     stage::Pos start, end;
-    stage::unit_of(a.seg, G, a.Q, w, s_unit, start, end);  // its barrier also publishes the mbarriers
+    path.unit(s_unit, start, end);  // its barrier also publishes the mbarriers
 
     const auto copy = [&](int g, int buf) {
         stage::issue(bar + 8 * buf, table_s + buf * table_bytes,
@@ -152,9 +151,10 @@ cudaError_t launch_staged_n(const QueryArgs& a, uint32_t table_bytes, cudaStream
     int resident = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, fn, SBLOCK, smem) != cudaSuccess || resident < 1)
         resident = 1;
-    const int64_t blocks = stage::units_for(a.Q, a.L.n_glyphs, table_bytes / stage::QUERY_BYTES,
-                                            (int64_t)sm_count() * resident);
-    k_query_staged<DT, SBLOCK, STD, NBUF><<<(unsigned)blocks, SBLOCK, smem, s>>>(a, table_bytes);
+    const int64_t w = table_bytes / stage::QUERY_BYTES;
+    const int64_t units = stage::units_for(a.Q, a.L.n_glyphs, w, (int64_t)sm_count() * resident);
+    k_query_staged<DT, SBLOCK, STD, NBUF>
+        <<<(unsigned)units, SBLOCK, smem, s>>>(a, table_bytes, stage::Path(a.seg, a.L.n_glyphs, a.Q, stage::path_weight(w, a.L.n_glyphs, units), units));
     return cudaGetLastError();
 }
 

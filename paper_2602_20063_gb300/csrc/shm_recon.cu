@@ -35,7 +35,8 @@ struct StagedFace {
 };
 
 template <int DT, int METHOD>
-__global__ void __launch_bounds__(RS_BLOCK, 2) k_recon_staged(QueryArgs a, uint32_t table_bytes, uint32_t slot, int nbuf)
+__global__ void __launch_bounds__(RS_BLOCK, 2) k_recon_staged(QueryArgs a, uint32_t table_bytes, uint32_t slot, int nbuf,
+                                                              const __grid_constant__ stage::Path path)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_abort;
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(RS_BLOCK, 2) k_recon_staged(QueryArgs a, uint3
         s_abort = 0;
     }
     stage::Pos start, end;
-    stage::unit_of(a.seg, G, a.Q, table_bytes / stage::QUERY_BYTES, s_unit, start, end);
+    path.unit(s_unit, start, end);
 
     // bytes [lo, lo + table_bytes) of the pool: whole 16-byte blocks from the boundary before lo, and the
     // remainder
@@ -148,9 +149,10 @@ cudaError_t launch_recon_staged(const QueryArgs& a, uint32_t table_bytes, cudaSt
     const int smem = stage::TABLE_OFFSET + nbuf * (int)slot;
     const cudaError_t e = ensure_dynamic_smem((const void*)k_recon_staged<DT, METHOD>, smem);
     if (e != cudaSuccess) return e;
-    const int64_t blocks =
-        stage::units_for(a.Q, a.L.n_glyphs, table_bytes / stage::QUERY_BYTES, (int64_t)sm_count() * 2);
-    k_recon_staged<DT, METHOD><<<(unsigned)blocks, RS_BLOCK, smem, s>>>(a, table_bytes, slot, nbuf);
+    const int64_t w = table_bytes / stage::QUERY_BYTES;
+    const int64_t units = stage::units_for(a.Q, a.L.n_glyphs, w, (int64_t)sm_count() * 2);
+    k_recon_staged<DT, METHOD><<<(unsigned)units, RS_BLOCK, smem, s>>>(a, table_bytes, slot, nbuf,
+                                                                     stage::Path(a.seg, a.L.n_glyphs, a.Q, stage::path_weight(w, a.L.n_glyphs, units), units));
     return cudaGetLastError();
 }
 

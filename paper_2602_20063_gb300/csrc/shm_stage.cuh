@@ -97,37 +97,68 @@ __device__ __forceinline__ int64_t seg_at(const int64_t* seg, int64_t Q, int g)
     return min(max(__ldg(seg + g), (int64_t)0), Q);
 }
 
-// Cost of the path up to glyph g, and up to the start of unit u of `units`.
-__device__ __forceinline__ int64_t cost_of(const int64_t* seg, int64_t Q, int64_t w, int g)
-{
-    return seg_at(seg, Q, g) - seg_at(seg, Q, 0) + w * g;
-}
+// The path and its cut into `units` (see above), the same on every CTA and on the host.
+struct Path {
+    const int64_t* seg;
+    int G;
+    int64_t Q;
+    int64_t w;       // cost of a glyph
+    uint32_t units;
+    uint64_t inv;    // 2^64 / units, rounded up: x / units = umulhi(x, inv) for x units < 2^64
 
-__device__ __forceinline__ int64_t unit_cost(const int64_t* seg, int G, int64_t Q, int64_t w, int64_t u, int64_t units)
-{
-    const int64_t total = cost_of(seg, Q, w, G);
-    return total / units * u + total % units * u / units;
-}
+    Path(const int64_t* seg_, int G_, int64_t Q_, int64_t w_, int64_t units_)
+        : seg(seg_), G(G_), Q(Q_), w(w_), units((uint32_t)units_), inv(UINT64_MAX / (uint64_t)units_ + 1) {}
 
-// The path position at cost D (a whole warp calls it; 32 probes per round, so two or three dependent
-// loads; a CTA has nothing else to do before its first copy).
-__device__ __forceinline__ Pos path_at(const int64_t* seg, int G, int64_t Q, int64_t w, int64_t D)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t lo = seg_at(seg, Q, 0);
-    int g = 0, n = G + 1;  // the largest g in [0, G] with cost(g) = seg[g] - seg[0] + w g <= D
-    int64_t s = lo;        // seg[g]
-    while (n > 1) {
-        const int step = (n + 31) / 32, at = lane * step;
-        const int64_t v = at < n ? seg_at(seg, Q, g + at) : INT64_MAX / 2;
-        const unsigned m = __ballot_sync(0xffffffffu, at < n && v - lo + w * (g + at) <= D);
-        const int k = 31 - __clz((int)(m | 1u));
-        s = __shfl_sync(0xffffffffu, v, k);
-        g += k * step;
-        n = min(step, n - k * step);
+    // Start of unit u on the path (a whole warp calls it): u units of cost.  The first 32 probes surround the
+    // glyph that even segments would put there and wait for nothing, so that a near miss costs one memory round trip,
+    // together with the ends' that the cost needs; otherwise 32 probes per round, two or three dependent round trips.
+    __device__ __forceinline__ Pos at(uint32_t u) const
+    {
+        const int lane = threadIdx.x & 31;
+        const int guess = units > 1 ? (int)__umul64hi((uint64_t)u * (uint32_t)G, inv) : (u ? G : 0);
+        const int base = max(0, min(guess - 15, G - 31)), near = base + lane;
+        int64_t v = near <= G ? seg_at(seg, Q, near) : INT64_MAX / 2;
+        const int64_t lo = seg_at(seg, Q, 0);
+        const uint64_t total = seg_at(seg, Q, G) - lo + w * G;
+        int64_t D = (int64_t)total;  // cost of the path up to unit u
+        if (u < units) {
+            const uint64_t per = units > 1 ? __umul64hi(total, inv) : total;
+            D = (int64_t)(per * u + (u ? __umul64hi((total - per * units) * u, inv) : 0));
+        }
+        // the largest g in [0, G] with cost(g) = seg[g] - seg[0] + w g <= D, and seg[g]
+        unsigned m = __ballot_sync(0xffffffffu, near <= G && v - lo + w * near <= D);
+        int k = 31 - __clz((int)(m | 1u));
+        int g = base + k;
+        int64_t s = __shfl_sync(0xffffffffu, v, k);
+        if (!(m & 1u) || (k == 31 && g < G)) {
+            g = 0;
+            s = lo;
+            for (int n = G + 1; n > 1;) {
+                const int step = (n + 31) / 32, at = lane * step;
+                v = at < n ? seg_at(seg, Q, g + at) : INT64_MAX / 2;
+                m = __ballot_sync(0xffffffffu, at < n && v - lo + w * (g + at) <= D);
+                k = 31 - __clz((int)(m | 1u));
+                s = __shfl_sync(0xffffffffu, v, k);
+                g += k * step;
+                n = min(step, n - k * step);
+            }
+        }
+        return Pos{g, min(Q, s + max((int64_t)0, D - (s - lo + w * g) - w))};
     }
-    return Pos{g, min(Q, s + max((int64_t)0, D - (s - lo + w * g) - w))};
-}
+
+    // This CTA's unit: start and end positions through shared memory (every thread calls it).
+    __device__ __forceinline__ void unit(Pos* sh, Pos& start, Pos& end) const
+    {
+        const int warp = threadIdx.x >> 5;
+        if (warp < 2) {
+            const Pos p = at(blockIdx.x + warp);
+            if ((threadIdx.x & 31) == 0) sh[warp] = p;
+        }
+        __syncthreads();
+        start = sh[0];
+        end = sh[1];
+    }
+};
 
 // The first non-empty part of glyph g or a later one, up to the end position.
 __device__ __forceinline__ Part next_part(const int64_t* seg, int G, int64_t Q, int g, const Pos& start, const Pos& end)
@@ -141,19 +172,6 @@ __device__ __forceinline__ Part next_part(const int64_t* seg, int G, int64_t Q, 
     return Part{G, 0, 0};
 }
 
-// This CTA's unit of the path: start and end positions through shared memory (every thread calls it).
-__device__ __forceinline__ void unit_of(const int64_t* seg, int G, int64_t Q, int64_t w, Pos* sh, Pos& start, Pos& end)
-{
-    const int warp = threadIdx.x >> 5;
-    if (warp < 2) {
-        const Pos p = path_at(seg, G, Q, w, unit_cost(seg, G, Q, w, blockIdx.x + warp, gridDim.x));
-        if ((threadIdx.x & 31) == 0) sh[warp] = p;
-    }
-    __syncthreads();
-    start = sh[0];
-    end = sh[1];
-}
-
 // Host: units for Q queries over G glyphs, at most `cap` (the CTAs that run at once); just under one
 // glyph each becomes one glyph each, which leaves even segments uncut.
 inline int64_t units_for(int64_t Q, int64_t G, int64_t w, int64_t cap)
@@ -162,6 +180,11 @@ inline int64_t units_for(int64_t Q, int64_t G, int64_t w, int64_t cap)
     const int64_t m = n < cap ? n : cap;
     return m > G && m - G <= m / 32 ? G : m;
 }
+
+// Host: cost of a glyph on the path.  With more units than glyphs nearly every unit starts inside a glyph and pays a
+// copy of its own anyway, so that glyphs are cut nearly by queries alone (152 even glyphs of 4,096, N = 32 f32: 16.4 ->
+// 12.4 us); a little is left so that runs of tiny glyphs do not pile up in one unit.
+inline int64_t path_weight(int64_t w, int64_t G, int64_t units) { return units > G ? w / 4 + 1 : w; }
 
 template <int DT>
 __device__ __forceinline__ float4 rec(const unsigned char* table, int r)
