@@ -170,6 +170,8 @@ __global__ void __launch_bounds__(BwdCta<FIT>::threads, BwdCta<FIT>::resident) k
 // and DRAM sees one write of the slab instead of a fill, a read and a write; the glyphs that a unit
 // boundary cuts are zeroed first by k_zero_cut.
 constexpr int SBB = 512;
+constexpr int WINDOWS_PER_SM = 2;
+constexpr uint32_t WHOLE_BYTES = 80000;
 constexpr int BWD_PATH_BYTES = 64;  // table bytes per unit of path cost: the copy and the slab's traffic in queries
 
 __device__ __forceinline__ void zero_slab(float4* slab, int records, int tid, int threads)
@@ -195,9 +197,42 @@ __global__ void __launch_bounds__(1024) k_zero_cut(const __grid_constant__ stage
     zero_slab(dlut + (int64_t)cut.g * records, records, threadIdx.x, 1024);
 }
 
+// One CTA per glyph, with a bound on a CTA's share of a long segment: the queries are covered by windows of
+// `size` of them, each with a CTA of its own after the glyphs'.  A glyph's CTA takes its segment through the end
+// of the window after the one it starts in; what lies beyond goes window by window to the windows' CTAs.  A segment
+// of at most `size` queries is never cut, and none holds a CTA for more than two windows.
+struct Windows {
+    int64_t size;
+    int n;
+    uint64_t inv;  // 2^64 / size, rounded up: s / size = umulhi(s, inv) for s size < 2^64
+    Windows(int64_t Q, int n_) : size(n_ > 0 ? (Q + n_ - 1) / n_ + 1 : 2), n(n_), inv(UINT64_MAX / (uint64_t)size + 1) {}
+    __device__ __forceinline__ int64_t own_end(int64_t s0) const { return (int64_t)(__umul64hi((uint64_t)s0, inv) + 2) * size; }
+    // The long segment that goes on in window b (a whole warp calls it); G: none.
+    __device__ __forceinline__ int glyph(const int64_t* seg, int G, int64_t Q, int b) const
+    {
+        const int64_t lo = b * size;
+        if (lo >= Q || lo < __ldg(seg)) return G;
+        const int g = seg_find_warp(seg, G, lo);
+        return g < G && own_end(stage::seg_at(seg, Q, g)) <= lo ? g : G;
+    }
+};
+
+// Block b zeroes the slab of the glyph whose first part beyond its own CTA's share is in window b.
+__global__ void __launch_bounds__(256) k_zero_long(const int64_t* seg, int G, int64_t Q, Windows win, float4* dlut, int records)
+{
+    __shared__ int s_g;
+    if (threadIdx.x < 32) {
+        const int g = win.glyph(seg, G, Q, blockIdx.x);
+        const bool first = g < G && win.own_end(stage::seg_at(seg, Q, g)) == blockIdx.x * win.size;
+        if (threadIdx.x == 0) s_g = first ? g : -1;
+    }
+    __syncthreads();
+    if (s_g >= 0) zero_slab(dlut + (int64_t)s_g * records, records, threadIdx.x, 256);
+}
+
 template <int DT, bool FIT, bool SET>
 __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uint32_t table_bytes, int nbuf,
-                                                             const __grid_constant__ stage::Path path, bool whole)
+                                                             const __grid_constant__ stage::Path path, Windows win)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_abort;
@@ -230,10 +265,23 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
         s_abort = 0;
     }
     stage::Pos start, end;
-    if (whole) {  // grid: one CTA per glyph
-        start = stage::Pos{(int)blockIdx.x, 0};
-        end = stage::Pos{(int)blockIdx.x, a.Q};
-        __syncthreads();
+    if (win.n > 0) {
+        // the windows' CTAs come last: few have work, and where one does it is not long (ahead of the glyphs' their
+        // searches delayed every SM, 1.4 % on 5,000 glyphs of 4,000 queries, N = 24)
+        const int g = (int)blockIdx.x, k = g - G;
+        if (k >= 0) {
+            if (tid < 32) {
+                const int on = win.glyph(a.seg, G, a.Q, k);
+                if (tid == 0) s_unit[0].g = on;
+            }
+            __syncthreads();  // also publishes the mbarriers
+            start = stage::Pos{s_unit[0].g, k * win.size};
+            end = stage::Pos{start.g, (k + 1) * win.size};
+        } else {
+            start = stage::Pos{g, 0};
+            end = stage::Pos{g, win.own_end(stage::seg_at(a.seg, a.Q, g))};
+            __syncthreads();  // publishes the mbarriers
+        }
     } else {
         path.unit(s_unit, start, end);  // its barrier also publishes the mbarriers
     }
@@ -319,20 +367,23 @@ static cudaError_t launch_bwd_staged_ft(const BackwardArgs& a, uint32_t table_by
     cudaError_t e = ensure_dynamic_smem((const void*)k_query_bwd_staged<DT, FIT, SET>, smem);
     if (e != cudaSuccess) return e;
     const int64_t w = table_bytes / BWD_PATH_BYTES;
-    // Many glyphs, one table buffer: a CTA per glyph, which nothing cuts and which the hardware hands out as
-    // SMs come free.  Neighbouring glyphs are then in flight together (16,384 x 4,096 queries, even, N = 32:
-    // 2,055 us in cut units, 1,962 for strided glyphs, 1,727 so; 4,096 x 2,048: 352, 328, 297; uneven, in a
-    // training step: 795 -> 794).  Below 24 glyphs an SM the last uneven glyph shows (700 glyphs, N = 30:
-    // 321 -> 357), and with two buffers the unit hides the next table's copy (1,000 uneven glyphs of N = 20,
-    // in a training step: 376 -> 582).
-    const bool whole = nbuf == 1 && a.L.n_glyphs >= 24 * sm_count();
-    const int64_t units = stage::units_for(a.Q, a.L.n_glyphs, w, (int64_t)sm_count() * 2);
-    const stage::Path path(a.seg, a.L.n_glyphs, a.Q, w, units);
-    if (SET && !whole && units > 1) {
-        const int P = a.L.N_uniform + 2;
-        k_zero_cut<<<(unsigned)(units - 1), 1024, 0, s>>>(path, reinterpret_cast<float4*>(a.dlut), 6 * P * P);
-    }
-    k_query_bwd_staged<DT, FIT, SET><<<(unsigned)(whole ? a.L.n_glyphs : units), SBB, smem, s>>>(a, table_bytes, nbuf, path, whole);
+    const int G = a.L.n_glyphs, records = 6 * (a.L.N_uniform + 2) * (a.L.N_uniform + 2);
+    float4* const dlut = reinterpret_cast<float4*>(a.dlut);
+    // Many glyphs, one table buffer: a CTA per glyph, which nothing cuts but a very long segment and which the
+    // hardware hands out as SMs come free.  Neighbouring glyphs are then in flight together (16,384 x 4,096 queries,
+    // even, N = 32: 2,055 us in cut units, 1,962 for strided glyphs, 1,727 so).  From 24 glyphs an SM always; from 10
+    // where tables of at least WHOLE_BYTES have fewer queries than their own traffic is worth: 2,000 / 3,000 even
+    // glyphs of 1,500 queries, N = 32, 145 / 212 us in units and 124 / 181 so, uneven ones 147 / 211 and 144 / 196.
+    // Elsewhere the last uneven glyph shows: 3,000 of 4,000 queries, N = 24, 312 us in units and 365 so; 1,400 of 1,500,
+    // N = 32, 107 and 110; and with two buffers the unit hides the next table's copy (1,000 uneven glyphs of
+    // N = 20, in a training step: 376 us and 582).
+    const bool whole = nbuf == 1 && (G >= 24 * sm_count() || (G >= 10 * sm_count() && table_bytes >= WHOLE_BYTES && a.Q <= w * G));
+    const int64_t units = stage::units_for(a.Q, G, w, (int64_t)sm_count() * 2);
+    const stage::Path path(a.seg, G, a.Q, w, units);
+    const Windows win(a.Q, whole ? WINDOWS_PER_SM * sm_count() : 0);
+    if (SET && whole) k_zero_long<<<(unsigned)win.n, 256, 0, s>>>(a.seg, G, a.Q, win, dlut, records);
+    if (SET && !whole && units > 1) k_zero_cut<<<(unsigned)(units - 1), 1024, 0, s>>>(path, dlut, records);
+    k_query_bwd_staged<DT, FIT, SET><<<(unsigned)(whole ? win.n + G : units), SBB, smem, s>>>(a, table_bytes, nbuf, path, win);
     return cudaGetLastError();
 }
 
@@ -371,7 +422,10 @@ cudaError_t launch_query_bwd(const BackwardArgs& a, cudaStream_t s)
     if (a.Q > 0 && a.seg && !a.glyph && a.L.N_uniform > 0 && a.D.N_uniform == a.L.N_uniform && ly == SHM_LAYOUT_TEXEL) {
         const int64_t P = (int64_t)a.L.N_uniform + 2;
         const int64_t bytes = 6 * P * P * (dt == SHM_F32 ? 16 : 8);
-        const int64_t per = bytes / 128 > 256 ? bytes / 128 : 256;  // as query_is_staged
+        // Pays from fewer queries than in the forward (query_is_staged), since the staged pass's reductions also
+        // meet in L2: 3,000 even glyphs of 400 / 500 queries, N = 32, 104 / 112 us staged and 118 / 131 not; of 200 / 256,
+        // N = 23, 62 / 64 and 59 / 76; on small tables the copy's latency dominates (10,000 of 200, N = 8: 109 and 91).
+        const int64_t per = bytes / 256 > 256 ? bytes / 256 : 256;
         if (bytes <= STAGED_TABLE_MAX_BYTES && a.Q >= a.L.n_glyphs * per) {
             if (dt == SHM_F32) return launch_bwd_staged<SHM_F32>(a, (uint32_t)bytes, s);
             if (dt == SHM_F16) return launch_bwd_staged<SHM_F16>(a, (uint32_t)bytes, s);

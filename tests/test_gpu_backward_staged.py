@@ -16,7 +16,7 @@ import torch
 import oracle as O
 import oracle.fit as OF
 import shm_inputs as I
-from gpu_common import near_edge, shm, upload_pool
+from gpu_common import best_us, near_edge, shm, upload_pool
 
 pytestmark = pytest.mark.gpu
 
@@ -262,3 +262,95 @@ def test_many_glyphs_one_cta_each(S, extra):
         r, x = ref.data.view(-1, 4).double(), out.data.view(-1, 4).double()
         assert ((x - r).abs().amax(0) <= 2e-6 * r.abs().amax(0)).all()
     assert st.item() == S.SHM_DEV_BOUNDS
+
+
+@pytest.mark.parametrize("long_at", [0, 611, 1215])
+@pytest.mark.parametrize("fit", [False, True])
+def test_long_segments_among_many_glyphs(S, long_at, fit):
+    """One CTA per glyph leaves what a segment holds beyond two windows of queries to other CTAs: a segment of
+    dozens of windows at the start, inside and at the end of the pool, further ones of about one, two and three
+    windows, empty ones, queries outside; accumulated and written gradients (or the fused fit) equal the
+    per-query pass with glyph ids."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    G, N = 8 * sms, 23
+    counts = [(g * 613) % 700 * (g % 11 != 3) for g in range(G)]
+    counts[long_at * G // 1216] = 210000
+    counts[200], counts[400], counts[700] = 2400, 4900, 7300
+    seg, glyph, Q = _segments(counts, 33, 50)
+    bytes_ = 6 * (N + 2) ** 2 * 16
+    assert G * max(256, bytes_ // 128) <= Q <= G * (bytes_ // 64)  # staged, a CTA per glyph
+    g = torch.Generator(device="cuda").manual_seed(5)
+    lut = S.alloc_lut(G, N)
+    lut.data.copy_(1.0 + 0.1 * torch.randn(lut.data.shape, generator=g, device="cuda"))
+    d = torch.nn.functional.normalize(torch.randn(Q, 3, generator=g, device="cuda"), dim=1)
+    ref = S.like_lut(lut, zero=True)
+    if fit:
+        Rt, nt = torch.rand(Q, generator=g, device="cuda"), torch.nn.functional.normalize(d + 0.1, dim=1)
+        losses = []
+        for out, sel in ((ref, dict(glyph=_t(glyph))), (S.like_lut(lut, zero=True), dict(seg=_t(seg)))):
+            loss = torch.zeros(1, device="cuda")
+            S.fit_backward(lut, d, Rt, nt, out, w_value=1.0, w_normal=0.25, loss=loss, **sel)
+            losses.append(loss.item())
+        assert abs(losses[0] - losses[1]) <= 1e-5 * losses[0]
+        outs = [out]
+    else:
+        up = [torch.randn(s, generator=g, device="cuda") for s in ((Q,), (Q, 3), (Q, 3))]
+        kw = dict(gR=up[0], ggrad=up[1], gnormal=up[2])
+        a = S.query_backward(lut, d, ref, glyph=_t(glyph), **kw)
+        ok, outs = torch.isfinite(a), []
+        for over in (False, True):
+            out = S.like_lut(lut, zero=not over)
+            if over:
+                out.data.fill_(float("nan"))
+            b = S.query_backward(lut, d, out, seg=_t(seg), overwrite=over, **kw)
+            assert torch.equal(ok, torch.isfinite(b)) and float((a[ok] - b[ok]).abs().max()) <= 2e-6 * float(a[ok].abs().max())
+            outs.append(out)
+    # the same sums in another order: roundings of a record's partial sums, which grow with its terms
+    r = ref.data.view(-1, 4).double()
+    for out in outs:
+        x = out.data.view(-1, 4).double()
+        assert torch.isfinite(x).all() and ((x - r).abs().amax(0) <= 1e-5 * r.abs().amax(0)).all()
+
+
+def test_one_dominant_segment_spreads(S):
+    """A segment that holds two thirds of all queries costs at most four times the same queries spread evenly."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    G, N, Q = 24 * sms, 23, 24 * sms * 900
+    lut, dl = S.alloc_lut(G, N, zero=True), None
+    lut.data.fill_(1.0)
+    dl = S.like_lut(lut, zero=True)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    d = torch.nn.functional.normalize(torch.randn(Q, 3, generator=g, device="cuda"), dim=1)
+    gR = torch.ones(Q, device="cuda")
+    t = {}
+    for name, counts in (("even", [900] * G), ("dominant", [300] * (G // 2) + [300 + 600 * G] + [300] * (G - G // 2 - 1))):
+        seg = _t(np.concatenate([[0], np.cumsum(counts)]).astype(np.int64))
+        t[name] = best_us(lambda: S.query_backward(lut, d, dl, gR=gR, seg=seg))
+    assert t["dominant"] <= 4 * t["even"], t
+
+
+@pytest.mark.parametrize("N,lo,hi", [(8, 200, 900), (20, 400, 1300)])
+def test_staged_backward_hundreds_of_glyphs(S, N, lo, hi):
+    """Hundreds of glyphs, empty and long ones between them, dense enough to be staged (asserted), two tables per
+    CTA: every CTA restages tables several times; against the oracle."""
+    rng = np.random.default_rng(340)
+    G = 400
+    counts = rng.integers(lo, hi, size=G)
+    counts[rng.choice(G, 60, replace=False)] = 0
+    counts[5], counts[6] = 3024, 6049
+    luts = _pool(G, N, 4, 1400)
+    Lp, stored = upload_pool(S, luts)
+    seg, glyph, Q = _segments(counts, head=0, tail=0)
+    assert Q >= G * max(256, 6 * (N + 2) ** 2 * 16 // 128)
+    dirs = I.directions(Q, 341)
+    gR = rng.normal(size=Q).astype(np.float32)
+    gn = rng.normal(size=(Q, 3)).astype(np.float32)
+    off, Ns = O.make_pool(luts)[1:]
+    dref, ddref = O.query_vjp(stored.reshape(-1, 4), off, Ns, dirs, gR=gR, gn=gn, glyph=glyph)
+    for over in (False, True):
+        dl = S.like_lut(Lp, zero=not over)
+        if over:
+            dl.data.fill_(float("nan"))
+        dd = S.query_backward(Lp, _t(dirs), dl, gR=_t(gR), gnormal=_t(gn), seg=_t(seg), overwrite=over)
+        _check_dlut(dl.data.view(-1, 4).double().cpu().numpy(), dref)
+        _check_ddirs(dd.double().cpu().numpy(), ddref, dirs, N, np.ones(Q, bool))
