@@ -148,9 +148,9 @@ shm_status shm_tune_reset(void);
  *   - lut: any dtype, texel or cell layout, uniform resolution (N_uniform > 0, else
  *     SHM_ERR_UNSUPPORTED); only glyph 0 is read.
  *   - ws: device workspace of at least shm_query_binned_workspace_bytes(lut, Q, band_bytes)
- *     (about 25 B per query: the partitioned directions, replaced by R / R_u / R_v, one bin byte
- *     per query, per-block offsets and counters), else SHM_ERR_WORKSPACE.  Its contents need no clearing and
- *     are scratch after the call; two calls that overlap on the GPU must not share it.
+ *     (about 14 B per query: the partitioned directions, replaced by R / R_u / R_v, and a 16-bit slot;
+ *     per-block offsets and counters), else SHM_ERR_WORKSPACE.  Its contents need no clearing and are
+ *     scratch after the call; two calls that overlap on the GPU must not share it.
  *   - dirs and the outputs follow shm_query's rules (device or page-locked host memory); the
  *     directions are read twice, so device memory is the fast case.
  *   - band_bytes < 0 or Q < 0: SHM_ERR_INVALID_ARG. */

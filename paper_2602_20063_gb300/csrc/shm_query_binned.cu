@@ -253,6 +253,7 @@ __global__ void __launch_bounds__(PT, 2) k_bin_partition(BinParams p, const floa
 // results cross a 96-float buffer so that every global access is 128 contiguous bytes.  Bound: requests
 // from L1 to L2, about three per footprint; three CTAs per SM keep the bins in flight fewer than four.
 constexpr int QB = 256, QILP = 2;
+constexpr int SHORT_RUN = 100;  // queries of a block's mean run
 
 template <int DT, int LAYOUT>
 __global__ void __launch_bounds__(QB, 3) k_bin_query(BinParams p, LutView L, const unsigned short* __restrict__ starts,
@@ -502,10 +503,11 @@ cudaError_t launch_bin_query(const BinParams& p, const LutView& L, const unsigne
     const int64_t most = PQ / (32 * (int64_t)p.B);
     if (pieces > most) pieces = most;
     if (pieces < 1) pieces = 1;
-    // One unit at a time keeps the units in flight within the fewest bins; two halve the counter's load, which
-    // pays where they still cover less than half a bin (2^26 queries: 1,751 against 1,788 us; 2^24: 548
-    // against 486).
-    const int grab = 4 * warps <= p.nblk * pieces ? 2 : 1;
+    // One unit at a time keeps the units in flight within the fewest bins; two halve the counter's load.  They pay
+    // where they still cover less than half a bin (2^26 queries: 1,751 against 1,788 us; 2^24: 548 against 486), and where
+    // runs are short: one address takes about 500 additions per microsecond, which bound 54 bins of 76 queries a block
+    // (f32 cells of N = 2048, 2^22 / 2^24 / 2^25 queries: 221 / 727 / 1,055 us one at a time, 171 / 538 / 986 two).
+    const int grab = 4 * warps <= p.nblk * pieces || PQ / p.B < SHORT_RUN ? 2 : 1;
     int64_t blocks = (runs * pieces + QB / 32 - 1) / (QB / 32);
     if (blocks > cap) blocks = cap;
     k_bin_query<DT, LAYOUT><<<(unsigned)blocks, QB, 0, s>>>(p, L, starts, (int)pieces, grab, sorted, taken, dev_status);
@@ -564,11 +566,7 @@ bool binned_plan(const LutView& L, int64_t Q, int64_t band_bytes, BinLayout* out
     z.o_slot = o;   o = align256(o + 2 * Q);
     z.o_start = o;  o = align256(o + 2 * z.p.B * z.p.nblk);
     z.o_taken = o;  // three counters
-    // The size asked of the caller is that of the earlier global partition (25 B per query and 12 B per
-    // bin and 16,384 queries), which exceeds what is used: sizes that callers keep stay valid.
-    const int64_t tiles = (Q + 16383) / 16384, B = z.p.B;
-    z.bytes = align256(12 * Q) + align256(4 * Q) + align256(8 * Q) + align256(Q) + align256(4 * B * tiles) +
-              align256(8 * B * tiles) + align256(8 * B);
+    z.bytes = align256(o + 3 * (int64_t)sizeof(uint32_t));
     *out = z;
     return true;
 }

@@ -184,3 +184,22 @@ def test_binned_blocks(S, Q, kind):
             out[k] = torch.empty(n * Q + 1, device="cuda")[1:].view(Q, 3)
     out = S.query_binned(L, d, ws, band_bytes=20000, want=WANT, out=out)
     _equal(out, S.query(L, d, want=WANT))
+
+
+@pytest.mark.parametrize("Q", [1, 31, 4096, 4097, 70000])
+@pytest.mark.parametrize("layout,band", [(0, 20000), (1, 6000), (0, 0)])
+def test_binned_workspace_is_what_it_uses(S, Q, layout, band):
+    """The size asked for is 14 B a query, two per bin and block, and alignment; a workspace of exactly that size at the
+    end of a larger buffer is enough, nothing beyond or before it is written, and one byte less is refused."""
+    lut = _glyph(23, N=48, L=4)
+    L, _ = upload_pool(S, [lut], layout=layout)
+    bins = S.query_binned_bins(L, band)["bins"]
+    n = S.query_binned_workspace_bytes(L, Q, band)
+    assert 14 * Q <= n <= 14 * Q + 2 * bins * ((Q + 4095) // 4096) + 5 * 256
+    d = torch.from_numpy(I.directions(Q, 9)).cuda()
+    buf = torch.full((256 + n + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    out = S.query_binned(L, d, buf[256:256 + n], band_bytes=band, want=WANT)
+    _equal(out, S.query(L, d, want=WANT))
+    assert (buf[:256] == 0xA5).all() and (buf[256 + n:] == 0xA5).all()
+    with pytest.raises(S.ShmError, match="workspace"):
+        S.query_binned(L, d, buf[256:255 + n], band_bytes=band, want=WANT)
