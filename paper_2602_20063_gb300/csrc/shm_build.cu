@@ -550,8 +550,8 @@ __global__ void __launch_bounds__(256) k_value_build(LutView out, void* data, sh
 // Uniform pools split each face into 2 x 2 equal regions once a whole face's samples would need
 // more than FACE_SPLIT_SMEM bytes, i.e. fewer CTAs per SM than the register limit of five allows
 // (512 bump objects: N = 128 0.944 vs 0.982 ms, N = 144 1.171 vs 1.340 ms; N <= 96 stays whole,
-// where splitting measured -1 % to +1 %).  The sample directions and values are those of the
-// value tables (k_value_build).
+// where splitting measured -1 % to +1 %).  The sample directions are those of the value tables
+// (k_value_build), and so are the values, but for octaves of k_fbm_face whose frequency is no power of two.
 constexpr int FACE_N_MAX = 144;   // (N+4)^2 floats <= 87.6 KB
 constexpr int REGION_T = 64;      // region edge for larger tables: 66^2 floats = 17.4 KB
 constexpr int FACE_SPLIT_T = 66;  // uneven pools: N <= 64 faces stay whole, N = 128 faces split 2 x 2
@@ -649,7 +649,8 @@ __global__ void __launch_bounds__(256) k_fd_face(LutView out, void* data, shm_so
 // (each component of (1, X, Y)/rho is monotone or has its extreme at the smallest |X| and |Y|), widened by
 // 1e-6 against rounding.  Octaves whose box does not fit the cache are hashed per sample.
 // Bound: FP32 issue (about 70 instructions per pair of samples and octave; 73 % of the issue slots).  N = 2048,
-// 8 octaves: 708 -> 470 us, the same values; before, boxes padded by a lattice step on each side left the
+// 8 octaves: 708 -> 470 us, the same values where the frequency is a power of two (a boxed octave no longer rounds the
+// product w f first, others and the value tables do); before, boxes padded by a lattice step on each side left the
 // last octave of 60 % of the regions to per-sample hashing, floor and integer conversions took 12 of the
 // slow conversion operations per pair, and corner indices were clamped.
 template <class Map>

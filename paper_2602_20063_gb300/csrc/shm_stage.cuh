@@ -6,7 +6,8 @@
 // glyphs in order, paying `w` for every glyph (its table copy) and 1 for every query.  A unit is a CTA's
 // whole work: it starts and ends anywhere inside a glyph, so a few long segments spread over every SM
 // and uneven ones balance (one CTA per glyph left 37 glyphs of 60,000 queries on 37 of 304 CTAs).  w is
-// the copy's cost in queries at memory bandwidth, table bytes / 40 B of directions and outputs.
+// the copy's cost in queries at memory bandwidth, table bytes / 40 B of directions and outputs (a quarter of
+// it where units outnumber the glyphs, path_weight).
 #pragma once
 #include "shm_internal.h"
 
