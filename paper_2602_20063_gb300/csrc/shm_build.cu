@@ -419,8 +419,9 @@ __device__ __forceinline__ float2 value_noise_lattice2(float2 x, float2 y, float
 constexpr int FS = 18, MAX_BUMPS_SMEM = 128;
 // Longest region edge of the fBm bake: 64 / 48 / 32 texels measured 470 / 474 / 590 us at N = 2048, 160 / 154 / 186 at
 // N = 1024 (larger regions miss the cache there).  A face is cut into equal regions of at most that: 48 + 2 texels
-// for N = 48 took 60 us (64 glyphs, six octaves), 2 x 25 take 49 and the whole face 38.  Faces of up to FBM_WHOLE
-// texels stay whole where there are enough of them for every SM (16 glyphs: whole 20.5 us, cut 16.5).
+// for N = 48 took 60 us (64 glyphs, six octaves), 2 x 25 take 49 and the whole face 38.  One region fewer a side where
+// they would be shorter than 44, the fewer ones are no longer than FBM_WHOLE and there is one for every SM (64 / 16
+// glyphs: N = 48 whole 38 / 20.5 us, in two 49 / 16.5; N = 95 in two 99 / 33, in three 127 / 39).
 constexpr int FBM_T = 48;
 constexpr int FBM_WHOLE = 66;
 constexpr int FBM_CACHE = 5376;  // lattice entries of the octaves' boxes per CTA (42 KB, four CTAs per SM)
@@ -803,9 +804,9 @@ cudaError_t launch_fd_build(const LutView& out, void* data, const shm_source& sr
     const bool fbm = src.kind == SHM_SRC_FBM;
     if (fbm) {
         const int P = sz.max_N + 2;
-        T = P <= FBM_T || (P <= FBM_WHOLE && 6LL * sz.G >= sm_count()) ? P : FBM_T;
-        const int nr = (P + T - 1) / T;
-        if (sz.N_uniform > 0) T = (P + nr - 1) / nr;
+        int nr = (P + FBM_T - 1) / FBM_T;
+        if (nr > 1 && P < 44 * nr && P <= FBM_WHOLE * (nr - 1) && 6LL * sz.G * (nr - 1) * (nr - 1) >= sm_count()) --nr;
+        T = (P + nr - 1) / nr;
     } else {
         if (sz.N_uniform == 0 && T > FACE_SPLIT_T) T = FACE_SPLIT_T;
         if (sz.N_uniform > 0 && T <= FACE_N_MAX + 2 && (T + 2) * (T + 2) * (int)sizeof(float) > FACE_SPLIT_SMEM)
