@@ -7,7 +7,7 @@
 // whole work: it starts and ends anywhere inside a glyph, so a few long segments spread over every SM
 // and uneven ones balance (one CTA per glyph left 37 glyphs of 60,000 queries on 37 of 304 CTAs).  w is
 // the copy's cost in queries at memory bandwidth, table bytes / 40 B of directions and outputs (a quarter of
-// it where units outnumber the glyphs, path_weight).
+// it where there are one to four units a glyph, path_weight).
 #pragma once
 #include "shm_internal.h"
 
@@ -182,10 +182,12 @@ inline int64_t units_for(int64_t Q, int64_t G, int64_t w, int64_t cap)
     return m > G && m - G <= m / 32 ? G : m;
 }
 
-// Host: cost of a glyph on the path.  With more units than glyphs nearly every unit starts inside a glyph and pays a
-// copy of its own anyway, so that glyphs are cut nearly by queries alone (152 even glyphs of 4,096, N = 32 f32: 16.4 ->
-// 12.4 us); a little is left so that runs of tiny glyphs do not pile up in one unit.
-inline int64_t path_weight(int64_t w, int64_t G, int64_t units) { return units > G ? w / 4 + 1 : w; }
+// Host: cost of a glyph on the path.  With up to four units a glyph most units start inside one and pay a copy of
+// their own, so that glyphs are cut nearly by queries alone (152 even glyphs of 4,096, N = 32 f32: 16.4 -> 12.4 us); a
+// quarter is left so that runs of tiny glyphs do not pile up in one unit.  More units, or tables below 40 KB, keep
+// the whole cost, which spares slivers of glyphs (152 uneven glyphs, N = 13: 12.4 against 14.4 us; 37 of N = 32 f16,
+// 60,000 queries each: 28.9 against 29.2).
+inline int64_t path_weight(int64_t w, int64_t G, int64_t units) { return units > G && units < 4 * G && w >= 1024 ? w / 4 : w; }
 
 template <int DT>
 __device__ __forceinline__ float4 rec(const unsigned char* table, int r)
