@@ -424,8 +424,9 @@ cudaError_t launch_query_bwd(const BackwardArgs& a, cudaStream_t s)
         const int64_t bytes = 6 * P * P * (dt == SHM_F32 ? 16 : 8);
         // Pays from fewer queries than in the forward (query_is_staged), since the staged pass's reductions also
         // meet in L2: 3,000 even glyphs of 400 / 500 queries, N = 32, 104 / 112 us staged and 118 / 131 not; of 200 / 256,
-        // N = 23, 62 / 64 and 59 / 76; on small tables the copy's latency dominates (10,000 of 200, N = 8: 109 and 91).
-        const int64_t per = bytes / 256 > 256 ? bytes / 256 : 256;
+        // N = 23, 62 / 64 and 59 / 76; on small tables the copy's latency dominates (10,000 of 200, N = 8: 109 and 91), and below
+        // ten glyphs an SM uneven ones lose (300 of 600, N = 32: 20 staged and 14 not).
+        const int64_t least = bytes / (a.L.n_glyphs >= 10 * sm_count() ? 256 : 128), per = least > 256 ? least : 256;
         if (bytes <= STAGED_TABLE_MAX_BYTES && a.Q >= a.L.n_glyphs * per) {
             if (dt == SHM_F32) return launch_bwd_staged<SHM_F32>(a, (uint32_t)bytes, s);
             if (dt == SHM_F16) return launch_bwd_staged<SHM_F16>(a, (uint32_t)bytes, s);
