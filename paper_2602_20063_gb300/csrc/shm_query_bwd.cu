@@ -247,18 +247,6 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
     uint32_t status = 0;
     float loss_acc = 0.0f;
     const float qnan = __int_as_float(0x7fc00000);
-    {
-        const int64_t lo = min(max(__ldg(a.seg), (int64_t)0), a.Q);
-        const int64_t hi = min(max(__ldg(a.seg + G), lo), a.Q);
-        const int64_t stride = (int64_t)gridDim.x * SBB;
-        for (int part = 0; part < 2; ++part) {
-            const int64_t b = part ? hi : 0, e = part ? a.Q : lo;
-            for (int64_t q = b + (int64_t)blockIdx.x * SBB + tid; q < e; q += stride) {
-                status |= SHM_DEV_BOUNDS;
-                if (a.ddirs) { a.ddirs[3 * q] = qnan; a.ddirs[3 * q + 1] = qnan; a.ddirs[3 * q + 2] = qnan; }
-            }
-        }
-    }
     if (tid == 0) {
         stage::init(bar);
         stage::init(bar + 8);
@@ -301,6 +289,19 @@ __global__ void __launch_bounds__(SBB, 2) k_query_bwd_staged(BackwardArgs a, uin
     int buf = 0;
     stage::Part part = stage::next_part(a.seg, G, a.Q, start.g, start, end);
     if (tid == 0 && part.a < part.b) copy(part.g, 0);
+    // queries outside every segment, under the first copy
+    {
+        const int64_t lo = min(max(__ldg(a.seg), (int64_t)0), a.Q);
+        const int64_t hi = min(max(__ldg(a.seg + G), lo), a.Q);
+        const int64_t stride = (int64_t)gridDim.x * SBB;
+        for (int side = 0; side < 2; ++side) {
+            const int64_t b = side ? hi : 0, e = side ? a.Q : lo;
+            for (int64_t q = b + (int64_t)blockIdx.x * SBB + tid; q < e; q += stride) {
+                status |= SHM_DEV_BOUNDS;
+                if (a.ddirs) { a.ddirs[3 * q] = qnan; a.ddirs[3 * q + 1] = qnan; a.ddirs[3 * q + 2] = qnan; }
+            }
+        }
+    }
     while (part.a < part.b) {
         const int g = part.g;
         const int64_t s1 = part.b;

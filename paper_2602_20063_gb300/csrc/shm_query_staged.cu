@@ -46,24 +46,6 @@ __global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArg
     const float qnan = __int_as_float(0x7fc00000);
     uint32_t status = 0;
 
-    // queries outside every segment: NaN and SHM_DEV_BOUNDS, as in the unstaged kernel
-    {
-        const int64_t lo = min(max(__ldg(a.seg), (int64_t)0), a.Q);
-        const int64_t hi = min(max(__ldg(a.seg + G), lo), a.Q);
-        const int64_t stride = (int64_t)gridDim.x * SBLOCK;
-        for (int part = 0; part < 2; ++part) {
-            const int64_t b = part ? hi : 0, e = part ? a.Q : lo;
-            for (int64_t q = b + (int64_t)blockIdx.x * SBLOCK + tid; q < e; q += stride) {
-                status |= SHM_DEV_BOUNDS;
-                if (a.R) a.R[q] = qnan;
-                if (a.grad) { a.grad[3 * q] = qnan; a.grad[3 * q + 1] = qnan; a.grad[3 * q + 2] = qnan; }
-                if (a.normal) { a.normal[3 * q] = qnan; a.normal[3 * q + 1] = qnan; a.normal[3 * q + 2] = qnan; }
-                if (a.chart) { a.chart[2 * q] = qnan; a.chart[2 * q + 1] = qnan; }
-                if (a.fij) { a.fij[3 * q] = -1; a.fij[3 * q + 1] = -1; a.fij[3 * q + 2] = -1; }
-            }
-        }
-    }
-
     if (tid == 0) {
         stage::init(bar);
         stage::init(bar + 8);
@@ -80,6 +62,23 @@ __global__ void __launch_bounds__(SBLOCK, 1024 / SBLOCK) k_query_staged(QueryArg
     int buf = 0;
     stage::Part part = stage::next_part(a.seg, G, a.Q, start.g, start, end);
     if (tid == 0 && part.a < part.b) copy(part.g, 0);
+    // queries outside every segment, under the first copy: NaN and SHM_DEV_BOUNDS, as in the unstaged kernel
+    {
+        const int64_t lo = min(max(__ldg(a.seg), (int64_t)0), a.Q);
+        const int64_t hi = min(max(__ldg(a.seg + G), lo), a.Q);
+        const int64_t stride = (int64_t)gridDim.x * SBLOCK;
+        for (int side = 0; side < 2; ++side) {
+            const int64_t b = side ? hi : 0, e = side ? a.Q : lo;
+            for (int64_t q = b + (int64_t)blockIdx.x * SBLOCK + tid; q < e; q += stride) {
+                status |= SHM_DEV_BOUNDS;
+                if (a.R) a.R[q] = qnan;
+                if (a.grad) { a.grad[3 * q] = qnan; a.grad[3 * q + 1] = qnan; a.grad[3 * q + 2] = qnan; }
+                if (a.normal) { a.normal[3 * q] = qnan; a.normal[3 * q + 1] = qnan; a.normal[3 * q + 2] = qnan; }
+                if (a.chart) { a.chart[2 * q] = qnan; a.chart[2 * q + 1] = qnan; }
+                if (a.fij) { a.fij[3 * q] = -1; a.fij[3 * q + 1] = -1; a.fij[3 * q + 2] = -1; }
+            }
+        }
+    }
     while (part.a < part.b) {
         const int g = part.g;
         const int64_t s1 = part.b;

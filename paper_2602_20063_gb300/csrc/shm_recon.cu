@@ -59,18 +59,6 @@ __global__ void __launch_bounds__(RS_BLOCK, 2) k_recon_staged(QueryArgs a, uint3
         if (a.fij) { a.fij[3 * q] = f; a.fij[3 * q + 1] = i; a.fij[3 * q + 2] = j; }
     };
     const Vec3 nan3{qnan, qnan, qnan};
-    // queries outside every segment
-    {
-        const int64_t lo = stage::seg_at(a.seg, a.Q, 0), hi = max(stage::seg_at(a.seg, a.Q, G), lo);
-        const int64_t stride = (int64_t)gridDim.x * RS_BLOCK;
-        for (int part = 0; part < 2; ++part) {
-            const int64_t b = part ? hi : 0, e = part ? a.Q : lo;
-            for (int64_t q = b + (int64_t)blockIdx.x * RS_BLOCK + tid; q < e; q += stride) {
-                status |= SHM_DEV_BOUNDS;
-                store(q, qnan, nan3, nan3, qnan, qnan, -1, -1, -1);
-            }
-        }
-    }
     if (tid == 0) {
         stage::init(bar);
         stage::init(bar + 8);
@@ -96,6 +84,18 @@ __global__ void __launch_bounds__(RS_BLOCK, 2) k_recon_staged(QueryArgs a, uint3
     int buf = 0;
     stage::Part part = stage::next_part(a.seg, G, a.Q, start.g, start, end);
     if (tid == 0 && part.a < part.b) copy(part.g, 0);
+    // queries outside every segment, under the first copy
+    {
+        const int64_t lo = stage::seg_at(a.seg, a.Q, 0), hi = max(stage::seg_at(a.seg, a.Q, G), lo);
+        const int64_t stride = (int64_t)gridDim.x * RS_BLOCK;
+        for (int side = 0; side < 2; ++side) {
+            const int64_t b = side ? hi : 0, e = side ? a.Q : lo;
+            for (int64_t q = b + (int64_t)blockIdx.x * RS_BLOCK + tid; q < e; q += stride) {
+                status |= SHM_DEV_BOUNDS;
+                store(q, qnan, nan3, nan3, qnan, qnan, -1, -1, -1);
+            }
+        }
+    }
     while (part.a < part.b) {
         const int g = part.g;
         int64_t q = part.a + tid;
