@@ -11,7 +11,7 @@
 //
 // Each CTA takes one unit of equal cost of the path through glyphs and queries (shm_stage.cuh), so long
 // segments are shared and uneven ones balance: 37 glyphs, 2.2 M queries in uneven segments (f16, N = 32)
-// 348 -> 28.7 us, the glyph field (16,384 even segments) 1,229 -> 1,201 us with its bake.
+// 348 -> 28.7 us, the glyph field (16,384 even segments) 1,229 -> 1,195 us with its bake.
 //
 // Results are bit-identical to k_query_fwd (same device functions on the same values).  Directions
 // and outputs are touched once, so they are loaded and stored with the streaming cache hint
